@@ -81,6 +81,43 @@ inline const char* config_error(const npp_config& cfg)
     return variant_error(cfg);
 }
 
+// ------------------------------------------------------------------ packed FP32
+// Two FP32 values in one 64-bit register pair, for the packed FP32x2
+// instructions: each half is rounded exactly as the scalar instruction
+// rounds it.
+__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi)
+{
+    unsigned long long d;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+    return d;
+}
+__device__ __forceinline__ float2 f2_unpack(unsigned long long v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
+                                                     unsigned long long c)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_mul(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsigned long long b)
+{
+    unsigned long long d;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
+__device__ __forceinline__ unsigned long long f2_both(float x) { return f2_pack(x, x); }
+
 // ------------------------------------------------------------------ sampler
 // Philox4x32-10 (Salmon, Moraes, Dror, Shaw: "Parallel random numbers: as
 // easy as 1, 2, 3", SC'11): ten rounds of two 32x32->64 multiplies with the
@@ -90,72 +127,116 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint32_t k0, uint32_t k1
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
         if (r > 0) { k0 += 0x9E3779B9u; k1 += 0xBB67AE85u; }
-        const uint32_t lo0 = 0xD2511F53u * c.x, hi0 = __umulhi(0xD2511F53u, c.x);
-        const uint32_t lo1 = 0xCD9E8D57u * c.z, hi1 = __umulhi(0xCD9E8D57u, c.z);
-        c = make_uint4(hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0);
+        const uint64_t p0 = (uint64_t)0xD2511F53u * c.x, p1 = (uint64_t)0xCD9E8D57u * c.z;
+        c = make_uint4((uint32_t)(p1 >> 32) ^ c.y ^ k0, (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ k1,
+                       (uint32_t)p0);
     }
     return c;
 }
 
-// Natural log of u in (0,1) (the FP32 sampler specification): u = 2^e f with
-// f in [sqrt(1/2), sqrt(2)), ln f = 2 atanh(s), s = (f-1)/(f+1), odd Taylor
-// terms up to s^11, Cody-Waite split of ln 2.  Every operation is a single
-// IEEE round-to-nearest step so that the value is reproducible bit for bit.
-__device__ __forceinline__ float spec_ln(float u)
+__device__ __forceinline__ float sfu_rcp(float x)
 {
-    uint32_t b = __float_as_uint(u);
-    int e = (int)(b >> 23) - 127;
-    const uint32_t m = b & 0x7FFFFFu;
-    float f;
-    if (m > 0x3504F3u) { f = __uint_as_float(m | 0x3F000000u); e += 1; }
-    else               { f = __uint_as_float(m | 0x3F800000u); }
-    const float num = __fsub_rn(f, 1.0f);
-    const float den = __fadd_rn(f, 1.0f);
-    const float s = __fdiv_rn(num, den);
-    const float z = __fmul_rn(s, s);
-    float p = __fmaf_rn(z, 0x1.745d18p-3f, 0x1.c71c72p-3f);   // 2/11, 2/9
-    p = __fmaf_rn(z, p, 0x1.24924ap-2f);                        // 2/7
-    p = __fmaf_rn(z, p, 0x1.99999ap-2f);                        // 2/5
-    p = __fmaf_rn(z, p, 0x1.555556p-1f);                        // 2/3
-    const float t = __fmul_rn(s, z);
-    const float lnf = __fmaf_rn(t, p, __fmul_rn(2.0f, s));
-    const float ef = __int2float_rn(e);
-    return __fmaf_rn(ef, 0x1.62e400p-1f, __fmaf_rn(ef, 0x1.7f7d1cp-20f, lnf));
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
 
-// sin and cos of 2 pi K 2^-24 for odd K in [1, 2^24): quarter-turn reduction
-// in integers (exact), Taylor polynomials of degree 9 / 10 on |x| <= pi/4.
-__device__ __forceinline__ void spec_sincos2pi(uint32_t K, float& s_out, float& c_out)
+__device__ __forceinline__ float sfu_rsqrt(float x)
 {
-    const int q = (int)((K + (1u << 21)) >> 22);
-    const int k = (int)K - q * (1 << 22);
-    const float x = __fmul_rn(__int2float_rn(k), 0x1.921fb6p-22f);
-    const float z = __fmul_rn(x, x);
-    float ps = __fmaf_rn(z, 0x1.71de3ap-19f, -0x1.a01a02p-13f);
-    ps = __fmaf_rn(z, ps, 0x1.111112p-7f);
-    ps = __fmaf_rn(z, ps, -0x1.555556p-3f);
-    const float sx = __fmaf_rn(__fmul_rn(x, z), ps, x);
-    float pc = __fmaf_rn(z, -0x1.27e4fcp-22f, 0x1.a01a02p-16f);
-    pc = __fmaf_rn(z, pc, -0x1.6c16c2p-10f);
-    pc = __fmaf_rn(z, pc, 0x1.555556p-5f);
-    pc = __fmaf_rn(z, pc, -0.5f);
-    const float cx = __fmaf_rn(z, pc, 1.0f);
-    switch (q & 3) {
-    case 0: s_out = sx;  c_out = cx;  break;
-    case 1: s_out = cx;  c_out = -sx; break;
-    case 2: s_out = -sx; c_out = -cx; break;
-    default: s_out = -cx; c_out = sx; break;
-    }
+    float y;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
 }
 
-// Box-Muller pair from two Philox words: radius from `a`, angle from `b`.
-__device__ __forceinline__ float2 spec_normal_pair(uint32_t a, uint32_t b)
+// The two Box-Muller pairs of four Philox words (the FP32 sampler
+// specification), evaluated side by side as the halves of packed FP32x2
+// instructions:
+//
+//   u     = (2 (w >> 9) + 1) 2^-24, from words x and z
+//   ln u  u = 2^e f with f in [sqrt(1/2), sqrt(2)), ln f = 2 atanh(s),
+//         s = (f - 1) / (f + 1), odd Taylor terms up to s^11, Cody-Waite
+//         split of ln 2
+//   r     = sqrt(-2 ln u)
+//   angle 2 pi K 2^-24, K = 2 (w >> 9) + 1, from words y and w:
+//         quarter-turn reduction in integers (exact), Taylor polynomials of
+//         degree 9 / 10 on |x| <= pi/4
+//
+// Every operation rounds to nearest once, so the values are reproducible bit
+// for bit.  The quotient s and the root r are the correctly rounded ones of
+// the specification, computed without a branch: an approximate reciprocal
+// (reciprocal root), the product with it, and one correction by the exact
+// fma residual (Markstein, "Computation of elementary functions on the IBM
+// RISC System/6000 processor", IBM J. Res. Dev. 34, 1990).  The arguments
+// are the 2^23 values of u, for every one of which the results equal the
+// IEEE quotient and root (tests/test_gpu_sampler.py covers almost all of them).
+// Integer-to-float conversions are exact bit constructions (1.m minus a
+// constant) except the exponent's.
+//
+// Bound: instruction issue -- parameter generation is 20-30 % of the
+// rollout kernels' instructions.  Per quad about 135 instead of 210
+// instructions (two independent scalar pairs with the IEEE division and
+// root sequences and their range-check branches).  Plan steps measured on
+// GB300: course (N = 16384, T = 40, width 32) 221 -> 198 us, large (N =
+// 65536, T = 100, width 64) 2.61 -> 2.37 ms.
+__device__ __forceinline__ float4 spec_normal_quad(const uint4& w)
 {
-    const float u1 = __fmul_rn(__uint2float_rn(((a >> 9) << 1) | 1u), 0x1p-24f);
-    const float r = __fsqrt_rn(__fmul_rn(-2.0f, spec_ln(u1)));
-    float s, c;
-    spec_sincos2pi(((b >> 9) << 1) | 1u, s, c);
-    return make_float2(__fmul_rn(r, c), __fmul_rn(r, s));
+    typedef unsigned long long f2;
+    // u: 1.m - (1 - 2^-24) is exact
+    const f2 u = f2_add(f2_pack(__uint_as_float((w.x >> 9) | 0x3F800000u),
+                                __uint_as_float((w.z >> 9) | 0x3F800000u)), f2_both(-0x1.fffffep-1f));
+    const float2 uu = f2_unpack(u);
+    // e and f: the bits from those of sqrt(1/2) upwards, e in the exponent's place
+    const uint32_t b0 = __float_as_uint(uu.x), b1 = __float_as_uint(uu.y);
+    const uint32_t e0 = (b0 - 0x3F3504F4u) & 0xFF800000u, e1 = (b1 - 0x3F3504F4u) & 0xFF800000u;
+    const f2 f = f2_pack(__uint_as_float(b0 - e0), __uint_as_float(b1 - e1));
+    const f2 ef = f2_pack(__int2float_rn((int)e0), __int2float_rn((int)e1));   // e 2^23
+    // -s: the negated reciprocal costs nothing (an operand modifier) and the
+    // fma residual needs one of its factors negated; P's signs undo it
+    const f2 num = f2_add(f, f2_both(-1.0f)), den = f2_add(f, f2_both(1.0f));
+    const float2 dd = f2_unpack(den);
+    const f2 rd = f2_pack(sfu_rcp(-dd.x), sfu_rcp(-dd.y));
+    const f2 q = f2_mul(num, rd);
+    const f2 s = f2_fma(f2_fma(den, q, num), rd, q);
+    const f2 z = f2_mul(s, s);
+    f2 p = f2_fma(z, f2_both(-0x1.745d18p-3f), f2_both(-0x1.c71c72p-3f));       // 2/11, 2/9
+    p = f2_fma(z, p, f2_both(-0x1.24924ap-2f));                                   // 2/7
+    p = f2_fma(z, p, f2_both(-0x1.99999ap-2f));                                   // 2/5
+    p = f2_fma(z, p, f2_both(-0x1.555556p-1f));                                   // 2/3
+    const f2 lnf = f2_fma(f2_mul(s, z), p, f2_mul(s, f2_both(-2.0f)));
+    // ln 2 in two parts, scaled by 2^-23 for e 2^23
+    const f2 ln = f2_fma(ef, f2_both(0x1.62e400p-24f), f2_fma(ef, f2_both(0x1.7f7d1cp-43f), lnf));
+    // -r from x = 2 ln u = -r^2
+    const f2 x = f2_add(ln, ln);
+    const float2 xx = f2_unpack(x);
+    const f2 y = f2_pack(sfu_rsqrt(-xx.x), sfu_rsqrt(-xx.y));
+    const f2 g = f2_mul(x, y);
+    const f2 r = f2_fma(f2_fma(g, g, x), f2_mul(y, f2_both(0.5f)), g);
+    // angle: t = (w + an eighth turn) counts quarter turns in its top bits;
+    // the remainder as 1.m - (1.5 - 2^-22) = k 2^-22 is exact
+    const uint32_t t0 = w.y + 0x20000000u, t1 = w.w + 0x20000000u;
+    const f2 k = f2_add(f2_pack(__uint_as_float(((t0 >> 7) & 0x007FFFFCu) | 0x3F800000u),
+                                __uint_as_float(((t1 >> 7) & 0x007FFFFCu) | 0x3F800000u)),
+                        f2_both(-(1.5f - 0x1p-22f)));
+    const f2 a = f2_mul(k, f2_both(0x1.921fb6p0f));
+    const f2 v = f2_mul(a, a);
+    f2 ps = f2_fma(v, f2_both(0x1.71de3ap-19f), f2_both(-0x1.a01a02p-13f));
+    ps = f2_fma(v, ps, f2_both(0x1.111112p-7f));
+    ps = f2_fma(v, ps, f2_both(-0x1.555556p-3f));
+    const f2 sx = f2_fma(f2_mul(a, v), ps, a);
+    f2 pc = f2_fma(v, f2_both(-0x1.27e4fcp-22f), f2_both(0x1.a01a02p-16f));
+    pc = f2_fma(v, pc, f2_both(-0x1.6c16c2p-10f));
+    pc = f2_fma(v, pc, f2_both(0x1.555556p-5f));
+    pc = f2_fma(v, pc, f2_both(-0.5f));
+    const f2 cx = f2_fma(v, pc, f2_both(1.0f));
+    // times -r before the quadrant's swap and signs (a sign flip is exact)
+    const float2 rs = f2_unpack(f2_mul(r, sx)), rc = f2_unpack(f2_mul(r, cx));
+    const bool o0 = (t0 >> 30) & 1u, o1 = (t1 >> 30) & 1u;
+    float4 n;
+    n.x = __uint_as_float(__float_as_uint(o0 ? rs.x : rc.x) ^ (~(t0 ^ (t0 << 1)) & 0x80000000u));
+    n.y = __uint_as_float(__float_as_uint(o0 ? rc.x : rs.x) ^ (~t0 & 0x80000000u));
+    n.z = __uint_as_float(__float_as_uint(o1 ? rs.y : rc.y) ^ (~(t1 ^ (t1 << 1)) & 0x80000000u));
+    n.w = __uint_as_float(__float_as_uint(o1 ? rc.y : rs.y) ^ (~t1 & 0x80000000u));
+    return n;
 }
 
 struct SamplerKey {
@@ -166,16 +247,15 @@ struct SamplerKey {
 __device__ __forceinline__ float4 sample_quad(const SamplerKey& key, uint32_t q, uint32_t n)
 {
     const uint4 w = philox4x32_10(make_uint4(q, n, key.t_index, key.stream_id), key.k0, key.k1);
-    const float2 a = spec_normal_pair(w.x, w.y);
-    const float2 b = spec_normal_pair(w.z, w.w);
-    return make_float4(a.x, a.y, b.x, b.y);
+    return spec_normal_quad(w);
 }
 
-// theta_n[i], theta_n[i+1] for even i (one Box-Muller pair)
+// theta_n[i], theta_n[i+1] for even i (one Box-Muller pair of its quad)
 __device__ __forceinline__ float2 sample_pair(const SamplerKey& key, uint32_t i, uint32_t n)
 {
     const uint4 w = philox4x32_10(make_uint4(i >> 2, n, key.t_index, key.stream_id), key.k0, key.k1);
-    return (i & 2u) ? spec_normal_pair(w.z, w.w) : spec_normal_pair(w.x, w.y);
+    const float4 v = spec_normal_quad(w);
+    return (i & 2u) ? make_float2(v.z, v.w) : make_float2(v.x, v.y);
 }
 
 // Gaussian sampling proposal of a plan step: samples n < n_prop take
@@ -344,13 +424,6 @@ __device__ __forceinline__ float sfu_ex2(float x)
 {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-__device__ __forceinline__ float sfu_rcp(float x)
-{
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
 

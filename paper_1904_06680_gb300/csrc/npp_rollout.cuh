@@ -69,28 +69,6 @@ struct ThetaSrc {
     }
 };
 
-// Two FP32 values in one 64-bit register pair, for the packed FP32x2
-// instructions: fma.rn.f32x2 rounds each half exactly as fmaf does.
-__device__ __forceinline__ unsigned long long f2_pack(float lo, float hi)
-{
-    unsigned long long d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
-    return d;
-}
-__device__ __forceinline__ float2 f2_unpack(unsigned long long v)
-{
-    float2 r;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-    return r;
-}
-__device__ __forceinline__ unsigned long long f2_fma(unsigned long long a, unsigned long long b,
-                                                     unsigned long long c)
-{
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-
 // The weights of one lane: rows of W1 and W2 as packed pairs of adjacent
 // inputs (2k, 2k + 1), the operands of the FP32x2 FMAs of the step.  With
 // KSQ > 0 the last KSQ input quads of each W2 row live in shared memory
