@@ -478,6 +478,7 @@ struct LoopDev {
     uint32_t t_index;                  // sampling time (Philox counter word)
     int warm_valid;                    // the warm-start buffer holds theta*_{t-1}
     double px, py, pphi, pv;           // simulated vehicle (FP64)
+    double cphi, sphi;                 // cosine and sine of pphi
     int waypoint, n_wp, done, t;
     int status, best_idx, n_infeasible;
     float best_cost;

@@ -75,81 +75,122 @@ struct PlantCfg {
 // space index on, up to the stop, with it and all before it within or on the
 // range field xi in [-back, front], |eta| <= side (EV frame at t).
 
+// The vehicle's pose with its heading's cosine and sine (computed once per
+// sampling time: every setpoint and point is moved into the same frame).
+struct Pose {
+    double px, py, pphi, pv, c, s;
+};
+
 // (xi, eta) of a world point in the vehicle's frame
-__device__ __forceinline__ void ev_of(const LoopDev* d, double px, double py, double& xi, double& eta)
+__device__ __forceinline__ void ev_of(const Pose& v, double px, double py, double& xi, double& eta)
 {
-    const double c = cos(d->pphi), s = sin(d->pphi);
-    const double dx = px - d->px, dy = py - d->py;
-    xi = c * dx + s * dy;
-    eta = -s * dx + c * dy;
+    const double dx = px - v.px, dy = py - v.py;
+    xi = v.c * dx + v.s * dy;
+    eta = -v.s * dx + v.c * dy;
 }
 
-__device__ __forceinline__ bool in_field(const LoopDev* d, double px, double py)
+__device__ __forceinline__ bool in_field(const Pose& v, const float* field, double px, double py)
 {
     double xi, eta;
-    ev_of(d, px, py, xi, eta);
-    return -(double)d->field[1] <= xi && xi <= (double)d->field[0] && fabs(eta) <= (double)d->field[2];
+    ev_of(v, px, py, xi, eta);
+    return -(double)field[1] <= xi && xi <= (double)field[0] && fabs(eta) <= (double)field[2];
 }
 
-__device__ __forceinline__ bool is_stop(const float4* ref, int n, int k) { return k == n - 1 || ref[k].w == 0.0f; }
-
+// the first stop setpoint from k on, searched by the warp 32 at a time
 __device__ __forceinline__ int next_stop(const float4* ref, int n, int k)
 {
-    while (!is_stop(ref, n, k)) ++k;
-    return k;
+    const int lane = threadIdx.x & 31;
+    for (;; k += 32) {
+        const int j = min(k + lane, n - 1);
+        const unsigned stops = __ballot_sync(FULL, j == n - 1 || ref[j].w == 0.0f);
+        if (stops) return min(k + __ffs(stops) - 1, n - 1);
+    }
 }
 
 // the tolerances of Table hyperparameters at the vehicle's pose and speed
-__device__ __forceinline__ bool reached(const LoopDev* d, const float4 g)
+__device__ __forceinline__ bool reached(const Pose& v, const float* eps, const float4 g)
 {
     double dxi, deta;
-    ev_of(d, g.x, g.y, dxi, deta);
-    const double dphi = remainder((double)g.z - d->pphi, 2.0 * M_PI);
-    return fabs(dxi) <= d->eps[0] && fabs(deta) <= d->eps[1] && fabs(dphi) <= d->eps[2] &&
-           fabs((double)g.w - d->pv) <= d->eps[3];
+    ev_of(v, g.x, g.y, dxi, deta);
+    const double dphi = remainder((double)g.z - v.pphi, 2.0 * M_PI);
+    return fabs(dxi) <= eps[0] && fabs(deta) <= eps[1] && fabs(dphi) <= eps[2] &&
+           fabs((double)g.w - v.pv) <= eps[3];
 }
 
-__device__ void select_goal(LoopDev* d, const float4* ref)
+// the last setpoint from idx on, up to stop, that the range field holds
+// with all before it (idx itself when the field does not hold it)
+__device__ __forceinline__ int select_goal(const Pose& v, const float* field, const float4* ref, int idx, int stop)
 {
-    int k = d->idx;
-    if (in_field(d, ref[k].x, ref[k].y))
-        while (k + 1 <= d->stop && in_field(d, ref[k + 1].x, ref[k + 1].y)) ++k;
-    d->goal_k = k;
+    const int lane = threadIdx.x & 31;
+    for (int k = idx;; k += 32) {
+        const int j = k + lane;
+        const unsigned out = __ballot_sync(FULL, j > stop || !in_field(v, field, ref[min(j, stop)].x,
+                                                                       ref[min(j, stop)].y));
+        if (out) return max(k + __ffs(out) - 2, idx);
+    }
 }
 
 // Step 7 (stop setpoints, completion) and Steps 3-4 (space index, goal) at
-// the vehicle's current pose
-__device__ void mission_update(LoopDev* d, const float4* ref)
+// the vehicle's current pose, by one warp: its lanes take the setpoints of
+// the index window, of the way to the next stop and of the range field (one
+// thread taking them in turn, each with its own FP64 sine and cosine, took
+// 67 us of a 200 us sampling time; now 13 us, the FP64 vehicle step itself).
+__device__ __forceinline__ void mission_update(LoopDev* d, const Pose& v, const float4* ref)
 {
     if (d->done) return;
+    const int lane = threadIdx.x & 31;
     const int n = d->n_wp;
-    int best = d->idx;
+    int idx = d->idx, stop = d->stop;
+    int best = 0x7fffffff;
     double bd = INFINITY;
-    const int last = min(d->idx + d->window, d->stop);
-    for (int k = d->idx; k <= last; ++k) {
-        const double dd = hypot((double)ref[k].x - d->px, (double)ref[k].y - d->py);
+    const int last = min(idx + d->window, stop);
+    for (int k = idx + lane; k <= last; k += 32) {
+        const double dd = hypot((double)ref[k].x - v.px, (double)ref[k].y - v.py);
         if (dd < bd) { best = k; bd = dd; }
     }
-    d->idx = best;
-    if (reached(d, ref[d->stop])) {
-        if (d->stop == n - 1) {
-            d->done = 1;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const double od = __shfl_xor_sync(FULL, bd, off);
+        const int ob = __shfl_xor_sync(FULL, best, off);
+        if (od < bd || (od == bd && ob < best)) { best = ob; bd = od; }
+    }
+    if (best != 0x7fffffff) idx = best;
+    int done = 0;
+    if (reached(v, d->eps, ref[stop])) {
+        if (stop == n - 1) {
+            done = 1;
         } else {
-            d->idx = d->stop;
-            d->stop = next_stop(ref, n, d->stop + 1);
+            idx = stop;
+            stop = next_stop(ref, n, stop + 1);
         }
     }
-    select_goal(d, ref);
+    const int k = select_goal(v, d->field, ref, idx, stop);
+    __syncwarp();
+    if (lane == 0) {
+        if (done) d->done = 1;
+        d->idx = idx;
+        d->stop = stop;
+        d->goal_k = k;
+    }
+    __syncwarp();
 }
 
-// mission start: first stop, goal at the initial pose
+// mission start: first stop, goal at the initial pose (one warp)
 __global__ void mission_init_kernel(LoopDev* d, const float4* __restrict__ ref)
 {
-    d->idx = 0;
-    d->stop = next_stop(ref, d->n_wp, 0);
-    select_goal(d, ref);
-    const float4 g = ref[d->goal_k];
-    d->gx = g.x; d->gy = g.y; d->gphi = g.z; d->gv = g.w;
+    const Pose v = { d->px, d->py, d->pphi, d->pv, cos(d->pphi), sin(d->pphi) };
+    const int stop = next_stop(ref, d->n_wp, 0);
+    const int k = select_goal(v, d->field, ref, 0, stop);
+    __syncwarp();
+    if (threadIdx.x == 0) {
+        d->idx = 0;
+        d->stop = stop;
+        d->goal_k = k;
+        d->cphi = v.c;
+        d->sphi = v.s;
+        const float4 g = ref[k];
+        d->gx = g.x; d->gy = g.y; d->gphi = g.z; d->gv = g.w;
+    }
 }
 
 // Obstacle points at the current sampling time t (the state kernel has
@@ -159,10 +200,11 @@ __global__ void advance_obstacles_kernel(const LoopDev* d, const float4* __restr
                                          float4* __restrict__ obs, int M, float Ts)
 {
     const float tau = (float)d->t * Ts;
+    const Pose v = { d->px, d->py, d->pphi, d->pv, d->cphi, d->sphi };
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < M; j += gridDim.x * blockDim.x) {
         const float4 o = obs0[j];
         const float px = fmaf(tau, o.z, o.x), py = fmaf(tau, o.w, o.y);
-        if (d->hide && !in_field(d, px, py)) obs[j] = make_float4(HIDDEN_POINT, HIDDEN_POINT, 0.0f, 0.0f);
+        if (d->hide && !in_field(v, d->field, px, py)) obs[j] = make_float4(HIDDEN_POINT, HIDDEN_POINT, 0.0f, 0.0f);
         else obs[j] = make_float4(px, py, o.z, o.w);
     }
 }
@@ -170,58 +212,54 @@ __global__ void advance_obstacles_kernel(const LoopDev* d, const float4* __restr
 // Steps 6 and 7 of Alg. 1: one sampling time of the simulated vehicle (the
 // kinematic bicycle of Sect. IV, FP64, explicit Euler on the old state) under
 // the winner's first applied control; waypoint switch or mission update;
-// log row (x, y, phi, v, a0, a1, best cost, goal index).  One thread.
+// log row (x, y, phi, v, a0, a1, best cost, goal index).  One warp: every
+// lane computes the same vehicle step, lane 0 writes.
 __global__ void advance_state_kernel(LoopDev* d, const float* __restrict__ controls,
                                      const npp_best* __restrict__ best, const float4* __restrict__ wps,
                                      float* __restrict__ log, int max_log, PlantCfg pc)
 {
+    const int lane = threadIdx.x & 31;
     const double a0 = controls[0], a1 = controls[1];
-    d->status = best->status;
-    d->best_idx = best->best_idx;
-    d->best_cost = best->best_cost;
-    if (best->status == NPP_INFEASIBLE) d->n_infeasible += 1;
-    if (d->t < max_log) {
-        float* row = log + 8 * d->t;
-        row[0] = (float)d->px; row[1] = (float)d->py; row[2] = (float)d->pphi; row[3] = (float)d->pv;
-        row[4] = (float)a0; row[5] = (float)a1; row[6] = best->best_cost;
-        row[7] = (float)(d->mission ? d->goal_k : d->waypoint);
+    const double x = d->px, y = d->py, ph = d->pphi, v = d->pv;
+    if (lane == 0) {
+        d->status = best->status;
+        d->best_idx = best->best_idx;
+        d->best_cost = best->best_cost;
+        if (best->status == NPP_INFEASIBLE) d->n_infeasible += 1;
+        if (d->t < max_log) {
+            float* row = log + 8 * d->t;
+            row[0] = (float)x; row[1] = (float)y; row[2] = (float)ph; row[3] = (float)v;
+            row[4] = (float)a0; row[5] = (float)a1; row[6] = best->best_cost;
+            row[7] = (float)(d->mission ? d->goal_k : d->waypoint);
+        }
     }
+    __syncwarp();
     const double L = pc.lf + pc.lr;
     const double delta = pc.delta_max * a0;
     const double u = pc.u_min + 0.5 * (a1 + 1.0) * (pc.u_max - pc.u_min);
     const double beta = atan(pc.lr * tan(delta) / L);
-    const double x = d->px, y = d->py, ph = d->pphi, v = d->pv;
-    d->px = x + pc.Ts * v * cos(ph + beta) / cos(beta);
-    d->py = y + pc.Ts * v * sin(ph + beta) / cos(beta);
-    d->pphi = ph + pc.Ts * v * tan(delta) / L;
-    d->pv = v + pc.Ts * u;
+    Pose p;
+    p.px = x + pc.Ts * v * cos(ph + beta) / cos(beta);
+    p.py = y + pc.Ts * v * sin(ph + beta) / cos(beta);
+    p.pphi = ph + pc.Ts * v * tan(delta) / L;
+    p.pv = v + pc.Ts * u;
+    p.c = cos(p.pphi);
+    p.s = sin(p.pphi);
+    if (d->mission) {
+        mission_update(d, p, wps);
+    } else if (lane == 0 && !d->done && reached(p, d->eps, wps[d->waypoint])) {
+        // completion check against the current waypoint (Table hyperparameters)
+        if (d->waypoint + 1 < d->n_wp) d->waypoint += 1;
+        else d->done = 1;
+    }
+    if (lane != 0) return;
+    d->px = p.px; d->py = p.py; d->pphi = p.pphi; d->pv = p.pv;
+    d->cphi = p.c; d->sphi = p.s;
     d->t += 1;
     d->t_index += 1;
-    if (d->mission) {
-        mission_update(d, wps);
-        const float4 g = wps[d->goal_k];
-        d->gx = g.x; d->gy = g.y; d->gphi = g.z; d->gv = g.w;
-        d->x0 = (float)d->px; d->y0 = (float)d->py; d->phi0 = (float)d->pphi; d->v0 = (float)d->pv;
-        d->ap0 = (float)a0; d->ap1 = (float)a1;
-        d->warm_valid = 1;
-        return;
-    }
-    // completion check against the current waypoint (Table hyperparameters)
-    if (!d->done) {
-        const float4 g = wps[d->waypoint];
-        const double c = cos(d->pphi), s = sin(d->pphi);
-        const double dx = g.x - d->px, dy = g.y - d->py;
-        const double dxi = c * dx + s * dy, deta = -s * dx + c * dy;
-        const double dphi = remainder((double)g.z - d->pphi, 2.0 * M_PI);
-        if (fabs(dxi) <= d->eps[0] && fabs(deta) <= d->eps[1] && fabs(dphi) <= d->eps[2] &&
-            fabs((double)g.w - d->pv) <= d->eps[3]) {
-            if (d->waypoint + 1 < d->n_wp) d->waypoint += 1;
-            else d->done = 1;
-        }
-    }
-    const float4 g = wps[d->waypoint];
+    const float4 g = wps[d->mission ? d->goal_k : d->waypoint];
     d->gx = g.x; d->gy = g.y; d->gphi = g.z; d->gv = g.w;
-    d->x0 = (float)d->px; d->y0 = (float)d->py; d->phi0 = (float)d->pphi; d->v0 = (float)d->pv;
+    d->x0 = (float)p.px; d->y0 = (float)p.py; d->phi0 = (float)p.pphi; d->v0 = (float)p.pv;
     d->ap0 = (float)a0; d->ap1 = (float)a1;
     d->warm_valid = 1;
 }
@@ -312,7 +350,7 @@ npp_status enqueue_step(npp_loop* L, uint64_t seed)
     PlantCfg pc;
     pc.lf = h->cfg.lf; pc.lr = h->cfg.lr; pc.delta_max = h->cfg.delta_max;
     pc.u_min = h->cfg.u_min; pc.u_max = h->cfg.u_max; pc.Ts = h->cfg.Ts;
-    advance_state_kernel<<<1, 1, 0, s>>>(L->d_dyn, L->d_controls, L->d_best, L->d_wp, L->d_log,
+    advance_state_kernel<<<1, 32, 0, s>>>(L->d_dyn, L->d_controls, L->d_best, L->d_wp, L->d_log,
                                          L->max_log, pc);
     CUDA_TRY(h, cudaGetLastError());
     if (L->M > 0) {
@@ -405,7 +443,7 @@ npp_status loop_create(npp_handle* h, const npp_state* s0, const float* waypoint
     }
     if (e == cudaSuccess && mission) {
         // the first goal and the points seen at t = 0
-        mission_init_kernel<<<1, 1, 0, L->cap>>>(L->d_dyn, L->d_wp);
+        mission_init_kernel<<<1, 32, 0, L->cap>>>(L->d_dyn, L->d_wp);
         e = cudaGetLastError();
         if (e == cudaSuccess && M > 0) {
             advance_obstacles_kernel<<<(M + 255) / 256, 256, 0, L->cap>>>(L->d_dyn, L->d_obs0, L->d_obs, M,
