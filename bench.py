@@ -258,9 +258,16 @@ def workload_setup(name, seed):
     return inputs.scene_course(seed=seed), COURSE_DESC
 
 
+def states_auto(M, N, W):
+    """Whether the library's automatic collision choice is the state-parallel
+    check of a few points (the same rule as its states_auto; else the binned
+    check)."""
+    return M < (128 if W == 64 else 257 if N <= 1024 else 160)
+
+
 def brute_auto(M, N):
-    """The library's automatic brute-force collision variant (the same rule
-    as its brute_auto), to name the kernel that ran."""
+    """The fastest of the fixed brute-force collision variants (0..4) for M
+    points and N samples."""
     if N >= 6144:
         return 2 if M <= 1200 else 4
     if M >= 6000:
@@ -493,10 +500,10 @@ def run_npp(args):
     # the library's own FMA-stream microbenchmark, beside the derived peak
     fma_measured = {"ffma": npp.npp_measure_fma_peak(local, False) / 1e12,
                     "ffma2": npp.npp_measure_fma_peak(local, True) / 1e12, "unit": "T FP32-FMA/s"}
-    # the library's automatic collision choice (binned from 128 points);
+    # the library's automatic collision choice (binned, but for a few points);
     # "fuse" runs the binned check inside the trajectory kernel
     cv = int(options.get("collide_variant", -1))
-    binned = poly or cv == 5 or (cv < 0 and M >= 128)
+    binned = poly or cv == 5 or (cv < 0 and not states_auto(M, N, W))
     fz = int(options.get("fuse", DEFAULT_FUSE))
     fused = binned and not poly and (fz == 1 or (fz < 0 and W == 64))
     # the library's step chunks of the split binned path (option "chunks";
@@ -596,7 +603,8 @@ def run_npp(args):
         tname = "traj_kernel" + shape
         cname = {0: "collide_block_kernel<16,128,1>", 1: "collide_block_kernel<8,64,2>",
                  2: "collide_warp_kernel<8,2>", 3: "collide_slice_kernel<4,2,0,2>",
-                 4: "collide_slice_kernel<2,2,0,4>"}[cv if cv >= 0 else brute_auto(M, N)]
+                 4: "collide_slice_kernel<2,2,0,4>",
+                 -1: "collide_states_kernel<%d>" % (16 if N >= 8192 and M < 64 else 32)}[cv]
         fps_c = res["fma_c"] / (collide_ms / 1e3)
         fps_t = res["fma_t"] / (traj_ms / 1e3)
         roofline = {"bound": "alu", "kernel": cname,
@@ -1078,7 +1086,7 @@ def run_mission(args):
             if t >= args.warmup or k > 0:
                 step_ms.append(tm["total"])
             # trajectories, collision check (+ grid build when binned), epilogue, vehicle, points
-            launches += 6 if M >= 128 else 5
+            launches += 5 if states_auto(M, N, W) else 6
             st = npp.npp_loop_read(L)
             if st["done"]:
                 done_at = st["t"]

@@ -600,6 +600,7 @@ cudaError_t launch_fused_w16(const RolloutArgs& a, cudaStream_t s, int variant);
 cudaError_t launch_fused_w32(const RolloutArgs& a, cudaStream_t s, int variant);
 cudaError_t launch_fused_w64(const RolloutArgs& a, cudaStream_t s, int variant);
 cudaError_t launch_collide_resident(const RolloutArgs& a, cudaStream_t s, int variant);
+cudaError_t launch_collide_states(const RolloutArgs& a, cudaStream_t s);   // one lane per state (few points)
 cudaError_t launch_collide_global(const RolloutArgs& a, cudaStream_t s);
 int collide_global_blocks_per_sm();
 int collide_resident_blocks_per_sm(int M, int variant);

@@ -9,27 +9,21 @@
 #include "../../include/npp.h"
 #include "npp_device.cuh"
 
-// collision-kernel variant number of the spatially binned check, and when
-// the automatic choice takes it: from 128 points, whatever the number of
-// samples (measured on GB300, plan steps at widths 16-64 against the best
-// brute-force variant: 1.0-1.3x faster from 128 to 300 points, 1.3-1.8x
-// beyond; below 128 points within 2-14 % either way; the grid build runs on
-// a side stream while the trajectories are rolled out)
+// collision-kernel variant numbers of the spatially binned check and of the
+// state-parallel one (the automatic choice only), and when the automatic
+// choice takes the latter: below 160 points (128 at width 64, where the
+// binned check runs inside the trajectory kernel), up to 256 for at most 1024
+// samples of the smaller widths.  Measured on GB300 (plan steps at width 16, us, states against
+// binned): N = 20480, T = 60: 122 / 179 at 20 points, 150 / 165 at 128,
+// 162 / 154 at 200; N = 8192, T = 40: 56 / 69 at 64, 63 / 69 at 128, 69 / 65
+// at 200; N = 2048: 43 / 46 at 128, 46 / 46 at 200; N = 256, T = 20: 29 / 33
+// at 64, 31 / 33 at 200, 33 / 33 at 300.  The fixed brute-force variants
+// (0..4) take 43-348 us on these.
 constexpr int COLLIDE_BINNED = 5;
-inline bool binned_auto(int M, int N) { (void)N; return M >= 128; }
-
-// the brute-force variant the automatic choice takes otherwise (measured on
-// GB300 over M = 20..8000 points and N = 1k..30k samples, every variant
-// computing the same flags): with many samples one warp per 8-sample item
-// (2) unless the points are many (4: two point slices per item); with few
-// samples items on four point slices (3), one warp per item for a handful
-// of points, the block-balanced kernel (1) for very many points.  Within 4 %
-// of the fastest variant on every measured case.
-inline int brute_auto(int M, int N)
+constexpr int COLLIDE_STATES = 6;
+inline bool states_auto(int M, int N, int width)
 {
-    if (N >= 6144) return M <= 1200 ? 2 : 4;
-    if (M >= 6000) return 1;
-    return M <= 64 ? 2 : 3;
+    return M < (width == 64 ? 128 : N <= 1024 ? 257 : 160);
 }
 
 // most step chunks of one plan step, and the stage events they need
