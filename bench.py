@@ -948,7 +948,7 @@ def run_proposal(args):
                          "traffic": None, "peak_basis": "measured cuBLAS bf16 burst (MEASURED_PEAKS.json)",
                          "kernel_ms": gemm_ms,
                          "train_step_gemm_tflops": flops / (step_ms * 1e-3) / 1e12},
-            "e2e": None, "gpu_launches": 14 * args.steps, "clocks": ck,
+            "e2e": None, "gpu_launches": 4 * args.steps, "clocks": ck,
             "cpu_baseline": None if args.no_cpu_baseline else proposal_cpu_baseline(),
             "quality": {str(k): v for k, v in quality.items()},
             "training": {"rounds": args.rounds, "seconds": train_s,

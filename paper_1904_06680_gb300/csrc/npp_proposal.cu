@@ -8,10 +8,15 @@
 // (mean, std) only feeds npp_plan_step_proposal, whose proposal samples
 // are mixed with isotropic ones and judged by the exact rollout cost.
 //
-// Layout of the FP32 master parameters (padded for the GEMM tiles):
+// Layout of the FP32 master parameters (padded for the tensor-core tiles):
 //   W1 [256][128] (inputs 72..127 zero), b1 [256], W2 [256][256], b2 [256],
 //   W3 [1024][256] (rows 900..1023 zero), b3 [1024]
-// BF16 copies W1, W2, W2^T, W3, W3^T are refreshed after every update.
+// BF16 copies W1, W2, W3 and W3 in the forward pass's row order (W3f) are
+// refreshed by every update.
+//
+// A training step is four launches: the forward pass with the loss and its
+// gradient, the activations' gradients, the weight gradients (npp_mlp.cu) and
+// the update below.
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -21,17 +26,18 @@
 
 #include "../../include/npp_proposal.h"
 #include "npp_gemm.cuh"
+#include "npp_mlp.cuh"
 #include "npp_internal.h"
 
 using namespace npp;
 
 namespace {
 
-constexpr int NIN_X = NPP_PROP_NIN;        // 72
-constexpr int D0 = 128;                    // padded input width
-constexpr int HID = NPP_PROP_HIDDEN;       // 256
-constexpr int NTH = NPP_PROP_NTHETA;       // 450
-constexpr int D3 = 1024;                   // padded output width (900 used)
+constexpr int NIN_X = MLP_NIN;
+constexpr int D0 = MLP_D0;
+constexpr int HID = MLP_HID;
+constexpr int NTH = MLP_NTH;
+constexpr int D3 = MLP_D3;
 constexpr int NBINS = 64;
 constexpr float R_HIST = 20.0f;
 
@@ -97,195 +103,162 @@ __global__ void __launch_bounds__(256) encode_kernel(const DevCfg c, const npp_s
     }
 }
 
-// x [n][72] FP32 -> X [B][128] BF16 and its transpose XT [128][B] (zero
-// rows beyond n, zero inputs beyond 72).  A block takes PX_TB rows: X is
-// written along the inputs, the tile staged in shared memory and XT written
-// along the batch, so both stores are coalesced.
-constexpr int PX_TB = 32;
-__global__ void __launch_bounds__(256) pack_x_kernel(const float* __restrict__ x, int n, int B,
-                                                     bf16* __restrict__ X, bf16* __restrict__ XT)
-{
-    __shared__ bf16 tile[D0][PX_TB + 2];                  // input x batch row
-    const int b0 = blockIdx.x * PX_TB;
-    for (int e = threadIdx.x; e < PX_TB * D0; e += blockDim.x) {
-        const int k = e % D0, bb = e / D0, b = b0 + bb;
-        const float v = (b < n && k < NIN_X) ? x[(size_t)b * NIN_X + k] : 0.0f;
-        const bf16 q = __float2bfloat16_rn(v);
-        X[(size_t)b * D0 + k] = q;
-        tile[k][bb] = q;
-    }
-    __syncthreads();
-    for (int e = threadIdx.x; e < PX_TB * D0; e += blockDim.x) {
-        const int bb = e % PX_TB, k = e / PX_TB;
-        XT[(size_t)k * B + b0 + bb] = tile[k][bb];
-    }
-}
-
-// Gaussian NLL of theta under (mu, exp(clamp(raw))) and its gradient with
-// respect to the network output, both layouts in BF16; the loss (mean over
-// B x 450) is added to *loss.  A block takes a tile of NLL_TB batch rows x
-// NLL_TI parameters: the row-major gradient is written along the
-// parameters, the tile is staged in shared memory and the transposed
-// gradient written along the batch, so both stores are coalesced.  The
-// padding outputs 900..1023 are never written: their gradient rows stay at
-// the zeros the handle set at creation.
-constexpr int NLL_TB = 64;
-constexpr int NLL_TI = 32;
-__global__ void __launch_bounds__(256) nll_kernel(const float* __restrict__ Y, const float* __restrict__ theta, int B,
-                                                  float ls_min, float ls_max, bf16* __restrict__ dY,
-                                                  bf16* __restrict__ dYT, float* __restrict__ loss)
-{
-    __shared__ float red[8];
-    __shared__ bf16 tile[2][NLL_TI][NLL_TB + 2];          // (mu, log-std) x parameter x batch row
-    const float scale = 1.0f / ((float)B * (float)NTH);
-    const int i0 = blockIdx.x * NLL_TI, b0 = blockIdx.y * NLL_TB;
-    float acc = 0.0f;
-    for (int e = threadIdx.x; e < NLL_TI * NLL_TB; e += blockDim.x) {
-        const int ii = e % NLL_TI, bb = e / NLL_TI;
-        const int i = i0 + ii, b = b0 + bb;
-        if (i < NTH) {
-            const float mu = Y[(size_t)b * D3 + i];
-            const float raw = Y[(size_t)b * D3 + NTH + i];
-            const float ls = fminf(fmaxf(raw, ls_min), ls_max);
-            const float r = theta[(size_t)b * NTH + i] - mu;
-            const float e2 = expf(-2.0f * ls);
-            acc += ls + 0.5f * r * r * e2;
-            const float dmu = -r * e2 * scale;
-            const float dls = (raw > ls_min && raw < ls_max) ? (1.0f - r * r * e2) * scale : 0.0f;
-            const bf16 qm = __float2bfloat16_rn(dmu), ql = __float2bfloat16_rn(dls);
-            dY[(size_t)b * D3 + i] = qm;
-            dY[(size_t)b * D3 + NTH + i] = ql;
-            tile[0][ii][bb] = qm;
-            tile[1][ii][bb] = ql;
-        }
-    }
-    __syncthreads();
-    // transposed rows i and NTH + i, NLL_TB consecutive batch entries each
-    for (int e = threadIdx.x; e < 2 * NLL_TI * NLL_TB; e += blockDim.x) {
-        const int bb = e % NLL_TB, k = e / NLL_TB, half = k / NLL_TI, ii = k % NLL_TI;
-        const int i = i0 + ii;
-        if (i < NTH) dYT[(size_t)(half * NTH + i) * B + b0 + bb] = tile[half][ii][bb];
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, off);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        float s = 0.0f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-        atomicAdd(loss, s * scale);
-    }
-}
-
-// bias gradients: row sums of dY^T (1024 rows), dZ2^T and dZ1^T (256 each);
-// one warp per row, each lane summing 8 consecutive entries per 16-byte
-// load, then the lanes in a fixed tree: a fixed summation order
-__global__ void bias_grad_kernel(const bf16* __restrict__ dYT, const bf16* __restrict__ dZ2T,
-                                 const bf16* __restrict__ dZ1T, int B, float* __restrict__ g)
-{
-    const int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    const int lane = threadIdx.x & 31;
-    if (row >= D3 + 2 * HID) return;
-    const bf16* src;
-    float* dst;
-    if (row < D3) { src = dYT + (size_t)row * B; dst = g + OFF_B3 + row; }
-    else if (row < D3 + HID) { src = dZ2T + (size_t)(row - D3) * B; dst = g + OFF_B2 + (row - D3); }
-    else { src = dZ1T + (size_t)(row - D3 - HID) * B; dst = g + OFF_B1 + (row - D3 - HID); }
-    float s = 0.0f;
-    const uint4* src8 = reinterpret_cast<const uint4*>(src);      // B is a multiple of 128
-    for (int q = lane; q < B / 8; q += 32) {
-        const uint4 u = src8[q];
-        const uint32_t w[4] = { u.x, u.y, u.z, u.w };
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            s += __bfloat162float(__ushort_as_bfloat16((unsigned short)(w[k] & 0xFFFFu)));
-            s += __bfloat162float(__ushort_as_bfloat16((unsigned short)(w[k] >> 16)));
-        }
-    }
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
-    if (lane == 0) *dst = s;
-}
-
-// weight gradients summed over the K slices of the split GEMMs, in slice
-// order (deterministic): segment k has n[k] outputs at dst[k] and n[k] x
-// splits[k] partials at src[k] (slice z at src[k] + z n[k])
-struct SplitSum {
-    const float* src[3];
-    float* dst[3];
-    int n[3];
-    int splits[3];
-};
-__global__ void __launch_bounds__(256) splitk_sum_kernel(const SplitSum a)
-{
-    const int total = a.n[0] + a.n[1] + a.n[2];
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
-        int k = 0, i = t;
-        if (i >= a.n[0]) { i -= a.n[0]; k = 1; if (i >= a.n[1]) { i -= a.n[1]; k = 2; } }
-        const float* p = a.src[k] + i;
-        const size_t st = (size_t)a.n[k];
-        const int S = a.splits[k];
-        float s = 0.0f;
-        int z = 0;
-        // eight loads in flight, added in slice order
-        for (; z + 8 <= S; z += 8) {
-            float v[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) v[u] = p[(size_t)(z + u) * st];
-#pragma unroll
-            for (int u = 0; u < 8; ++u) s += v[u];
-        }
-        for (; z < S; ++z) s += p[(size_t)z * st];
-        a.dst[k][i] = s;
-    }
-}
-
-// Adam with bias correction on the flat FP32 masters
-__global__ void adam_kernel(float* __restrict__ w, float* __restrict__ m, float* __restrict__ v,
-                            const float* __restrict__ g, size_t n, float lr, float b1, float b2, float eps,
-                            float c1, float c2)
-{
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-        const float gi = g[i];
-        const float mi = b1 * m[i] + (1.0f - b1) * gi;
-        const float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-        m[i] = mi;
-        v[i] = vi;
-        const float mhat = mi / c1, vhat = vi / c2;
-        w[i] -= lr * mhat / (sqrtf(vhat) + eps);
-    }
-}
-
-// BF16 copies of the weight matrices (row-major and, for W2, W3, transposed)
+// BF16 copies of the weight matrices
 __global__ void convert_kernel(const float* __restrict__ w, bf16* __restrict__ W1, bf16* __restrict__ W2,
-                               bf16* __restrict__ W2T, bf16* __restrict__ W3, bf16* __restrict__ W3T)
+                               bf16* __restrict__ W3, bf16* __restrict__ W3f)
 {
     const int n1 = HID * D0, n2 = HID * HID, n3 = D3 * HID;
     for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n1 + n2 + n3; t += gridDim.x * blockDim.x) {
-        if (t < n1) {
-            W1[t] = __float2bfloat16_rn(w[OFF_W1 + t]);
-        } else if (t < n1 + n2) {
-            const int u = t - n1, r = u / HID, k = u % HID;
-            const bf16 q = __float2bfloat16_rn(w[OFF_W2 + u]);
-            W2[u] = q;
-            W2T[(size_t)k * HID + r] = q;
-        } else {
-            const int u = t - n1 - n2, r = u / HID, k = u % HID;
+        if (t < n1) W1[t] = __float2bfloat16_rn(w[OFF_W1 + t]);
+        else if (t < n1 + n2) W2[t - n1] = __float2bfloat16_rn(w[OFF_W2 + t - n1]);
+        else {
+            const int u = t - n1 - n2, r = u / HID;
             const bf16 q = __float2bfloat16_rn(w[OFF_W3 + u]);
             W3[u] = q;
-            W3T[(size_t)k * D3 + r] = q;
+            if (r < 2 * NTH) W3f[(size_t)mlp_row(r) * HID + u % HID] = q;
         }
     }
 }
 
-// mean and std of rows 0..n-1 from the network output
-__global__ void mean_std_kernel(const float* __restrict__ Y, int n, float ls_min, float ls_max,
-                                float* __restrict__ mean, float* __restrict__ sd)
+// Adam with bias correction (c1, c2) on one parameter
+struct Adam {
+    float lr, b1, b2, eps, c1, c2;
+};
+__device__ __forceinline__ float adam_step(const Adam& a, float g, float w, float& m, float& v)
 {
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < n * NTH; t += gridDim.x * blockDim.x) {
-        const int b = t / NTH, i = t % NTH;
-        mean[t] = Y[(size_t)b * D3 + i];
-        sd[t] = expf(fminf(fmaxf(Y[(size_t)b * D3 + NTH + i], ls_min), ls_max));
+    // (every rounding written out: the updates are the same bits however the
+    // step is compiled)
+    m = fmaf(1.0f - a.b1, g, __fmul_rn(a.b1, m));
+    v = fmaf(__fmul_rn(1.0f - a.b2, g), g, __fmul_rn(a.b2, v));
+    const float mhat = __fdiv_rn(m, a.c1), vhat = __fdiv_rn(v, a.c2);
+    return __fsub_rn(w, __fdiv_rn(__fmul_rn(a.lr, mhat), __fadd_rn(__fsqrt_rn(vhat), a.eps)));
+}
+
+// The end of a training step: gradients summed in a fixed order (weights
+// over the batch slices; biases over the batch, lane l of 32 taking rows
+// 8 l .. 8 l + 7 of every 256, then the lanes in a pairwise tree), Adam on
+// the FP32 masters, BF16 copies, the loss.
+// Blocks 0 .. UPD_B - 1: UPD_COLS biases each, the longest; then four weights
+// a thread; the last block the loss.
+// Bound: L2 reads of the partials (40 MB at batch 8192) and of the batch's
+// gradients for the bias sums.  One launch instead of four (split sum, bias
+// gradients, Adam, BF16 copies: 36 us of a 187 us step at batch 8192).
+struct UpdateArgs {
+    float *w, *m, *v, *g;
+    bf16 *W[3], *W3f;                        // W1, W2, W3; W3 in the forward order
+    const float* part[3];                    // dW1, dW2, dW3 partials
+    int splits[3];
+    const bf16* dz[3];                       // dZ1, dZ2, dY
+    int batch;
+    const float* loss_part;
+    int n_loss;
+    float* loss;
+    Adam adam;
+};
+constexpr int UPD_THREADS = 256;
+constexpr int UPD_COLS = 32;
+constexpr int UPD_B = (D3 + 2 * HID) / UPD_COLS;
+constexpr int UPD_W = (HID * D0 + HID * HID + D3 * HID) / 4 / UPD_THREADS;
+
+__device__ __forceinline__ float bf_lo(uint32_t w) { return __uint_as_float(w << 16); }
+__device__ __forceinline__ float bf_hi(uint32_t w) { return __uint_as_float(w & 0xFFFF0000u); }
+
+__global__ void __launch_bounds__(UPD_THREADS) update_kernel(const UpdateArgs a)
+{
+    __shared__ float red[32][UPD_COLS + 1];
+    const int tid = threadIdx.x;
+    if (blockIdx.x < UPD_B) {
+        // thread (lane l of the sum, four columns); 32 rows' loads in flight
+        const int c0 = blockIdx.x * UPD_COLS, lc = tid % 8 * 4, l = tid / 8;
+        const int k = c0 < HID ? 0 : c0 < 2 * HID ? 1 : 2;
+        const int col = c0 - k * HID, width = k == 2 ? D3 : HID;
+        const bf16* p = a.dz[k] + (size_t)(8 * l) * width + col + lc;
+        float s[4] = { 0.f, 0.f, 0.f, 0.f };
+        int r = 8 * l;
+        for (; r + 3 * 256 < a.batch; r += 4 * 256, p += (size_t)4 * 256 * width) {
+            uint2 t[32];
+#pragma unroll
+            for (int u = 0; u < 32; ++u)
+                t[u] = __ldg(reinterpret_cast<const uint2*>(p + (size_t)((u >> 3) * 256 + (u & 7)) * width));
+#pragma unroll
+            for (int u = 0; u < 32; ++u) {
+                s[0] += bf_lo(t[u].x); s[1] += bf_hi(t[u].x);
+                s[2] += bf_lo(t[u].y); s[3] += bf_hi(t[u].y);
+            }
+        }
+        for (; r < a.batch; r += 256, p += (size_t)256 * width) {
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const uint2 t = __ldg(reinterpret_cast<const uint2*>(p + (size_t)u * width));
+                s[0] += bf_lo(t.x); s[1] += bf_hi(t.x);
+                s[2] += bf_lo(t.y); s[3] += bf_hi(t.y);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) red[l][lc + j] = s[j];
+        for (int off = 16; off > 0; off >>= 1) {
+            __syncthreads();
+            for (int e = tid; e < off * UPD_COLS; e += UPD_THREADS)
+                red[e / UPD_COLS][e % UPD_COLS] += red[e / UPD_COLS + off][e % UPD_COLS];
+        }
+        __syncthreads();
+        if (tid < UPD_COLS) {
+            const float g = red[0][tid];
+            const size_t i = (k == 0 ? OFF_B1 : k == 1 ? OFF_B2 : OFF_B3) + col + tid;
+            float m = a.m[i], v = a.v[i];
+            a.w[i] = adam_step(a.adam, g, a.w[i], m, v);
+            a.g[i] = g; a.m[i] = m; a.v[i] = v;
+        }
+    } else if (blockIdx.x < UPD_B + UPD_W) {
+        constexpr int n1 = HID * D0 / 4, n2 = HID * HID / 4, n3 = D3 * HID / 4;
+        int i = (blockIdx.x - UPD_B) * UPD_THREADS + tid;
+        const int k = i < n1 ? 0 : i < n1 + n2 ? 1 : 2;
+        i -= k == 0 ? 0 : k == 1 ? n1 : n1 + n2;
+        const size_t size = k == 0 ? n1 : k == 1 ? n2 : n3;
+        const size_t off = k == 0 ? OFF_W1 : k == 1 ? OFF_W2 : OFF_W3;
+        const float4* p = reinterpret_cast<const float4*>(a.part[k]) + i;
+        const int S = a.splits[k];
+        float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
+        int z = 0;
+        for (; z + 8 <= S; z += 8) {             // eight loads in flight, added in slice order
+            float4 t[8];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) t[u] = p[(size_t)(z + u) * size];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) { g.x += t[u].x; g.y += t[u].y; g.z += t[u].z; g.w += t[u].w; }
+        }
+        for (; z < S; ++z) {
+            const float4 t = p[(size_t)z * size];
+            g.x += t.x; g.y += t.y; g.z += t.z; g.w += t.w;
+        }
+        float4* G = reinterpret_cast<float4*>(a.g + off) + i;
+        float4* W = reinterpret_cast<float4*>(a.w + off) + i;
+        float4* M = reinterpret_cast<float4*>(a.m + off) + i;
+        float4* V = reinterpret_cast<float4*>(a.v + off) + i;
+        float4 w = *W, m = *M, v = *V;
+        w.x = adam_step(a.adam, g.x, w.x, m.x, v.x);
+        w.y = adam_step(a.adam, g.y, w.y, m.y, v.y);
+        w.z = adam_step(a.adam, g.z, w.z, m.z, v.z);
+        w.w = adam_step(a.adam, g.w, w.w, m.w, v.w);
+        *G = g; *W = w; *M = m; *V = v;
+        bf16 h[4] = { __float2bfloat16_rn(w.x), __float2bfloat16_rn(w.y), __float2bfloat16_rn(w.z),
+                      __float2bfloat16_rn(w.w) };
+        const uint2 q = *reinterpret_cast<const uint2*>(h);
+        reinterpret_cast<uint2*>(a.W[k])[i] = q;
+        const int r = i / (HID / 4);
+        if (k == 2 && r < 2 * NTH) reinterpret_cast<uint2*>(a.W3f)[mlp_row(r) * (HID / 4) + i % (HID / 4)] = q;
+    } else {
+        float s = 0.0f;
+        for (int i = tid; i < a.n_loss; i += UPD_THREADS) s += a.loss_part[i];
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+        if ((tid & 31) == 0) red[tid >> 5][0] = s;
+        __syncthreads();
+        if (tid == 0) {
+            float t = 0.0f;
+            for (int j = 0; j < UPD_THREADS / 32; ++j) t += red[j][0];
+            *a.loss = t;
+        }
     }
 }
 
@@ -307,92 +280,37 @@ struct npp_proposal {
     int B;
     int t;                                  // Adam steps taken
     float* w; float* m; float* v; float* g; // flat FP32 [N_FLAT]
-    bf16 *W1, *W2, *W2T, *W3, *W3T;
-    bf16 *X, *XT, *H1, *H1T, *H2, *H2T, *dY, *dYT, *dZ2, *dZ2T, *dZ1T;
-    float* Y;
+    bf16 *W1, *W2, *W3, *W3f;               // W3f: W3 in the forward pass's row order
+    bf16 *X, *H1, *H2, *dY, *dZ2, *dZ1;     // activations and their gradients, row-major [batch][..]
     float* loss;                            // scratch loss when the caller passes none
     int* err;
-    // the weight-gradient GEMMs (K = batch) split K into sp[k] slices, each
-    // slice's FP32 partial in ws (dW3, dW2, dW1 at ws_off[k]), summed by
-    // splitk_sum_kernel
-    float* ws;
-    int sp[3];
-    size_t ws_off[3];
-    CUtensorMap tX, tW1, tH1, tW2, tH2, tW3, tdY, tW3T, tdZ2, tW2T, tdYT, tH2T, tdZ2T, tH1T, tdZ1T, tXT;
+    int splits[3];                          // batch slices of the weight gradients
+    float* part[3];                         // their partials: dW3, dW2, dW1
+    float* loss_part;
+    uint4* mask;                            // bits of the positive activations
+    MlpForwardMaps fmaps;
+    MlpBackwardMaps bmaps;
+    MlpGradMaps grads;
 };
 
 namespace {
 
-// K slices of a weight-gradient GEMM with `tiles` output tiles and nk K
-// blocks: doubled while the CTAs stay within about one wave of the 152 SMs
-// and every slice keeps two K blocks or more
-int grad_splits(int tiles, int nk)
+MlpForward forward_args(const npp_proposal* P, const float* x, int n)
 {
-    int sp = 1;
-    while (2 * sp * tiles <= 160 && nk % (2 * sp) == 0 && nk / (2 * sp) >= 2) sp *= 2;
-    return sp;
-}
-
-cudaError_t forward_gemms(npp_proposal* P, cudaStream_t s)
-{
-    const int B = P->B;
-    GemmEpilogue e;
-    memset(&e, 0, sizeof e);
-    e.err = P->err;
-    e.mode = EPI_BIAS_RELU_BF16;
-    e.bias = P->w + OFF_B1; e.out_bf16 = P->H1; e.ldo = HID; e.out_t = P->H1T; e.ldt = B;
-    cudaError_t r = launch_gemm(P->tX, P->tW1, B, HID, D0, 128, e, s);
-    if (r != cudaSuccess) return r;
-    e.bias = P->w + OFF_B2; e.out_bf16 = P->H2; e.out_t = P->H2T;
-    r = launch_gemm(P->tH1, P->tW2, B, HID, HID, 128, e, s);
-    if (r != cudaSuccess) return r;
-    memset(&e, 0, sizeof e);
-    e.err = P->err;
-    e.mode = EPI_BIAS_F32;
-    e.bias = P->w + OFF_B3; e.out_f32 = P->Y; e.ldo = D3;
-    return launch_gemm(P->tH2, P->tW3, B, D3, HID, 256, e, s);
-}
-
-cudaError_t backward_gemms(npp_proposal* P, cudaStream_t s)
-{
-    const int B = P->B;
-    GemmEpilogue e;
-    memset(&e, 0, sizeof e);
-    e.err = P->err;
-    // dZ2 = (dY W3) masked by H2 > 0
-    e.mode = EPI_MASK_BF16;
-    e.mask = P->H2; e.ldm = HID; e.out_bf16 = P->dZ2; e.ldo = HID; e.out_t = P->dZ2T; e.ldt = B;
-    cudaError_t r = launch_gemm(P->tdY, P->tW3T, B, HID, D3, 128, e, s);
-    if (r != cudaSuccess) return r;
-    // dZ1 = (dZ2 W2) masked by H1 > 0 (transposed only)
-    e.mask = P->H1; e.out_bf16 = nullptr; e.out_t = P->dZ1T;
-    r = launch_gemm(P->tdZ2, P->tW2T, B, HID, HID, 128, e, s);
-    if (r != cudaSuccess) return r;
-    // weight gradients (K = B): K split into slices (partials in ws), then
-    // summed in slice order into the flat gradient
-    memset(&e, 0, sizeof e);
-    e.err = P->err;
-    e.mode = EPI_F32;
-    e.out_f32 = P->ws + P->ws_off[0]; e.ldo = HID; e.split_stride = (size_t)D3 * HID;
-    r = launch_gemm(P->tdYT, P->tH2T, D3, HID, B, 256, e, s, P->sp[0]);          // dW3 = dY^T H2
-    if (r != cudaSuccess) return r;
-    e.out_f32 = P->ws + P->ws_off[1]; e.ldo = HID; e.split_stride = (size_t)HID * HID;
-    r = launch_gemm(P->tdZ2T, P->tH1T, HID, HID, B, 256, e, s, P->sp[1]);        // dW2 = dZ2^T H1
-    if (r != cudaSuccess) return r;
-    e.out_f32 = P->ws + P->ws_off[2]; e.ldo = D0; e.split_stride = (size_t)HID * D0;
-    r = launch_gemm(P->tdZ1T, P->tXT, HID, D0, B, 128, e, s, P->sp[2]);          // dW1 = dZ1^T X
-    if (r != cudaSuccess) return r;
-    SplitSum ss;
-    ss.src[0] = P->ws + P->ws_off[0]; ss.dst[0] = P->g + OFF_W3; ss.n[0] = D3 * HID; ss.splits[0] = P->sp[0];
-    ss.src[1] = P->ws + P->ws_off[1]; ss.dst[1] = P->g + OFF_W2; ss.n[1] = HID * HID; ss.splits[1] = P->sp[1];
-    ss.src[2] = P->ws + P->ws_off[2]; ss.dst[2] = P->g + OFF_W1; ss.n[2] = HID * D0; ss.splits[2] = P->sp[2];
-    splitk_sum_kernel<<<(D3 * HID + HID * HID + HID * D0 + 255) / 256, 256, 0, s>>>(ss);
-    return cudaGetLastError();
+    MlpForward f;
+    memset(&f, 0, sizeof f);
+    f.x = x;
+    f.n = n;
+    f.b1 = P->w + OFF_B1; f.b2 = P->w + OFF_B2; f.b3 = P->w + OFF_B3;
+    f.ls_min = P->cfg.ls_min; f.ls_max = P->cfg.ls_max;
+    f.groups = mlp_groups(n, mlp_sm_count());
+    f.err = P->err;
+    return f;
 }
 
 cudaError_t refresh_bf16(npp_proposal* P, cudaStream_t s)
 {
-    convert_kernel<<<512, 256, 0, s>>>(P->w, P->W1, P->W2, P->W2T, P->W3, P->W3T);
+    convert_kernel<<<512, 256, 0, s>>>(P->w, P->W1, P->W2, P->W3, P->W3f);
     return cudaGetLastError();
 }
 
@@ -459,49 +377,46 @@ npp_status npp_proposal_create(const npp_proposal_config* cfg, npp_proposal** ou
     const size_t B = (size_t)cfg->batch;
     auto A = [&](void** p, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(p, bytes); };
     A((void**)&P->w, N_FLAT * 4); A((void**)&P->m, N_FLAT * 4); A((void**)&P->v, N_FLAT * 4); A((void**)&P->g, N_FLAT * 4);
-    A((void**)&P->W1, (size_t)HID * D0 * 2); A((void**)&P->W2, (size_t)HID * HID * 2); A((void**)&P->W2T, (size_t)HID * HID * 2);
-    A((void**)&P->W3, (size_t)D3 * HID * 2); A((void**)&P->W3T, (size_t)D3 * HID * 2);
-    A((void**)&P->X, B * D0 * 2); A((void**)&P->XT, B * D0 * 2);
-    A((void**)&P->H1, B * HID * 2); A((void**)&P->H1T, B * HID * 2);
-    A((void**)&P->H2, B * HID * 2); A((void**)&P->H2T, B * HID * 2);
-    A((void**)&P->dY, B * D3 * 2); A((void**)&P->dYT, B * D3 * 2);
-    A((void**)&P->dZ2, B * HID * 2); A((void**)&P->dZ2T, B * HID * 2); A((void**)&P->dZ1T, B * HID * 2);
-    A((void**)&P->Y, B * D3 * 4);
+    A((void**)&P->W1, (size_t)HID * D0 * 2); A((void**)&P->W2, (size_t)HID * HID * 2);
+    A((void**)&P->W3, (size_t)D3 * HID * 2); A((void**)&P->W3f, (size_t)D3 * HID * 2);
+    A((void**)&P->X, B * D0 * 2);
+    A((void**)&P->H1, B * HID * 2); A((void**)&P->H2, B * HID * 2);
+    A((void**)&P->dY, B * D3 * 2);
+    A((void**)&P->dZ2, B * HID * 2); A((void**)&P->dZ1, B * HID * 2);
     A((void**)&P->loss, sizeof(float));
     A((void**)&P->err, sizeof(int));
-    const int nkb = cfg->batch / 64;
-    P->sp[0] = grad_splits((D3 / 128) * (HID / 256), nkb);
-    P->sp[1] = grad_splits((HID / 128) * (HID / 256), nkb);
-    P->sp[2] = grad_splits((HID / 128) * (D0 / 128), nkb);
-    P->ws_off[0] = 0;
-    P->ws_off[1] = P->ws_off[0] + (size_t)P->sp[0] * D3 * HID;
-    P->ws_off[2] = P->ws_off[1] + (size_t)P->sp[1] * HID * HID;
-    A((void**)&P->ws, (P->ws_off[2] + (size_t)P->sp[2] * HID * D0) * 4);
+    mlp_grad_splits(cfg->batch, P->splits);
+    A((void**)&P->part[0], (size_t)P->splits[0] * D3 * HID * 4);
+    A((void**)&P->part[1], (size_t)P->splits[1] * HID * HID * 4);
+    A((void**)&P->part[2], (size_t)P->splits[2] * HID * D0 * 4);
+    A((void**)&P->loss_part, B / 128 * 32 * 4);
+    A((void**)&P->mask, B * 2 * 2 * sizeof(uint4));
     if (e == cudaSuccess) e = cudaMemset(P->w, 0, N_FLAT * 4);
     if (e == cudaSuccess) e = cudaMemset(P->m, 0, N_FLAT * 4);
     if (e == cudaSuccess) e = cudaMemset(P->v, 0, N_FLAT * 4);
     if (e == cudaSuccess) e = cudaMemset(P->g, 0, N_FLAT * 4);
     if (e == cudaSuccess) e = cudaMemset(P->err, 0, sizeof(int));
-    // the padding outputs' gradient rows stay zero (the loss kernel writes 0..899)
+    // the padding inputs, the padding outputs' gradients and the padding rows
+    // of the forward pass's W3 stay zero (nothing writes them)
+    if (e == cudaSuccess) e = cudaMemset(P->X, 0, B * D0 * 2);
     if (e == cudaSuccess) e = cudaMemset(P->dY, 0, B * D3 * 2);
-    if (e == cudaSuccess) e = cudaMemset(P->dYT, 0, B * D3 * 2);
+    if (e == cudaSuccess) e = cudaMemset(P->W3f, 0, (size_t)D3 * HID * 2);
     if (e != cudaSuccess) {
         npp_proposal_destroy(P);
         return perr(NPP_CUDA_ERROR, std::string("proposal allocation: ") + cudaGetErrorString(e));
     }
     const int b = cfg->batch;
-    // A operands: boxes of 128 rows; B operands: boxes of the tile width
-    // (128 for the N = 256 products over the batch: twice the CTAs of
-    // 256-wide tiles, on 152 SMs)
+    // whole K-major operand blocks; 64 x 64 boxes of the MN-major ones
     struct M { CUtensorMap* map; const void* base; int rows, cols, box; } maps[] = {
-        { &P->tX, P->X, b, D0, 128 },     { &P->tW1, P->W1, HID, D0, 128 },
-        { &P->tH1, P->H1, b, HID, 128 },  { &P->tW2, P->W2, HID, HID, 128 },
-        { &P->tH2, P->H2, b, HID, 128 },  { &P->tW3, P->W3, D3, HID, 256 },
-        { &P->tdY, P->dY, b, D3, 128 },   { &P->tW3T, P->W3T, HID, D3, 128 },
-        { &P->tdZ2, P->dZ2, b, HID, 128 }, { &P->tW2T, P->W2T, HID, HID, 128 },
-        { &P->tdYT, P->dYT, D3, b, 128 }, { &P->tH2T, P->H2T, HID, b, 256 },
-        { &P->tdZ2T, P->dZ2T, HID, b, 128 }, { &P->tH1T, P->H1T, HID, b, 256 },
-        { &P->tdZ1T, P->dZ1T, HID, b, 128 }, { &P->tXT, P->XT, D0, b, 128 },
+        { &P->fmaps.w1, P->W1, HID, D0, 256 }, { &P->fmaps.w2, P->W2, HID, HID, 256 },
+        { &P->fmaps.w3, P->W3f, D3, HID, 256 }, { &P->fmaps.h1, P->H1, b, HID, 128 },
+        { &P->fmaps.h2, P->H2, b, HID, 128 },
+        { &P->bmaps.dy, P->dY, b, D3, 128 }, { &P->bmaps.w3, P->W3, D3, HID, 64 },
+        { &P->bmaps.w2, P->W2, HID, HID, 64 }, { &P->bmaps.dz2, P->dZ2, b, HID, 128 },
+        { &P->bmaps.dz1, P->dZ1, b, HID, 128 },
+        { &P->grads.a[0], P->dY, b, D3, 64 }, { &P->grads.b[0], P->H2, b, HID, 64 },
+        { &P->grads.a[1], P->dZ2, b, HID, 64 }, { &P->grads.b[1], P->H1, b, HID, 64 },
+        { &P->grads.a[2], P->dZ1, b, HID, 64 }, { &P->grads.b[2], P->X, b, D0, 64 },
     };
     for (auto& mp : maps) {
         e = make_tmap_bf16(mp.map, mp.base, mp.rows, mp.cols, mp.box);
@@ -525,8 +440,8 @@ npp_status npp_proposal_destroy(npp_proposal* P)
     if (!P) return NPP_OK;
     cudaSetDevice(P->cfg.device);
     cudaDeviceSynchronize();
-    void* ptrs[] = { P->w, P->m, P->v, P->g, P->W1, P->W2, P->W2T, P->W3, P->W3T, P->X, P->XT, P->H1, P->H1T,
-                     P->H2, P->H2T, P->dY, P->dYT, P->dZ2, P->dZ2T, P->dZ1T, P->Y, P->loss, P->err, P->ws };
+    void* ptrs[] = { P->w, P->m, P->v, P->g, P->W1, P->W2, P->W3, P->W3f, P->X, P->H1, P->H2, P->dY, P->dZ2, P->dZ1,
+                     P->loss, P->err, P->part[0], P->part[1], P->part[2], P->loss_part, P->mask };
     for (void* p : ptrs) if (p) cudaFree(p);
     delete P;
     return NPP_OK;
@@ -587,13 +502,10 @@ npp_status npp_proposal_forward(npp_proposal* P, const float* x_dev, int32_t n, 
     if (n < 1 || n > P->B) return perr(NPP_INVALID_ARG, "npp_proposal_forward: n outside [1, batch]");
     cudaSetDevice(P->cfg.device);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    pack_x_kernel<<<P->B / PX_TB, 256, 0, s>>>(x_dev, n, P->B, P->X, P->XT);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = forward_gemms(P, s);
-    if (e == cudaSuccess) {
-        mean_std_kernel<<<256, 256, 0, s>>>(P->Y, n, P->cfg.ls_min, P->cfg.ls_max, mean_dev, std_dev);
-        e = cudaGetLastError();
-    }
+    MlpForward f = forward_args(P, x_dev, n);
+    f.mean = mean_dev;
+    f.sd = std_dev;
+    const cudaError_t e = launch_mlp_forward(P->fmaps, f, s);
     if (e != cudaSuccess) return perr(NPP_CUDA_ERROR, std::string("proposal forward: ") + cudaGetErrorString(e));
     return NPP_OK;
 }
@@ -606,30 +518,36 @@ npp_status npp_proposal_train_step(npp_proposal* P, const float* x_dev, const fl
     cudaSetDevice(P->cfg.device);
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
     const int B = P->B;
-    pack_x_kernel<<<B / PX_TB, 256, 0, s>>>(x_dev, B, B, P->X, P->XT);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = forward_gemms(P, s);
-    float* lp = loss_dev ? loss_dev : P->loss;
-    if (e == cudaSuccess) e = cudaMemsetAsync(lp, 0, sizeof(float), s);
+    MlpForward f = forward_args(P, x_dev, B);
+    f.theta = theta_dev;
+    f.X = P->X; f.dY = P->dY; f.mask = P->mask;
+    f.loss_part = P->loss_part;
+    cudaError_t e = launch_mlp_forward(P->fmaps, f, s);
     if (e == cudaSuccess) {
-        nll_kernel<<<dim3((NTH + NLL_TI - 1) / NLL_TI, B / NLL_TB), 256, 0, s>>>(P->Y, theta_dev, B, P->cfg.ls_min,
-                                                                        P->cfg.ls_max, P->dY, P->dYT, lp);
-        e = cudaGetLastError();
+        e = launch_mlp_backward(P->bmaps, MlpBackward{ B, P->mask, P->err }, s);
     }
-    if (e == cudaSuccess) e = backward_gemms(P, s);
     if (e == cudaSuccess) {
-        bias_grad_kernel<<<(D3 + 2 * HID) / 8, 256, 0, s>>>(P->dYT, P->dZ2T, P->dZ1T, B, P->g);
-        e = cudaGetLastError();
+        MlpGrads gr = { B, { P->splits[0], P->splits[1], P->splits[2] }, { P->part[0], P->part[1], P->part[2] }, P->err };
+        e = launch_mlp_grads(P->grads, gr, s);
     }
     if (e == cudaSuccess) {
         P->t += 1;
-        const double c1 = 1.0 - std::pow((double)P->cfg.beta1, P->t);
-        const double c2 = 1.0 - std::pow((double)P->cfg.beta2, P->t);
-        adam_kernel<<<512, 256, 0, s>>>(P->w, P->m, P->v, P->g, N_FLAT, lr, P->cfg.beta1, P->cfg.beta2, P->cfg.eps,
-                                        (float)c1, (float)c2);
+        UpdateArgs u;
+        u.w = P->w; u.m = P->m; u.v = P->v; u.g = P->g;
+        u.W[0] = P->W1; u.W[1] = P->W2; u.W[2] = P->W3; u.W3f = P->W3f;
+        u.part[0] = P->part[2]; u.part[1] = P->part[1]; u.part[2] = P->part[0];
+        u.splits[0] = P->splits[2]; u.splits[1] = P->splits[1]; u.splits[2] = P->splits[0];
+        u.dz[0] = P->dZ1; u.dz[1] = P->dZ2; u.dz[2] = P->dY;
+        u.batch = B;
+        u.loss_part = P->loss_part;
+        u.n_loss = B / 128 * 32;
+        u.loss = loss_dev ? loss_dev : P->loss;
+        u.adam = { lr, P->cfg.beta1, P->cfg.beta2, P->cfg.eps,
+                   (float)(1.0 - std::pow((double)P->cfg.beta1, P->t)),
+                   (float)(1.0 - std::pow((double)P->cfg.beta2, P->t)) };
+        update_kernel<<<UPD_B + UPD_W + 1, UPD_THREADS, 0, s>>>(u);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = refresh_bf16(P, s);
     if (e != cudaSuccess) return perr(NPP_CUDA_ERROR, std::string("proposal train step: ") + cudaGetErrorString(e));
     return NPP_OK;
 }
