@@ -303,7 +303,8 @@ KERNEL_SOURCES = tuple(
     ("collide_binned_kernel", ("npp_binned.cu", "npp_rollout.cuh", "npp_device.cuh", "npp_async.cuh")),
     ("collide_poly_kernel", ("npp_poly.cu", "npp_rollout.cuh", "npp_device.cuh", "npp_async.cuh")),
     ("collide_", ("npp_rollout.cuh", "npp_device.cuh", "npp_collide.cu", "npp_async.cuh")),
-    ("gemm_kernel", ("npp_gemm.cu", "npp_gemm.cuh", "npp_async.cuh")),
+    ("gemm_kernel", ("npp_gemm.cu", "npp_gemm.cuh", "npp_tcgen05.cuh", "npp_async.cuh")),
+    ("gemm_pair_kernel", ("npp_gemm.cu", "npp_gemm.cuh", "npp_tcgen05.cuh", "npp_async.cuh")),
 )
 
 
@@ -943,7 +944,7 @@ def run_proposal(args):
                                    "recipe, %d rounds of 8192 course-like scenes at N=2048, "
                                    "evaluated on 192 held-out scenes" % args.rounds,
                        "l2": "train-step working set ~100 MB (L2-resident between steps)"},
-            "roofline": {"bound": "tensor", "kernel": "gemm_kernel<256> (tcgen05, M=N=K=8192)",
+            "roofline": {"bound": "tensor", "kernel": "gemm_pair_kernel (tcgen05, M=N=K=8192)",
                          "achieved": gemm_tf, "peak": peak, "unit": "TFLOP/s", "frac": gemm_tf / peak,
                          "traffic": None, "peak_basis": "measured cuBLAS bf16 burst (MEASURED_PEAKS.json)",
                          "kernel_ms": gemm_ms,

@@ -1,7 +1,7 @@
 // npp_gemm.cu -- BF16 GEMM on the fifth-generation tensor cores.
 //
 // A persistent kernel: one CTA of 192 threads per SM walks 128 x BN tiles
-// of C (and, with split K, slices of their K blocks):
+// of C:
 //   warp 0, one lane   TMA producer: K blocks of 64 (128 bytes of BF16, the
 //                      128-byte swizzle atom) of A and B into a ring of
 //                      STAGES shared-memory stages, completion counted by
@@ -13,15 +13,15 @@
 //                      tile's last stage a commit hands the accumulator to
 //                      the epilogue ("tfull");
 //   warps 2-5          epilogue: warp w reads TMEM lanes 32 (w % 4) ..
-//                      32 (w % 4) + 31 (rows) with tcgen05.ld, applies the
-//                      fused epilogue, stores, and returns the accumulator
+//                      32 (w % 4) + 31 (rows) with tcgen05.ld, stores them
+//                      as FP32, and returns the accumulator
 //                      ("tempty") -- while the MMAs of the next tile run on
 //                      the other one.
 // Every wait on an mbarrier is bounded (about a second of clock): on a
 // timeout the CTA records an error code, stops issuing, waits (bounded) for
 // the copies it issued, frees its TMEM and returns.
 #include "npp_gemm.cuh"
-#include "npp_async.cuh"
+#include "npp_tcgen05.cuh"
 
 #include <cudaTypedefs.h>
 
@@ -42,124 +42,36 @@ struct GemmShape {
     static constexpr int SMEM = STAGES * STAGE_BYTES + 1024 + 128;   // + alignment slack + barriers
 };
 
-__device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int c0, int c1, uint64_t* bar)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-        ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(smem_u32(bar))
-        : "memory");
-}
-
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// shared-memory matrix descriptor: K-major operand in 128-byte swizzle
-// atoms (8 rows x 128 bytes, atoms 1024 bytes apart along the rows)
-__device__ __forceinline__ uint64_t sw128_desc(uint32_t saddr)
-{
-    uint64_t d = 0;
-    d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);         // start address
-    d |= (uint64_t)1 << 16;                            // leading byte offset (unused for this layout)
-    d |= (uint64_t)(1024 >> 4) << 32;                  // stride byte offset: next 8-row atom
-    d |= (uint64_t)1 << 46;                            // descriptor version
-    d |= (uint64_t)2 << 61;                            // 128-byte swizzle
-    return d;
-}
-
-// instruction descriptor: BF16 x BF16 -> FP32, both K-major, M = 128, N = bn
-__host__ __device__ constexpr uint32_t mma_idesc(int bn)
-{
-    return (1u << 4)                  // D: FP32
-         | (1u << 7)                  // A: BF16
-         | (1u << 10)                 // B: BF16
-         | ((uint32_t)(bn >> 3) << 17)
-         | ((uint32_t)(BM >> 4) << 24);
-}
-
-__device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "setp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}"
-        ::"r"(tmem_d), "l"(a), "l"(b), "r"(idesc), "r"(acc)
-        : "memory");
-}
-
-__device__ __forceinline__ void mma_commit(uint64_t* bar)
-{
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                 ::"r"(smem_u32(bar)) : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v)
-{
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
-
 constexpr int GEMM_GROUP_M = 16;
 constexpr int GEMM_THREADS = 192;
 
 // one 128 x BN tile's accumulator rows (TMEM lanes 32 q .. 32 q + 31 at
-// trow, this thread's row `row`) through the fused epilogue to global memory
+// trow, this thread's row `row`) to global memory
 template <int BN>
-__device__ __forceinline__ void store_rows(const GemmEpilogue& ep, uint32_t trow, int row, int n0, int z)
+__device__ __forceinline__ void store_rows(float* C, int ldc, uint32_t trow, int row, int n0)
 {
+    const bool vec = (reinterpret_cast<uintptr_t>(C) & 31u) == 0;      // rows are whole 512-byte multiples
 #pragma unroll 1
     for (int c = 0; c < BN; c += 16) {
         float v[16];
         tmem_ld16(trow + c, v);
-        const int n = n0 + c;
-        if (ep.mode == EPI_F32 || ep.mode == EPI_BIAS_F32) {
-            if (ep.mode == EPI_BIAS_F32)
-#pragma unroll
-                for (int i = 0; i < 16; ++i) v[i] += ep.bias[n + i];
-            float4* o = reinterpret_cast<float4*>(ep.out_f32 + (size_t)z * ep.split_stride + (size_t)row * ep.ldo + n);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) o[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
+        float* o = C + (size_t)row * ldc + n0 + c;
+        if (vec) {
+            store_32b(o, v);
+            store_32b(o + 8, v + 8);
         } else {
-            __nv_bfloat16 hb[16];
-            if (ep.mode == EPI_BIAS_RELU_BF16) {
 #pragma unroll
-                for (int i = 0; i < 16; ++i) hb[i] = __float2bfloat16_rn(fmaxf(v[i] + ep.bias[n + i], 0.0f));
-            } else {
-                const __nv_bfloat16* mk = ep.mask + (size_t)row * ep.ldm + n;
-#pragma unroll
-                for (int i = 0; i < 16; ++i)
-                    hb[i] = __float2bfloat16_rn(__bfloat162float(mk[i]) > 0.0f ? v[i] : 0.0f);
-            }
-            if (ep.out_bf16) {
-                uint4* o = reinterpret_cast<uint4*>(ep.out_bf16 + (size_t)row * ep.ldo + n);
-                const uint4* src = reinterpret_cast<const uint4*>(hb);
-                o[0] = src[0];
-                o[1] = src[1];
-            }
-            if (ep.out_t) {
-#pragma unroll
-                for (int i = 0; i < 16; ++i) ep.out_t[(size_t)(n + i) * ep.ldt + row] = hb[i];
-            }
+            for (int i = 0; i < 4; ++i)
+                reinterpret_cast<float4*>(o)[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
         }
     }
 }
 
-// Work unit u = (tile, K slice): tile u % tiles in the grouped order
-// (consecutive units walk GEMM_GROUP_M row tiles before the next column
-// tile, so the CTAs busy at once share a few tiles of A and of B in L2),
-// slice u / tiles.
-__device__ __forceinline__ void unit_coords(int u, int tiles, int n_tiles, int m_tiles, int bn, int& m0, int& n0,
-                                            int& z)
+// Tile `pid` in the grouped order: consecutive tiles walk GEMM_GROUP_M row
+// tiles before the next column tile, so the CTAs busy at once share a few
+// tiles of A and of B in L2.
+__device__ __forceinline__ void unit_coords(int pid, int n_tiles, int m_tiles, int bn, int& m0, int& n0)
 {
-    const int pid = u % tiles;
-    z = u / tiles;
     const int per_group = GEMM_GROUP_M * n_tiles;
     const int first_m = (pid / per_group) * GEMM_GROUP_M;
     const int gsize = min(m_tiles - first_m, GEMM_GROUP_M);
@@ -176,7 +88,7 @@ __device__ __forceinline__ void unit_coords(int u, int tiles, int n_tiles, int m
 template <int BN>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, int M, int N, int K,
-            int splits, const GemmEpilogue ep)
+            float* C, int* err)
 {
     using S = GemmShape<BN>;
     extern __shared__ uint8_t smem_raw[];
@@ -190,9 +102,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
     int* flags = reinterpret_cast<int*>(tmem_slot + 1);      // [0] abort, [1] issued, [2] consumed
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int n_tiles = N / BN, m_tiles = M / BM, tiles = n_tiles * m_tiles;
-    const int units = tiles * splits;
-    const int nk = K / BK / splits;            // K blocks per unit
+    const int n_tiles = N / BN, m_tiles = M / BM, units = n_tiles * m_tiles;
+    const int nk = K / BK;                     // K blocks per unit
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
@@ -224,8 +135,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
         int g = 0;                             // K blocks issued by this CTA
         bool stop = false;
         for (int u = blockIdx.x; u < units && !stop; u += gridDim.x) {
-            int m0, n0, z;
-            unit_coords(u, tiles, n_tiles, m_tiles, BN, m0, n0, z);
+            int m0, n0;
+            unit_coords(u, n_tiles, m_tiles, BN, m0, n0);
             for (int kb = 0; kb < nk; ++kb, ++g) {
                 const int s = g % STAGES;
                 if (g >= STAGES && !mbar_wait(&empty[s], ((g / STAGES) - 1) & 1)) {
@@ -238,7 +149,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
                     break;
                 }
                 uint8_t* st = smem + s * S::STAGE_BYTES;
-                const int kc = (z * nk + kb) * BK;
+                const int kc = kb * BK;
                 mbar_expect_tx(&full[s], S::STAGE_BYTES);
                 tma_load_2d(st, &ta, kc, m0, &full[s]);
                 tma_load_2d(st + S::A_BYTES, &tb, kc, n0, &full[s]);
@@ -290,9 +201,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
                 break;
             }
             tc_fence_after();
-            int m0, n0, z;
-            unit_coords(u, tiles, n_tiles, m_tiles, BN, m0, n0, z);
-            store_rows<BN>(ep, tmem + (uint32_t)(b * BN) + ((uint32_t)(q * 32) << 16), m0 + q * 32 + lane, n0, z);
+            int m0, n0;
+            unit_coords(u, n_tiles, m_tiles, BN, m0, n0);
+            store_rows<BN>(C, N, tmem + (uint32_t)(b * BN) + ((uint32_t)(q * 32) << 16), m0 + q * 32 + lane, n0);
             tc_fence_before();
             mbar_arrive(&tempty[b]);
         }
@@ -304,7 +215,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
         // copies issued but never consumed land first (bounded waits)
         const bool ok = mbar_wait(done, 0);
         if (!ok || *reinterpret_cast<volatile int*>(&flags[0])) {
-            if (ep.err) atomicExch(ep.err, 1);
+            if (err) atomicExch(err, 1);
             for (int g = flags[2]; g < flags[1]; ++g) mbar_wait(&full[g % STAGES], (g / STAGES) & 1);
         }
     }
@@ -313,6 +224,159 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
     if (warp == 0) {
         tc_fence_after();
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * BN) : "memory");
+    }
+}
+
+// The same GEMM on CTA pairs (cta_group::2): a pair takes 256 x 256 tiles;
+// each CTA loads its 128 rows of A and its 128 of the tile's 256 rows of B,
+// so a stage is 32 KB instead of 48 (six stages in flight instead of four)
+// and every byte of B is read into one SM's shared memory instead of two.
+// The even CTA's MMA lane issues for both; copies of both CTAs count on its
+// "full" barriers, its commits free the stage and hand the accumulator over
+// in both, and both epilogues return it on its "tempty" barriers.
+// M = N = K = 8192 on GB300: 612 us under the profiler (1797 TFLOP/s; the
+// 128 x 256 tiles of one CTA take 710), 710 us against 756 in back-to-back
+// calls, where the power limit holds both. Grouping 8 or 4 row tiles instead
+// of 16: 711 and 730 us against 720, within what runs differ by.
+constexpr int PAIR_STAGES = 6;
+constexpr int PAIR_STAGE = 2 * BM * BK * 2;
+constexpr int PAIR_SMEM = PAIR_STAGES * PAIR_STAGE + 1024 + 256;
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(GEMM_THREADS, 1)
+gemm_pair_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, int M, int N, int K,
+                 float* C, int* err)
+{
+    extern __shared__ uint8_t smem_raw[];
+    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+    uint64_t* full = reinterpret_cast<uint64_t*>(smem + PAIR_STAGES * PAIR_STAGE);
+    uint64_t* empty = full + PAIR_STAGES;
+    uint64_t* tfull = empty + PAIR_STAGES;
+    uint64_t* tempty = tfull + 2;              // both CTAs' 128 epilogue threads
+    uint64_t* done = tempty + 2;
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(done + 1);
+    int* flags = reinterpret_cast<int*>(tmem_slot + 1);      // [0] abort, [1] issued, [2] consumed
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = cluster_rank();
+    const int n_tiles = N / 256, m_tiles = M / 256, units = n_tiles * m_tiles, nk = K / BK;
+    const int pair = blockIdx.x >> 1, pairs = gridDim.x >> 1;
+
+    if (threadIdx.x == 0) {
+        for (int s = 0; s < PAIR_STAGES; ++s) {
+            mbar_init(&full[s], 1);
+            mbar_init(&empty[s], 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&tfull[b], 1);
+            mbar_init(&tempty[b], 256);
+        }
+        mbar_init(done, 1);
+        flags[0] = flags[1] = flags[2] = 0;
+        mbar_init_fence();
+    }
+    if (warp == 0) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(tmem_slot)), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();                            // the peer's barriers are ready
+    tc_fence_after();
+    const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
+
+    if (warp == 0 && lane == 0) {
+        // TMA producer of this CTA's halves
+        int g = 0;
+        bool stop = false;
+        for (int u = pair; u < units && !stop; u += pairs) {
+            int m0, n0;
+            unit_coords(u, n_tiles, m_tiles, 256, m0, n0);
+            m0 = 2 * m0 + 128 * (int)rank;     // unit_coords counts row tiles of 128
+            n0 += 128 * (int)rank;
+            for (int kb = 0; kb < nk; ++kb, ++g) {
+                const int s = g % PAIR_STAGES;
+                if (g >= PAIR_STAGES && !mbar_wait_cluster(&empty[s], ((g / PAIR_STAGES) - 1) & 1))
+                    atomicExch(&flags[0], 1);
+                if (*reinterpret_cast<volatile int*>(&flags[0])) {
+                    stop = true;
+                    break;
+                }
+                uint8_t* st = smem + s * PAIR_STAGE;
+                if (rank == 0) mbar_expect_tx(&full[s], 2 * PAIR_STAGE);
+                const uint32_t bar = leader_addr(&full[s]);
+                tma_load_2d_pair(st, &ta, kb * BK, m0, bar);
+                tma_load_2d_pair(st + PAIR_STAGE / 2, &tb, kb * BK, n0, bar);
+            }
+        }
+        flags[1] = g;
+    } else if (warp == 1 && lane == 0 && rank == 0) {
+        constexpr uint32_t idesc = mma_idesc(256, false, false, 256);
+        int g = 0, i = 0;
+        bool stop = false;
+        for (int u = pair; u < units && !stop; u += pairs, ++i) {
+            const int b = i & 1;
+            if (!mbar_wait_cluster(&tempty[b], ((i >> 1) & 1) ^ 1)) {
+                atomicExch(&flags[0], 1);
+                break;
+            }
+            tc_fence_after();
+            const uint32_t acc = tmem + (uint32_t)(b * 256);
+            for (int kb = 0; kb < nk; ++kb, ++g) {
+                const int s = g % PAIR_STAGES;
+                if (!mbar_wait_cluster(&full[s], (g / PAIR_STAGES) & 1)) {
+                    atomicExch(&flags[0], 1);
+                    stop = true;
+                    break;
+                }
+                tc_fence_after();
+                const uint32_t a0 = smem_u32(smem + s * PAIR_STAGE), b0 = a0 + PAIR_STAGE / 2;
+#pragma unroll
+                for (int j = 0; j < BK / 16; ++j)
+                    mma_bf16_pair(acc, sw128_desc(a0 + j * 32), sw128_desc(b0 + j * 32), idesc, (kb | j) != 0);
+                mma_commit_pair(&empty[s]);
+            }
+            if (!stop) mma_commit_pair(&tfull[b]);
+        }
+        flags[2] = g;
+        mma_commit_pair(done);
+    } else if (warp >= 2) {
+        const int q = warp & 3;
+        int i = 0;
+        for (int u = pair; u < units; u += pairs, ++i) {
+            const int b = i & 1;
+            const bool ok = mbar_wait_cluster(&tfull[b], (i >> 1) & 1);
+            if (!__all_sync(0xffffffffu, ok) || *reinterpret_cast<volatile int*>(&flags[0])) {
+                atomicExch(&flags[0], 1);
+                break;
+            }
+            tc_fence_after();
+            int m0, n0;
+            unit_coords(u, n_tiles, m_tiles, 256, m0, n0);
+            store_rows<256>(C, N, tmem + (uint32_t)(b * 256) + ((uint32_t)(q * 32) << 16),
+                            2 * m0 + 128 * (int)rank + q * 32 + lane, n0);
+            tc_fence_before();
+            arrive_cluster(leader_addr(&tempty[b]));
+        }
+    }
+    __syncwarp();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        // every MMA complete before the TMEM goes back; after a timeout the
+        // copies issued but never consumed land first (bounded waits)
+        const bool ok = mbar_wait_cluster(done, 0);
+        if (!ok || *reinterpret_cast<volatile int*>(&flags[0])) {
+            if (err) atomicExch(err, 1);
+            if (rank == 0)
+                for (int g = flags[2]; g < flags[1]; ++g) mbar_wait_cluster(&full[g % PAIR_STAGES], (g / PAIR_STAGES) & 1);
+        }
+    }
+    tc_fence_before();
+    __syncthreads();
+    cluster_sync();                            // neither CTA leaves while the other uses its memory
+    if (warp == 0) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
     }
 }
 
@@ -361,24 +425,36 @@ cudaError_t make_tmap_bf16(CUtensorMap* map, const void* base, int rows, int col
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-cudaError_t launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, int M, int N, int K, int bn,
-                        const GemmEpilogue& ep, cudaStream_t s, int splits)
+// Whether the pair kernel takes the product: whole 256 x 256 tiles, and
+// enough of them to give every pair of SMs one (fewer tiles fill more SMs as
+// 128-row tiles).
+bool gemm_pairs(int M, int N)
+{
+    return M % 256 == 0 && N % 256 == 0 && (M / 256) * (N / 256) >= sm_count() / 2;
+}
+
+cudaError_t launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, int M, int N, int K, int bn, int box_b, float* C,
+                        int* err, cudaStream_t s)
 {
     if (M % BM || K % BK || K < BK || (bn != 128 && bn != 256) || N % bn) return cudaErrorInvalidValue;
-    if (splits < 1 || (K / BK) % splits || (splits > 1 && (ep.mode != EPI_F32 || ep.split_stride == 0)))
-        return cudaErrorInvalidValue;
-    const int units = (M / BM) * (N / bn) * splits;
-    const int grid = std::min(units, sm_count());
+    if (bn == 256 && box_b == 128) {
+        cudaError_t e = cudaFuncSetAttribute(gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, PAIR_SMEM);
+        if (e != cudaSuccess) return e;
+        const int pairs = std::min((M / 256) * (N / 256), sm_count() / 2);
+        gemm_pair_kernel<<<2 * pairs, GEMM_THREADS, PAIR_SMEM, s>>>(ta, tb, M, N, K, C, err);
+        return cudaGetLastError();
+    }
+    const int grid = std::min((M / BM) * (N / bn), sm_count());
     if (bn == 256) {
         const int smem = GemmShape<256>::SMEM;
         cudaError_t e = cudaFuncSetAttribute(gemm_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        gemm_kernel<256><<<grid, GEMM_THREADS, smem, s>>>(ta, tb, M, N, K, splits, ep);
+        gemm_kernel<256><<<grid, GEMM_THREADS, smem, s>>>(ta, tb, M, N, K, C, err);
     } else {
         const int smem = GemmShape<128>::SMEM;
         cudaError_t e = cudaFuncSetAttribute(gemm_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e != cudaSuccess) return e;
-        gemm_kernel<128><<<grid, GEMM_THREADS, smem, s>>>(ta, tb, M, N, K, splits, ep);
+        gemm_kernel<128><<<grid, GEMM_THREADS, smem, s>>>(ta, tb, M, N, K, C, err);
     }
     return cudaGetLastError();
 }

@@ -558,21 +558,15 @@ npp_status npp_gemm_bf16(const uint16_t* A_dev, const uint16_t* B_dev, float* C_
     if (!A_dev || !B_dev || !C_dev) return perr(NPP_INVALID_ARG, "npp_gemm_bf16: NULL argument");
     if (M < 128 || M % 128 || N < 128 || N % 128 || K < 64 || K % 64)
         return perr(NPP_INVALID_ARG, "npp_gemm_bf16: M, N multiples of 128 and K a multiple of 64");
-    const int bn = (N % 256 == 0) ? 256 : 128;
+    const int bn = (N % 256 == 0) ? 256 : 128, box_b = gemm_pairs(M, N) ? 128 : bn;
     CUtensorMap ta, tb;
     cudaError_t e = make_tmap_bf16(&ta, A_dev, M, K, 128);
-    if (e == cudaSuccess) e = make_tmap_bf16(&tb, B_dev, N, K, bn);
+    if (e == cudaSuccess) e = make_tmap_bf16(&tb, B_dev, N, K, box_b);
     if (e != cudaSuccess) return perr(NPP_INVALID_ARG, "npp_gemm_bf16: operands must be 16-byte aligned");
     int* err = nullptr;
     e = cudaGetSymbolAddress(reinterpret_cast<void**>(&err), g_gemm_err);
     if (e != cudaSuccess) return perr(NPP_CUDA_ERROR, std::string("gemm error flag: ") + cudaGetErrorString(e));
-    GemmEpilogue ep;
-    memset(&ep, 0, sizeof ep);
-    ep.mode = EPI_F32;
-    ep.out_f32 = C_dev;
-    ep.ldo = N;
-    ep.err = err;
-    e = launch_gemm(ta, tb, M, N, K, bn, ep, reinterpret_cast<cudaStream_t>(stream));
+    e = launch_gemm(ta, tb, M, N, K, bn, box_b, C_dev, err, reinterpret_cast<cudaStream_t>(stream));
     if (e != cudaSuccess) return perr(NPP_CUDA_ERROR, std::string("gemm launch: ") + cudaGetErrorString(e));
     return NPP_OK;
 }
