@@ -59,31 +59,60 @@ using bf16 = __nv_bfloat16;
 // the EV-aligned frame at t (fixed-point sums, so the result does not
 // depend on the order of the atomic adds), squashed h / (1 + h), then the
 // rollout's 8 network inputs at h = 0.
-__global__ void __launch_bounds__(256) encode_kernel(const DevCfg c, const npp_scene* __restrict__ scenes,
-                                                     const float4* __restrict__ obs, float* __restrict__ x)
+// A weight is a multiple of 2^-32; its upper and lower 16 bits are summed
+// apart (32-bit shared atomics, which the hardware does in place; 64-bit ones
+// loop), without overflow up to 65535 points; beyond, the upper sums carry
+// into a third word.
+// Bound: latency (reads, atan2, atomics); ENC_AHEAD points a thread in flight.
+// Encoding and forward pass of 300 scenes on GB300: 33 -> 28.5 us (256
+// threads, one point at a time and 64-bit atomics before).
+constexpr int ENC_THREADS = 512;
+constexpr int ENC_AHEAD = 4;
+__global__ void __launch_bounds__(ENC_THREADS) encode_kernel(const DevCfg c, const npp_scene* __restrict__ scenes,
+                                                             const float4* __restrict__ obs, float* __restrict__ x)
 {
-    __shared__ unsigned long long hist[NBINS];
-    const npp_scene sc = scenes[blockIdx.x];
-    for (int k = threadIdx.x; k < NBINS; k += blockDim.x) hist[k] = 0ull;
+    __shared__ unsigned lo[NBINS], hi[NBINS], over[NBINS];
+    const npp_scene& sc = scenes[blockIdx.x];
+    for (int k = threadIdx.x; k < NBINS; k += ENC_THREADS) lo[k] = hi[k] = over[k] = 0u;
     __syncthreads();
     float s0, c0;
     sincosf(sc.state.phi, &s0, &c0);
     const float4* p = obs + sc.obs_offset;
-    for (int j = threadIdx.x; j < sc.M; j += blockDim.x) {
-        float px, py, vx, vy;
-        ev_point(p[j], sc.state.x, sc.state.y, s0, c0, px, py, vx, vy);
-        const float d = sqrtf(fmaf(px, px, py * py));
-        const float w = 1.0f - d / R_HIST;
-        if (w > 0.0f) {
-            const float u = (atan2f(py, px) + 3.14159265358979323846f) * (NBINS / 6.28318530717958647692f);
-            const int k = min(max((int)floorf(u), 0), NBINS - 1);
-            atomicAdd(&hist[k], (unsigned long long)__float2ull_rn(w * 4294967296.0f));
+    const int M = sc.M;
+    const bool large = M > 65535;
+    for (int j0 = threadIdx.x; j0 < M; j0 += ENC_AHEAD * ENC_THREADS) {
+        float4 o[ENC_AHEAD];
+#pragma unroll
+        for (int u = 0; u < ENC_AHEAD; ++u) {
+            const int j = j0 + u * ENC_THREADS;
+            o[u] = p[j < M ? j : j0];
+        }
+#pragma unroll
+        for (int u = 0; u < ENC_AHEAD; ++u) {
+            float px, py, vx, vy;
+            ev_point(o[u], sc.state.x, sc.state.y, s0, c0, px, py, vx, vy);
+            const float d = sqrtf(fmaf(px, px, py * py));
+            const float w = 1.0f - d / R_HIST;
+            if (j0 + u * ENC_THREADS < M && w > 0.0f) {
+                const float t = (atan2f(py, px) + 3.14159265358979323846f) * (NBINS / 6.28318530717958647692f);
+                const int k = min(max((int)floorf(t), 0), NBINS - 1);
+                const unsigned long long v = __float2ull_rn(w * 4294967296.0f);
+                const unsigned l = (unsigned)(v & 0xFFFFu), h = (unsigned)(v >> 16);
+                const unsigned was_l = atomicAdd(&lo[k], l);
+                const unsigned was_h = atomicAdd(&hi[k], h);
+                if (large) {
+                    // carries of the two sums (2^32 of lo is 2^16 of hi)
+                    if (was_l + l < was_l && atomicAdd(&hi[k], 65536u) > 0xFFFEFFFFu) atomicAdd(&over[k], 1u);
+                    if (was_h + h < was_h) atomicAdd(&over[k], 1u);
+                }
+            }
         }
     }
     __syncthreads();
     float* xr = x + (size_t)blockIdx.x * NIN_X;
-    for (int k = threadIdx.x; k < NBINS; k += blockDim.x) {
-        const float h = (float)((double)hist[k] * (1.0 / 4294967296.0));
+    for (int k = threadIdx.x; k < NBINS; k += ENC_THREADS) {
+        const unsigned long long sum = ((unsigned long long)over[k] << 48) + ((unsigned long long)hi[k] << 16) + lo[k];
+        const float h = (float)((double)sum * (1.0 / 4294967296.0));
         xr[k] = h / (1.0f + h);
     }
     if (threadIdx.x == 0) {
@@ -488,7 +517,7 @@ npp_status npp_proposal_encode(const npp_handle* h, const npp_scene* scenes_dev,
     if (!obs_dev || (reinterpret_cast<uintptr_t>(obs_dev) & 15u))
         return perr(NPP_INVALID_ARG, "npp_proposal_encode: obstacle array must be non-NULL and 16-byte aligned");
     cudaSetDevice(h->device);
-    encode_kernel<<<S, 256, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
+    encode_kernel<<<S, ENC_THREADS, 0, reinterpret_cast<cudaStream_t>(stream)>>>(
         h->dc, scenes_dev, reinterpret_cast<const float4*>(obs_dev), x_dev);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return perr(NPP_CUDA_ERROR, std::string("encode launch: ") + cudaGetErrorString(e));
