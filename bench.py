@@ -295,14 +295,14 @@ def algorithmic_work(first_hit, T, M, W):
 
 
 # source files whose code each profiled kernel is built from
-_ROLLOUT = ("npp_rollout.cuh", "npp_device.cuh", "npp_async.cuh")
+_ROLLOUT = ("npp_rollout.cuh", "npp_device.cuh", "npp_async.cuh", "npp_tmem.cuh")
 KERNEL_SOURCES = tuple(
     (kind + "<%d" % w, _ROLLOUT + ("npp_rollout_w%d.cu" % w,))      # each width's own translation unit
-    for kind in ("traj_kernel", "fused_kernel") for w in (16, 32, 64)) + (
-    ("bin_build_kernel", ("npp_binned.cu", "npp_rollout.cuh", "npp_device.cuh", "npp_async.cuh")),
-    ("collide_binned_kernel", ("npp_binned.cu", "npp_rollout.cuh", "npp_device.cuh", "npp_async.cuh")),
-    ("collide_poly_kernel", ("npp_poly.cu", "npp_rollout.cuh", "npp_device.cuh", "npp_async.cuh")),
-    ("collide_", ("npp_rollout.cuh", "npp_device.cuh", "npp_collide.cu", "npp_async.cuh")),
+    for kind in ("traj_kernel", "fused_kernel", "traj_tmem_kernel", "fused_tmem_kernel") for w in (16, 32, 64)) + (
+    ("bin_build_kernel", _ROLLOUT + ("npp_binned.cu",)),
+    ("collide_binned_kernel", _ROLLOUT + ("npp_binned.cu",)),
+    ("collide_poly_kernel", _ROLLOUT + ("npp_poly.cu",)),
+    ("collide_", _ROLLOUT + ("npp_collide.cu",)),
     ("gemm_kernel", ("npp_gemm.cu", "npp_gemm.cuh", "npp_tcgen05.cuh", "npp_async.cuh")),
     ("gemm_pair_kernel", ("npp_gemm.cu", "npp_gemm.cuh", "npp_tcgen05.cuh", "npp_async.cuh")),
 )
@@ -514,15 +514,19 @@ def run_npp(args):
         nch = min(int(options.get("chunks", 0)) or (2 if W == 64 else 1), T)
     # per sampling time: plan step kernels, epilogue, vehicle and obstacle advance
     launches_per_step = (2 if fused else 1 + 2 * nch if binned and not poly else 3 if poly else 2) + 3
-    # default launch shapes; the last template argument is the variant flag
+    # default launch shapes; the fifth template argument is the variant flag
     # (off: no speed limits, features in the EV frame at t)
     var = int(bool(p.get("v_limits", 0) or p.get("feature_frame", 0)))
-    shape = {16: "<16,8,4,4,%d,0>" if var else "<16,8,8,3,%d,0>", 32: "<32,16,4,4,%d,0>",
-             64: "<64,32,1,16,%d,8>"}[W] % var
+    sms = torch.cuda.get_device_properties(local).multi_processor_count
+    wide = N >= 16384 if W == 64 else -(-N // {16: 16, 32: 8}[W]) > sms * 7 // 8
+    shape = "_tmem_kernel" + ({16: "<16,4,4,4,%d,4,0>", 32: "<32,8,4,4,%d,8,0>", 64: "<64,16,4,3,%d,8,8>"} if wide else
+                              {16: "<16,8,4,6,%d,4,0>", 32: "<32,16,4,5,%d,8,0>", 64: "<64,32,4,4,%d,16,0>"})[W] % var
     if fused:
         # [0] grid build, [1] the trajectory kernel with the windowed check
-        fshape = {16: "<16,8,4,4,%d,0,16,4>", 32: "<32,16,4,5,%d,5,8,4>", 64: "<64,32,1,16,%d,12,8,4>"}[W] % var
-        fname = "fused_kernel" + fshape
+        full = N >= 16 * sms
+        fshape = {16: "_kernel<16,8,4,4,%d,0,16,4>", 32: "_kernel<32,16,4,5,%d,5,8,4>",
+                  64: "_tmem_kernel<64,32,20,1,%d,12,4,8,4>" if full else "_tmem_kernel<64,32,4,4,%d,16,0,8,4>"}[W] % var
+        fname = "fused" + fshape
         fps = res["fma_t"] / (collide_ms / 1e3)
         rolled = res["rolled"] if res["rolled"] > 0 else float(N) * T * K
         fma_rolled = rolled * (W * W + 10 * W)
@@ -566,7 +570,7 @@ def run_npp(args):
         # the binned (or polygon) check does only the candidate work of the
         # cells a state overlaps, which has no fixed algorithmic count; the
         # MLP rollout is the work every plan step must do
-        tname = "traj_kernel" + shape
+        tname = "traj" + shape
         cname = "bin_build_kernel + " + ("collide_poly_kernel" if poly else "collide_binned_kernel")
         fps_t = res["fma_t"] / (traj_ms / 1e3)
         coll = {"ms_per_step": collide_ms / K}
@@ -601,7 +605,7 @@ def run_npp(args):
                     "other": {cname: coll},
                     "dominant": tname if traj_ms >= collide_ms else cname}
     else:
-        tname = "traj_kernel" + shape
+        tname = "traj" + shape
         cname = {0: "collide_block_kernel<16,128,1>", 1: "collide_block_kernel<8,64,2>",
                  2: "collide_warp_kernel<8,2>", 3: "collide_slice_kernel<4,2,0,2>",
                  4: "collide_slice_kernel<2,2,0,4>",

@@ -499,12 +499,10 @@ npp_status npp_plan_step_noalloc(const npp_config* cfg, const npp_state* state,
  * launch.  0 (default): automatic (2 at width 64, else 1), 1: one launch
  * each; at most T chunks.
  * "traj_variant" 0..4: launch shape of the trajectory kernel -- 0 (default)
- * 2 hidden units per lane in blocks sized for occupancy, 1 four hidden units
- * per lane, 2 eight-warp blocks, 3 another block size, 4 at width 64 every
- * weight in registers (12 warps per SM; the width-64 default keeps half of
- * each lane's layer-2 weights in shared memory so that 16 fit), at width 32
- * 5 of each lane's 8 layer-2 input quads in shared memory (20 warps per
- * SM), at width 16 the default shape.
+ * by the number of samples, 1 four hidden units per lane (with the windowed
+ * check at width 64: every SM's warps in one block), 2 two hidden units per
+ * lane (small blocks), both with layer-2 weights in tensor memory; 3 and 4
+ * every weight in registers (at width 64 a part in shared memory).
  * Returns NPP_INVALID_ARG for an unknown name or value. */
 npp_status npp_set_option(npp_handle* h, const char* name, int32_t value);
 

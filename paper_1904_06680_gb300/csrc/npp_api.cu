@@ -267,6 +267,7 @@ npp_status run_rollout(npp_handle* h, RolloutArgs& a, cudaStream_t s, bool no_re
     a.coefA = nullptr;
     a.coefB = nullptr;
     a.work = h->d_work;
+    a.sm_count = h->sm_count;
     if (h->timing) h->last_chunks = 1;
     if (h->fp_faces > 0) {
         // general footprint: grids sized by its radius (side stream, as

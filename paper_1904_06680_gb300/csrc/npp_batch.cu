@@ -384,8 +384,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) batch_traj_kernel(const BatchAr
                           (size_t)(tid / 32) * (32 / G) * BATCH_CW;
             unsigned steps = 0, ntest = 0, nstate = 0;
             const bool valid = n < s.N;
-            const FusedOut o = traj_sample_windowed<W, G, STAGE_TH, VAR, KSQ, BATCH_CW, 4>(
-                b.c, job, n, valid, gl, hx_all + bi * W, wnd, steps, ntest, nstate);
+            LaneNet<W, G, KSQ> net;
+            load_net<STAGE_TH>(net, job, n, valid, gl);
+            const FusedOut o = traj_sample_windowed<VAR, BATCH_CW, 4>(
+                b.c, job, net, n, valid, gl, hx_all + bi * W, wnd, steps, ntest, nstate);
             if (valid && gl == 0) {
                 unsigned long long key;
                 if (o.first_hit < 0)
@@ -397,7 +399,9 @@ __global__ void __launch_bounds__(NW * 32, MINB) batch_traj_kernel(const BatchAr
                 if (key < *reinterpret_cast<volatile unsigned long long*>(b.keys + si)) atomicMin(b.keys + si, key);
             }
         } else {
-            traj_sample<W, G, STAGE_TH, VAR, KSQ>(b.c, job, n, n < s.N, gl, hx_all + bi * W);
+            LaneNet<W, G, KSQ> net;
+            load_net<STAGE_TH>(net, job, n, n < s.N, gl);
+            traj_sample<VAR>(b.c, job, net, n, n < s.N, gl, hx_all + bi * W);
         }
     }
 }
@@ -621,7 +625,9 @@ __device__ void batch_reroll(const BatchArgs& b, const SceneDev& s, int idx, flo
     job.coef_base = 0;
     job.jfree = nullptr;
     job.vfirst = nullptr;
-    traj_sample<W, G, 0, VAR>(b.c, job, idx, true, lane % G, hrows + (lane / G) * W);
+    LaneNet<W, G> net;
+    load_net(net, job, idx, true, lane % G);
+    traj_sample<VAR>(b.c, job, net, idx, true, lane % G, hrows + (lane / G) * W);
 }
 
 __global__ void batch_epilogue_kernel(const BatchArgs b)

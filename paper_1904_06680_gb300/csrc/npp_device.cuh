@@ -275,18 +275,27 @@ __device__ __forceinline__ bool proposal_sample(const Proposal& p, uint32_t n)
     return p.mu != nullptr && (long long)n < (long long)p.n_prop;
 }
 
+// four values from index i on (a multiple of 4) of an array that may start at
+// any 4-byte boundary (vec: it starts at a 16-byte one)
+__device__ __forceinline__ float4 load_quad(const float* p, int i, bool vec)
+{
+    if (vec) return *reinterpret_cast<const float4*>(p + i);
+    return make_float4(p[i], p[i + 1], p[i + 2], p[i + 3]);
+}
+
 // theta_n[4q .. 4q+3] of a plan step with proposal p (all four indices
-// below n_theta)
+// below n_theta).  mu and sigma are read before the sampler's arithmetic,
+// which hides the reads (a rolled loop of quads has nothing else to).
 __device__ __forceinline__ float4 sample_quad_mixed(const SamplerKey& key, const Proposal& p, uint32_t q,
                                                     uint32_t n)
 {
     if (!proposal_sample(p, n)) return sample_quad(key, q, n);
     SamplerKey k1 = key;
     k1.stream_id = p.stream;
+    const bool vec = ((reinterpret_cast<uintptr_t>(p.mu) | reinterpret_cast<uintptr_t>(p.sigma)) & 15u) == 0;
+    const float4 s = load_quad(p.sigma, 4 * (int)q, vec), m = load_quad(p.mu, 4 * (int)q, vec);
     const float4 e = sample_quad(k1, q, n);
-    const int i = 4 * (int)q;
-    return make_float4(fmaf(p.sigma[i], e.x, p.mu[i]), fmaf(p.sigma[i + 1], e.y, p.mu[i + 1]),
-                       fmaf(p.sigma[i + 2], e.z, p.mu[i + 2]), fmaf(p.sigma[i + 3], e.w, p.mu[i + 3]));
+    return make_float4(fmaf(s.x, e.x, m.x), fmaf(s.y, e.y, m.y), fmaf(s.z, e.z, m.z), fmaf(s.w, e.w, m.w));
 }
 
 // theta_n[i], theta_n[i+1] for even i
@@ -296,8 +305,9 @@ __device__ __forceinline__ float2 sample_pair_mixed(const SamplerKey& key, const
     if (!proposal_sample(p, n)) return sample_pair(key, i, n);
     SamplerKey k1 = key;
     k1.stream_id = p.stream;
+    const float2 s = make_float2(p.sigma[i], p.sigma[i + 1]), m = make_float2(p.mu[i], p.mu[i + 1]);
     const float2 e = sample_pair(k1, i, n);
-    return make_float2(fmaf(p.sigma[i], e.x, p.mu[i]), fmaf(p.sigma[i + 1], e.y, p.mu[i + 1]));
+    return make_float2(fmaf(s.x, e.x, m.x), fmaf(s.y, e.y, m.y));
 }
 
 // Obstacle point o = (x, y, vx, vy) in the EV frame of the plan step (origin
@@ -523,6 +533,7 @@ struct RolloutArgs {
     unsigned long long* best_key;      // packed (class, cost, index) minimum
     unsigned* work;                    // work-queue counter of the persistent collision kernel
     int grid_collide;                  // persistent grid size
+    int sm_count;                      // SMs of the device
     const LoopDev* dyn;                // when set, per-step scalars come from here
     int warm_force;                    // the warm start replaces sample 0 even before the loop's
                                        // first step (restart rounds: it is the incumbent)

@@ -33,6 +33,7 @@
 #include "../../include/npp.h"
 #include "npp_device.cuh"
 #include "npp_async.cuh"
+#include "npp_tmem.cuh"
 
 namespace npp {
 
@@ -75,8 +76,9 @@ struct ThetaSrc {
 // instead of registers (fewer registers per thread, more warps per SM):
 // unit j's quad QR + q of this lane at w2s[(j KSQ + q) G] as two packed
 // pairs, lanes of a group adjacent (conflict-free 16-byte loads).
-template <int W, int G, int KSQ = 0>
+template <int W_, int G_, int KSQ = 0>
 struct LaneNet {
+    static constexpr int W = W_, G = G_;
     using S = Shape<W, G>;
     static constexpr int U = S::U;
     static constexpr int QR = W / 4 - KSQ;        // W2 input quads per unit in registers
@@ -171,6 +173,29 @@ struct LaneNet {
         }
     }
 
+    // nothing to fetch ahead of a step (TmemNet has)
+    struct Ahead {};
+    __device__ __forceinline__ Ahead fetch_ahead() const { return {}; }
+
+    // layer 2: each unit's dot product over the group's hidden row as four
+    // interleaved partial sums (inputs i = 4q + r go to partial r),
+    // partials 0, 1 and 2, 3 as packed pairs: two FP32x2 FMAs per input
+    // quad, each half rounded as a separate fmaf
+    __device__ __forceinline__ void layer2(const float4* hrow4, Ahead&, unsigned long long (&p01)[U],
+                                           unsigned long long (&p23)[U]) const {
+#pragma unroll
+        for (int i = 0; i < W / 4; ++i) {
+            const float4 hv = hrow4[i];
+            const unsigned long long h01 = f2_pack(hv.x, hv.y), h23 = f2_pack(hv.z, hv.w);
+#pragma unroll
+            for (int j = 0; j < U; ++j) {
+                const ulonglong2 w = get_w2(j, i);
+                p01[j] = f2_fma(w.x, h01, p01[j]);
+                p23[j] = f2_fma(w.y, h23, p23[j]);
+            }
+        }
+    }
+
     // lane gl of the group holds hidden units gl*U .. gl*U + U - 1
     __device__ __forceinline__ void load(const ThetaSrc& src, int gl) {
 #pragma unroll
@@ -257,6 +282,134 @@ struct LaneNet {
         }
         b3[0] = st[(4 * NQUAD + 2 * (2 * U)) * TH];
         b3[1] = st[(4 * NQUAD + 2 * (2 * U) + 1) * TH];
+    }
+};
+
+// The weights of one lane with its W2 rows in tensor memory: input quads
+// [0, KT) of the lane's U units at 4 U columns a quad (four weights a unit)
+// of the lane's own TMEM lane, the last KS quads in shared memory (as
+// LaneNet's), W1, W3 and the biases in registers.  No tensor-core
+// instruction is involved: TMEM serves as 256 KB of per-warp storage that a
+// warp reads 16 columns at a time (tcgen05.ld), next to the register file
+// (256 KB) and shared memory.
+//
+// Why: a sample's weights decide how many samples an SM holds, and the
+// rollout step is a serial chain (layers, tanh, shuffle tree, Euler step), so
+// resident samples are what fills the pipes.
+template <int W_, int G_, int KT, int KS = 0>
+struct TmemNet {
+    static constexpr int W = W_, G = G_;
+    using S = Shape<W, G>;
+    static constexpr int U = S::U;
+    static constexpr int QC = 4 * U;              // columns of one input quad
+    static constexpr int COLS = QC * KT;          // TMEM columns of one warp
+    static constexpr int QPR = 16 / QC;           // input quads per 16-column read
+    static_assert(KT % QPR == 0 && KT + KS == W / 4, "whole 16-column reads");
+    static_assert(COLS >= (U == 2 ? 32 : 64), "the registers' parameters are staged through the columns");
+    unsigned long long w1p[U][NIN / 2];
+    float b1[U], b2[U], w3[2][U], b3[2];
+    uint32_t tm;                                  // this warp's first column (lane quarter in bits 16..)
+    ulonglong2* w2s;                              // this lane's slot of the shared quads (KS > 0)
+
+    // parameters of the lane's units from the off-th on: one value a unit.
+    // (Samples of one warp can have different sources; the store to tensor
+    // memory is the whole warp's, hence the __syncwarp before each.)
+    __device__ __forceinline__ void put_units(const ThetaSrc& src, int off, uint32_t col) {
+        if constexpr (U == 2) {
+            const float2 v = src.pair(off);
+            __syncwarp();
+            tmem_st2(col, v);
+        } else {
+            const float4 v = src.quad(off);
+            __syncwarp();
+            tmem_st4(col, v);
+        }
+    }
+
+    __device__ __forceinline__ void load(const ThetaSrc& src, int gl) {
+        // W1's quads, then the biases and W3's rows, by rolled loops (one
+        // copy of the sampler's code each) through the columns into registers
+#pragma unroll 1
+        for (int it = 0; it < U * (NIN / 4); ++it) {
+            const float4 q = src.quad(gl * U * NIN + 4 * it);
+            __syncwarp();
+            tmem_st4(tm + 4 * it, q);
+        }
+#pragma unroll 1
+        for (int k = 0; k < 4; ++k) {
+            const int off = k == 0 ? S::OFF_B1 : k == 1 ? S::OFF_B2 : k == 2 ? S::OFF_W3 : S::OFF_W3 + W;
+            put_units(src, off + gl * U, tm + U * NIN + k * U);
+        }
+        const float2 o = src.pair(S::OFF_B3);
+        b3[0] = o.x; b3[1] = o.y;
+        __syncwarp();
+        tmem_wait_st();
+        Tmem16 a[U / 2], b;
+#pragma unroll
+        for (int k = 0; k < U / 2; ++k) tmem_ld16(tm + 16 * k, a[k]);
+        tmem_ld16(tm + U * NIN, b);
+#pragma unroll
+        for (int k = 0; k < U / 2; ++k) tmem_wait_ld(a[k]);
+        tmem_wait_ld(b);
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+#pragma unroll
+            for (int i = 0; i < NIN / 2; ++i) w1p[j][i] = a[j / 2].pair((j % 2) * (NIN / 2) + i);
+            b1[j] = b.f(j); b2[j] = b.f(U + j);
+            w3[0][j] = b.f(2 * U + j); w3[1][j] = b.f(3 * U + j);
+        }
+#pragma unroll 1
+        for (int it = 0; it < U * (W / 4); ++it) {
+            const int j = it % U, qi = it / U;
+            const float4 q = src.quad(S::OFF_W2 + (gl * U + j) * W + 4 * qi);
+            __syncwarp();
+            if (KS == 0 || qi < KT) tmem_st4(tm + QC * qi + 4 * j, q);
+            else w2s[(j * KS + (qi - KT)) * G] = make_ulonglong2(f2_pack(q.x, q.y), f2_pack(q.z, q.w));
+        }
+        tmem_wait_st();
+    }
+
+    // the first 16 columns, read while layer 1 runs
+    struct Ahead { Tmem16 w; };
+    __device__ __forceinline__ Ahead fetch_ahead() const {
+        Ahead f;
+        tmem_ld16(tm, f.w);
+        return f;
+    }
+
+    // LaneNet::layer2's sums in the same order; the next 16 columns are on
+    // their way while these are multiplied
+    __device__ __forceinline__ void layer2(const float4* hrow4, Ahead& f, unsigned long long (&p01)[U],
+                                           unsigned long long (&p23)[U]) const {
+        Tmem16 buf[2];
+        buf[0] = f.w;
+#pragma unroll
+        for (int c = 0; c < KT / QPR; ++c) {
+            Tmem16& w = buf[c & 1];
+            tmem_wait_ld(w);
+            if (c + 1 < KT / QPR) tmem_ld16(tm + 16 * (c + 1), buf[(c + 1) & 1]);
+#pragma unroll
+            for (int q = 0; q < QPR; ++q) {
+                const float4 hv = hrow4[QPR * c + q];
+                const unsigned long long h01 = f2_pack(hv.x, hv.y), h23 = f2_pack(hv.z, hv.w);
+#pragma unroll
+                for (int j = 0; j < U; ++j) {
+                    p01[j] = f2_fma(w.pair(2 * U * q + 2 * j), h01, p01[j]);
+                    p23[j] = f2_fma(w.pair(2 * U * q + 2 * j + 1), h23, p23[j]);
+                }
+            }
+        }
+#pragma unroll
+        for (int i = KT; i < W / 4; ++i) {
+            const float4 hv = hrow4[i];
+            const unsigned long long h01 = f2_pack(hv.x, hv.y), h23 = f2_pack(hv.z, hv.w);
+#pragma unroll
+            for (int j = 0; j < U; ++j) {
+                const ulonglong2 w = w2s[(j * KS + (i - KT)) * G];
+                p01[j] = f2_fma(w.x, h01, p01[j]);
+                p23[j] = f2_fma(w.y, h23, p23[j]);
+            }
+        }
     }
 };
 
@@ -594,18 +747,26 @@ __device__ __forceinline__ GoalEV goal_ev(const StepIn& si)
     return g;
 }
 
-// The network of sample n (valid: n < N) loaded into the lanes of its group.
-template <int W, int G, int STAGE_TH, int KSQ = 0>
-__device__ __forceinline__ void load_net(LaneNet<W, G, KSQ>& net, const TrajJob& job, int n, bool valid, int gl)
+// Where the parameters of sample n (valid: n < N) come from.
+template <int NT>
+__device__ __forceinline__ ThetaSrc theta_src(const TrajJob& job, int n, bool valid)
 {
-    net.w2s = job.w2s;
     ThetaSrc src;
     src.key = job.key;
     src.prop = job.prop;
     src.n = (uint32_t)(valid ? n : 0);
     src.mem = nullptr;
-    if (job.theta) src.mem = job.theta + (size_t)(valid ? n : 0) * Shape<W, G>::NT;
+    if (job.theta) src.mem = job.theta + (size_t)(valid ? n : 0) * NT;
     else if (job.warm && n == 0 && job.si.warm_ok) src.mem = job.warm;
+    return src;
+}
+
+// The network of sample n loaded into the lanes of its group.
+template <int STAGE_TH = 0, int W, int G, int KSQ>
+__device__ __forceinline__ void load_net(LaneNet<W, G, KSQ>& net, const TrajJob& job, int n, bool valid, int gl)
+{
+    net.w2s = job.w2s;
+    const ThetaSrc src = theta_src<Shape<W, G>::NT>(job, n, valid);
     if constexpr (STAGE_TH > 0) net.template load_staged<STAGE_TH>(src, gl, job.stage);
     else if constexpr (KSQ > 0) net.load_rolled(src, gl);
     else net.load(src, gl);
@@ -617,13 +778,13 @@ __device__ __forceinline__ void load_net(LaneNet<W, G, KSQ>& net, const TrajJob&
 // exchange row), rate-limited controls, effort, Euler step of the kinematic
 // bicycle on the old state (Sect. IV).  Updates the state, the last
 // controls, the effort E and rem = T - h; returns the applied controls.
-template <int W, int G, bool VAR, int KSQ = 0>
-__device__ __forceinline__ float2 control_step(const DevCfg& c, const LaneNet<W, G, KSQ>& net, const GoalEV& g,
-                                               float invT, int gl, float* hrow, float sp, float cp, float& x,
-                                               float& y, float& ph, float& v, float& ap0, float& ap1, float& E,
-                                               float& rem)
+template <class Net, bool VAR>
+__device__ __forceinline__ float2 control_step(const DevCfg& c, const Net& net, const GoalEV& g, float invT,
+                                               int gl, float* hrow, float sp, float cp, float& x, float& y, float& ph,
+                                               float& v, float& ap0, float& ap1, float& E, float& rem)
 {
-    constexpr int U = Shape<W, G>::U;
+    constexpr int G = Net::G, U = Net::U;
+    typename Net::Ahead ahead = net.fetch_ahead();
     float s[NIN];
     if (VAR && c.body_frame) {
         // goal offset in the vehicle's frame at t+h
@@ -658,26 +819,12 @@ __device__ __forceinline__ float2 control_step(const DevCfg& c, const LaneNet<W,
 #pragma unroll
     for (int j = 0; j < U; ++j) hrow[gl * U + j] = h1[j];
     __syncwarp();
-    // layer 2: each unit's dot product as four interleaved partial sums
-    // (inputs i = 4q + r go to partial r), added pairwise with the bias
-    // last: independent FMA chains keep the pipe busy
-    // (partials 0, 1 and 2, 3 as packed pairs: two FP32x2 FMAs per input
-    // quad, each half rounded as a separate fmaf)
+    // layer 2: four partial sums per unit (independent FMA chains keep the
+    // pipe busy), added pairwise with the bias last
     unsigned long long p01[U], p23[U];
 #pragma unroll
     for (int j = 0; j < U; ++j) p01[j] = p23[j] = 0ull;
-    const float4* hrow4 = reinterpret_cast<const float4*>(hrow);
-#pragma unroll
-    for (int i = 0; i < W / 4; ++i) {
-        const float4 hv = hrow4[i];
-        const unsigned long long h01 = f2_pack(hv.x, hv.y), h23 = f2_pack(hv.z, hv.w);
-#pragma unroll
-        for (int j = 0; j < U; ++j) {
-            const ulonglong2 w = net.get_w2(j, i);
-            p01[j] = f2_fma(w.x, h01, p01[j]);
-            p23[j] = f2_fma(w.y, h23, p23[j]);
-        }
-    }
+    net.layer2(reinterpret_cast<const float4*>(hrow), ahead, p01, p23);
     __syncwarp();
     float acc2[U];
 #pragma unroll
@@ -738,13 +885,11 @@ __device__ __forceinline__ float final_cost(const DevCfg& c, const GoalEV& g, fl
 // of c (body-frame goal offsets, speed limits) are honoured; without it the
 // kernel is the plain rollout, and the launchers pick VAR whenever c turns
 // a variant on.
-template <int W, int G, int STAGE_TH = 0, bool VAR = false, int KSQ = 0>
-__device__ __forceinline__ void traj_sample(const DevCfg& c, const TrajJob& job, int n, bool valid, int gl,
-                                            float* hrow)
+template <bool VAR, class Net>
+__device__ __forceinline__ void traj_sample(const DevCfg& c, const TrajJob& job, const Net& net, int n, bool valid,
+                                            int gl, float* hrow)
 {
     const GoalEV g = goal_ev(job.si);
-    LaneNet<W, G, KSQ> net;
-    load_net<W, G, STAGE_TH, KSQ>(net, job, n, valid, gl);
 
     float x = 0.f, y = 0.f, ph = 0.f, v = job.si.v0, ap0 = job.si.ap0, ap1 = job.si.ap1, E = 0.f;
     const int T = job.T, N = job.N;
@@ -782,8 +927,7 @@ __device__ __forceinline__ void traj_sample(const DevCfg& c, const TrajJob& job,
                 job.coefB[ci] = B;
             }
         }
-        const float2 a = control_step<W, G, VAR, KSQ>(c, net, g, invT, gl, hrow, sp, cp, x, y, ph, v, ap0, ap1,
-                                                      E, rem);
+        const float2 a = control_step<Net, VAR>(c, net, g, invT, gl, hrow, sp, cp, x, y, ph, v, ap0, ap1, E, rem);
         if (writer && job.ctrl) job.ctrl[h * job.rec_stride + rec] = a;
     }
     if (h_hi < T) {
@@ -829,18 +973,17 @@ __device__ __forceinline__ void traj_sample(const DevCfg& c, const TrajJob& job,
 // collides).  wnd: the warp's [32/G][CW] states; steps counts the control
 // steps the warp computed (lane 0 of each valid group), ntest / nstate the
 // check's candidate tests and states.
-template <int W, int G, int STAGE_TH, bool VAR, int KSQ, int CW, int R>
-__device__ __forceinline__ FusedOut traj_sample_windowed(const DevCfg& c, const TrajJob& job, int n, bool valid,
-                                                         int gl, float* hrow, float4* wnd, unsigned& steps,
-                                                         unsigned& ntest, unsigned& nstate)
+template <bool VAR, int CW, int R, class Net>
+__device__ __forceinline__ FusedOut traj_sample_windowed(const DevCfg& c, const TrajJob& job, const Net& net, int n,
+                                                         bool valid, int gl, float* hrow, float4* wnd,
+                                                         unsigned& steps, unsigned& ntest, unsigned& nstate)
 {
+    constexpr int G = Net::G;
     constexpr int NG = 32 / G;                 // groups (samples) per warp
     constexpr int SPI = 4 / NG;                // states of a group per check round
     static_assert(NG <= 4 && 32 % G == 0, "at most four groups per warp");
     const int lane = threadIdx.x & 31, grp = lane / G;
     const GoalEV g = goal_ev(job.si);
-    LaneNet<W, G, KSQ> net;
-    load_net<W, G, STAGE_TH, KSQ>(net, job, n, valid, gl);
     const BinView& bv = *job.bins;
 
     float x = 0.f, y = 0.f, ph = 0.f, v = job.si.v0, ap0 = job.si.ap0, ap1 = job.si.ap1, E = 0.f;
@@ -865,8 +1008,8 @@ __device__ __forceinline__ FusedOut traj_sample_windowed(const DevCfg& c, const 
             if (gl == 0) wnd[grp * CW + j] = z;
             if (writer && alive && job.traj) job.traj[h * job.rec_stride + rec] = z;
             if (h < T) {
-                const float2 a = control_step<W, G, VAR, KSQ>(c, net, g, invT, gl, hrow, sp, cp, x, y, ph, v,
-                                                              ap0, ap1, E, rem);
+                const float2 a = control_step<Net, VAR>(c, net, g, invT, gl, hrow, sp, cp, x, y, ph, v, ap0, ap1,
+                                                        E, rem);
                 if (writer && alive && job.ctrl) job.ctrl[h * job.rec_stride + rec] = a;
                 ++steps;
             }
@@ -959,7 +1102,9 @@ __global__ void __launch_bounds__(NW * 32, MINB) traj_kernel(const RolloutArgs a
         job.h_hi = a.chunk_hi;
         job.carry = a.carry;
     }
-    traj_sample<W, G, STAGE_TH, VAR, KSQ>(a.c, job, n, valid, gl, hx_all + b * W);
+    LaneNet<W, G, KSQ> net;
+    load_net<STAGE_TH>(net, job, n, valid, gl);
+    traj_sample<VAR>(a.c, job, net, n, valid, gl, hx_all + b * W);
     // measurement: sample-steps computed (timing on)
     if (a.counts && valid && gl == 0)
         atomicAdd(a.counts + 2, (unsigned long long)((a.chunk_hi > 0 ? a.chunk_hi : a.T) - a.chunk_lo));
@@ -1019,9 +1164,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_kernel(const RolloutArgs 
     float4* wnd = reinterpret_cast<float4*>(reinterpret_cast<char*>(stage_all) + traj_stage_bytes<W, G, NW, KSQ>()) +
                   (size_t)(tid / 32) * (32 / G) * CW;
     unsigned steps = 0, ntest = 0, nstate = 0;
-    const FusedOut r = traj_sample_windowed<W, G, STAGE_TH, VAR, KSQ, CW, R>(a.c, job, n, valid, gl,
-                                                                              hx_all + b * W, wnd, steps, ntest,
-                                                                              nstate);
+    LaneNet<W, G, KSQ> net;
+    load_net<STAGE_TH>(net, job, n, valid, gl);
+    const FusedOut r = traj_sample_windowed<VAR, CW, R>(a.c, job, net, n, valid, gl, hx_all + b * W, wnd, steps,
+                                                        ntest, nstate);
     if (valid && gl == 0) {
         unsigned long long key;
         if (r.first_hit < 0)
@@ -1047,6 +1193,155 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_kernel(const RolloutArgs 
         }
         if (valid && gl == 0) atomicAdd(a.counts + 2, (unsigned long long)steps);
     }
+}
+
+// ------------------------------------------------------------------ kernels with tensor-memory weights
+// TMEM columns a block of NW warps allocates (a power of two, 32 or more):
+// warps w, w + 4, ... share lane quarter w % 4, each with its own columns.
+template <class Net, int NW>
+__host__ __device__ constexpr int tmem_cols()
+{
+    int need = NW / 4 * Net::COLS, c = 32;
+    while (c < need) c *= 2;
+    return c;
+}
+
+template <int W, int G>
+__device__ __forceinline__ TrajJob traj_job(const RolloutArgs& a)
+{
+    TrajJob job;
+    job.si = step_in(a);
+    job.key = a.key;
+    job.key.t_index = job.si.t_index;
+    job.theta = a.theta;
+    job.warm = a.warm;
+    job.prop = a.prop;
+    job.N = a.N;
+    job.T = a.T;
+    job.traj = a.traj;
+    job.ctrl = a.ctrl;
+    job.rec_stride = a.N;
+    job.rec_shift = 0;
+    job.coefA = nullptr;
+    job.coefB = nullptr;
+    job.coef_base = 0;
+    job.jfree = a.jfree;
+    job.vfirst = a.c.vlim ? a.vfirst : nullptr;
+    job.bins = nullptr;
+    job.stage = nullptr;
+    job.w2s = nullptr;
+    return job;
+}
+
+// shared memory of a block: the hidden rows, the windows (CW > 0), the
+// shared W2 quads
+template <int W, int G, int NW, int KS, int CW>
+constexpr int tmem_block_bytes()
+{
+    return NW * 32 * (W / G) * KS * 16 + NW * (32 / G) * (CW * 16 + W * 4);
+}
+
+// Trajectories, one sample per group (as traj_kernel).
+template <int W, int G, int NW, int MINB, bool VAR, int KT, int KS>
+__global__ void __launch_bounds__(NW * 32, MINB) traj_tmem_kernel(const RolloutArgs a)
+{
+    using Net = TmemNet<W, G, KT, KS>;
+    static_assert(NW % 4 == 0 && tmem_cols<Net, NW>() * MINB <= 512, "the blocks of an SM fit its TMEM");
+    extern __shared__ __align__(16) ulonglong2 w2_all[];
+    __shared__ uint32_t tslot;
+    constexpr int B = NW * 32 / G;
+    float* hx_all = reinterpret_cast<float*>(w2_all + NW * 32 * Net::U * KS);
+    const int tid = threadIdx.x, b = tid / G, gl = tid % G, warp = tid >> 5;
+    const uint32_t tmem = tmem_alloc<tmem_cols<Net, NW>()>(&tslot);
+    int n = blockIdx.x * B + b;
+    bool valid = n < a.N;
+    bool idle = false;
+    if (a.live_in) {
+        const int cnt = *a.live_n_in;
+        idle = (int)blockIdx.x * B >= cnt;
+        valid = n < cnt;
+        n = valid ? a.live_in[n] : 0;
+    }
+    if (!idle) {
+        TrajJob job = traj_job<W, G>(a);
+        if (a.chunk_hi > 0) {
+            job.h_lo = a.chunk_lo;
+            job.h_hi = a.chunk_hi;
+            job.carry = a.carry;
+        }
+        Net net;
+        net.tm = tmem + ((uint32_t)(warp & 3) << 21) + (uint32_t)((warp >> 2) * Net::COLS);
+        net.w2s = w2_all + (size_t)b * (Net::U * KS * G) + gl;
+        net.load(theta_src<Net::S::NT>(job, n, valid), gl);
+        traj_sample<VAR>(a.c, job, net, n, valid, gl, hx_all + b * W);
+        if (a.counts && valid && gl == 0)
+            atomicAdd(a.counts + 2, (unsigned long long)((a.chunk_hi > 0 ? a.chunk_hi : a.T) - a.chunk_lo));
+    }
+    tmem_free<tmem_cols<Net, NW>()>(tmem);
+}
+
+// Trajectories with the windowed check (as fused_kernel): the warps of a
+// resident grid take samples from a queue, so that a warp whose sample ends
+// early starts another at once (a.work: the samples taken so far).
+template <int W, int G, int NW, int MINB, bool VAR, int KT, int KS, int CW, int R>
+__global__ void __launch_bounds__(NW * 32, MINB) fused_tmem_kernel(const RolloutArgs a)
+{
+    using Net = TmemNet<W, G, KT, KS>;
+    static_assert(NW % 4 == 0 && tmem_cols<Net, NW>() * MINB <= 512, "the blocks of an SM fit its TMEM");
+    extern __shared__ __align__(16) ulonglong2 w2_all[];
+    __shared__ uint32_t tslot;
+    constexpr int NG = 32 / G;
+    float4* wnd_all = reinterpret_cast<float4*>(w2_all + NW * 32 * Net::U * KS);
+    float* hx_all = reinterpret_cast<float*>(wnd_all + NW * NG * CW);
+    const int tid = threadIdx.x, b = tid / G, gl = tid % G, warp = tid >> 5, lane = tid & 31;
+    const uint32_t tmem = tmem_alloc<tmem_cols<Net, NW>()>(&tslot);
+    TrajJob job = traj_job<W, G>(a);
+    job.jfree = nullptr;
+    job.vfirst = nullptr;
+    job.bins = &a.bins;
+    Net net;
+    net.tm = tmem + ((uint32_t)(warp & 3) << 21) + (uint32_t)((warp >> 2) * Net::COLS);
+    net.w2s = w2_all + (size_t)b * (Net::U * KS * G) + gl;
+    unsigned steps = 0, ntest = 0, nstate = 0;
+    for (;;) {
+        unsigned n0 = 0;
+        if (lane == 0) n0 = atomicAdd(a.work, (unsigned)NG);
+        n0 = __shfl_sync(FULL, n0, 0);
+        if (n0 >= (unsigned)a.N) break;
+        const int n = (int)n0 + lane / G;
+        const bool valid = n < a.N;
+        net.load(theta_src<Net::S::NT>(job, n, valid), gl);
+        unsigned st = 0;
+        const FusedOut r = traj_sample_windowed<VAR, CW, R>(a.c, job, net, n, valid, gl, hx_all + b * W,
+                                                            wnd_all + warp * NG * CW, st, ntest, nstate);
+        if (valid && gl == 0) {
+            steps += st;
+            unsigned long long key;
+            if (r.first_hit < 0)
+                key = ((unsigned long long)__float_as_uint(r.cost) << 32) | (unsigned)n;
+            else
+                key = (1ull << 63) | ((unsigned long long)(a.T - r.first_hit) << 32) | (unsigned)n;
+            if (a.costs) a.costs[n] = r.cost;
+            if (a.first_hit) a.first_hit[n] = r.first_hit;
+            // the read skips atomics that cannot win
+            if (a.best_key && key < *reinterpret_cast<volatile unsigned long long*>(a.best_key))
+                atomicMin(a.best_key, key);
+        }
+    }
+    if (a.counts) {
+        unsigned long long t = ntest, s = nstate;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            t += __shfl_xor_sync(FULL, t, off);
+            s += __shfl_xor_sync(FULL, s, off);
+        }
+        if (lane == 0) {
+            atomicAdd(a.counts, t);
+            atomicAdd(a.counts + 1, s);
+        }
+        if (gl == 0) atomicAdd(a.counts + 2, (unsigned long long)steps);
+    }
+    tmem_free<tmem_cols<Net, NW>()>(tmem);
 }
 
 // ------------------------------------------------------------------ collide
@@ -1642,6 +1937,43 @@ cudaError_t launch_fused(const RolloutArgs& a, cudaStream_t stream)
     cudaError_t e = ensure_smem(fused_kernel<W, G, NW, MINB, VAR, KSQ, CW, R>, smem);
     if (e != cudaSuccess) return e;
     fused_kernel<W, G, NW, MINB, VAR, KSQ, CW, R><<<grid, K::THREADS, smem, stream>>>(a);
+    return cudaGetLastError();
+}
+
+// Whether widths 16 and 32 take four hidden units a lane (half the warps for
+// the same samples) instead of two, whose blocks hold `block` samples: from
+// the samples on that put two of those blocks on one SM (7/8: the scheduler
+// doubles up before every SM has one, and the check's grids are built beside
+// the trajectories).  Below, a block has its SM to itself and the shorter
+// chain of two units decides; above, the fewer instructions.  GB300, plan
+// steps one after another, four / two units (us): width 16, T = 40: N = 1024
+// 43 / 39, 2048 45 / 43, 4096 49 / 55, 6000 64 / 64, 8192 67 / 69; width 32:
+// 1024 53 / 44, 2048 54 / 56, 4096 68 / 70, 6000 83 / 91, 8192 95 / 110.
+inline bool rollout_wide(const RolloutArgs& a, int block)
+{
+    return (a.N + block - 1) / block > a.sm_count * 7 / 8;
+}
+
+template <int W, int G, int NW, int MINB, bool VAR, int KT, int KS = 0>
+cudaError_t launch_traj_tmem(const RolloutArgs& a, cudaStream_t stream)
+{
+    auto fn = traj_tmem_kernel<W, G, NW, MINB, VAR, KT, KS>;
+    constexpr int B = NW * 32 / G, smem = tmem_block_bytes<W, G, NW, KS, 0>();
+    cudaError_t e = ensure_smem(fn, smem);
+    if (e != cudaSuccess) return e;
+    fn<<<(a.N + B - 1) / B, NW * 32, smem, stream>>>(a);
+    return cudaGetLastError();
+}
+
+template <int W, int G, int NW, int MINB, bool VAR, int KT, int KS, int CW = 8, int R = 4>
+cudaError_t launch_fused_tmem(const RolloutArgs& a, cudaStream_t stream)
+{
+    auto fn = fused_tmem_kernel<W, G, NW, MINB, VAR, KT, KS, CW, R>;
+    constexpr int B = NW * 32 / G, smem = tmem_block_bytes<W, G, NW, KS, CW>();
+    cudaError_t e = ensure_smem(fn, smem);
+    if (e == cudaSuccess) e = cudaMemsetAsync(a.work, 0, sizeof(unsigned), stream);
+    if (e != cudaSuccess) return e;
+    fn<<<min((a.N + B - 1) / B, MINB * a.sm_count), NW * 32, smem, stream>>>(a);
     return cudaGetLastError();
 }
 

@@ -1,25 +1,30 @@
-// Trajectory kernel for the 8-16-16-2 network.  Launch shapes (all compute
-// identical values): 0 (default) <16, 8, 8, 3>, eight-warp blocks at three
-// per SM (24 warps) -- measured on GB300 8-11 % faster than <16, 8, 4, 4>
-// (16 warps per SM) on the parking scene (N = 16384, T = 60), the road at
-// the paper's horizon (N = 20480, T = 200) and the course (N = 16384,
-// T = 40); 1 four hidden units per lane, 2 eight-warp blocks with no
-// occupancy hint, 3 <16, 8, 4, 4>; template arguments <width, lanes per
-// sample, warps per block, blocks per SM hint>.
+// Trajectory kernels for the 8-16-16-2 network.  Launch shapes (all compute
+// identical values), template arguments <width, lanes per sample, warps per
+// block, blocks per SM, variants, W2 quads in tensor memory>:
+//   0 (default) 1 or 2 by the number of samples (rollout_wide)
+//   1 four hidden units a lane, eight samples a warp: fewer instructions per
+//     sample, so the faster one where samples fill the SMs
+//   2 two units a lane, four samples a warp: more warps from the same
+//     samples and a shorter chain per step, so the faster one below
+//   3, 4 every weight in registers <16, 8, 4, 4>
+// Measured on GB300 (trajectories, us; 1 / 2 / the earlier default in
+// registers): road N = 20480, T = 200: 223 / 248 / 280; course N = 16384,
+// T = 40: 58 / 70 / 72; N = 4096: 38 / 37 / 42; N = 256, T = 20: 20 / 18 / 20.
 #include "npp_rollout.cuh"
 
 namespace npp {
 
+template <bool VAR>
+static cudaError_t traj(const RolloutArgs& a, cudaStream_t s, bool wide)
+{
+    return wide ? launch_traj_tmem<16, 4, 4, 4, VAR, 4>(a, s) : launch_traj_tmem<16, 8, 4, 6, VAR, 4>(a, s);
+}
+
 cudaError_t launch_traj_w16(const RolloutArgs& a, cudaStream_t s, int variant)
 {
-    // rollout variants run in the default shape
-    if (uses_variants(a.c)) return launch_traj<16, 8, 4, 4, true>(a, s);
-    switch (variant) {
-    case 1: return launch_traj<16, 4, 8>(a, s);
-    case 2: return launch_traj<16, 8, 8>(a, s);
-    case 3: return launch_traj<16, 8, 4, 4>(a, s);
-    default: return launch_traj<16, 8, 8, 3>(a, s);
-    }
+    const bool wide = variant == 1 || (variant != 2 && rollout_wide(a, 16));
+    if (uses_variants(a.c)) return traj<true>(a, s, wide);
+    return variant >= 3 ? launch_traj<16, 8, 4, 4>(a, s) : traj<false>(a, s, wide);
 }
 
 // Trajectories with the windowed binned check (fused_kernel; template

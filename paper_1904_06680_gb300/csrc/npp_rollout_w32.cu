@@ -1,26 +1,30 @@
-// Trajectory kernel for the 8-32-32-2 network.  Launch shapes (all compute
-// identical values): 0 (default, fastest measured on GB300) <32, 16, 4, 4>,
-// 1 four hidden units per lane, 2 eight-warp blocks, 3 <32, 16, 8, 3>, 4 the
-// last 5 of each lane's 8 W2 input quads in shared memory (5 KB per warp;
-// parameters generated by rolled loops through those slots) so that 20
-// warps fit per SM (measured 0.161 against 0.164 ms on the course: this
-// width is not bound by occupancy, so it is not the default);
-// template arguments <width, lanes per sample, warps per block, blocks per SM hint>.
+// Trajectory kernels for the 8-32-32-2 network.  Launch shapes (all compute
+// identical values), template arguments <width, lanes per sample, warps per
+// block, blocks per SM, variants, W2 quads in tensor memory>:
+//   0 (default) 1 or 2 by the number of samples (rollout_wide)
+//   1 four hidden units a lane, four samples a warp (64 samples per SM)
+//   2 two units a lane, two samples a warp (40 samples per SM)
+//   3, 4 every weight in registers <32, 16, 4, 4>
+// Measured on GB300 (trajectories, us; 1 / 2 / the earlier default in
+// registers): N = 40000, T = 40: 254 / 306 / 318; course N = 16384: 123 /
+// 138 / 143; N = 8192: 74 / 86 / 89; N = 5003, T = 60: 91 / 75 / 85; N = 500,
+// T = 40: 39 / 32 / 32.  Shape 1 issues about 285 warp instructions per step
+// of four samples, 2 about 225 per step of two.
 #include "npp_rollout.cuh"
 
 namespace npp {
 
+template <bool VAR>
+static cudaError_t traj(const RolloutArgs& a, cudaStream_t s, bool wide)
+{
+    return wide ? launch_traj_tmem<32, 8, 4, 4, VAR, 8>(a, s) : launch_traj_tmem<32, 16, 4, 5, VAR, 8>(a, s);
+}
+
 cudaError_t launch_traj_w32(const RolloutArgs& a, cudaStream_t s, int variant)
 {
-    // rollout variants run in the default shape
-    if (uses_variants(a.c)) return launch_traj<32, 16, 4, 4, true>(a, s);
-    switch (variant) {
-    case 1: return launch_traj<32, 8, 8>(a, s);
-    case 2: return launch_traj<32, 16, 8>(a, s);
-    case 3: return launch_traj<32, 16, 8, 3>(a, s);
-    case 4: return launch_traj<32, 16, 4, 5, false, 5>(a, s);
-    default: return launch_traj<32, 16, 4, 4>(a, s);
-    }
+    const bool wide = variant == 1 || (variant != 2 && rollout_wide(a, 8));
+    if (uses_variants(a.c)) return traj<true>(a, s, wide);
+    return variant >= 3 ? launch_traj<32, 16, 4, 4>(a, s) : traj<false>(a, s, wide);
 }
 
 // Trajectories with the windowed binned check (fused_kernel; template

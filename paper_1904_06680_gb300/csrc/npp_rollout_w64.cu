@@ -1,45 +1,57 @@
-// Trajectory kernel for the 8-64-64-2 network.  Launch shapes (all compute
-// identical values): 0 (default, fastest measured on GB300: 3.29 against
-// 4.02 ms at N = 65536, T = 100) the last 8 of each lane's 16 W2 input quads
-// in shared memory (8 KB per warp), so that 127 registers without spills
-// and 16 one-warp blocks fit per SM, parameters generated by rolled loops; 1 four hidden units per lane, 2
-// eight-warp blocks, 3 <64, 32, 2, 5>, 4 every weight in registers
-// <64, 32, 1, 10> (168 registers with spills, 12 warps per SM);
-// template arguments <width, lanes per sample, warps per block, blocks per SM hint>.
+// Trajectory kernels for the 8-64-64-2 network.  Launch shapes (all compute
+// identical values), template arguments <width, lanes per sample, warps per
+// block, blocks per SM, variants, W2 quads in tensor memory, in shared
+// memory>:
+//   0 (default) 1 from 16384 samples on, else 2
+//   1 four hidden units a lane, two samples a warp, half of W2 in shared
+//     memory (24 samples per SM)
+//   2 two units a lane, one sample a warp, W2 in tensor memory (16 per SM)
+//   3, 4 the last 8 of each lane's 16 W2 quads in shared memory, the rest in
+//     registers <64, 32, 1, 16, false, 8>
+// Measured on GB300 (trajectories, us; 1 / 2 / 3): N = 65536, T = 100: 2590 /
+// 2782 / 3321; N = 2000, T = 50: 104 / 78 / 96.  A wave of shape 1 holds 3648
+// samples and takes 1.4 times a wave of 2 (2432 samples), so rounding to
+// waves decides below a few of them.
 #include "npp_rollout.cuh"
 
 namespace npp {
 
-cudaError_t launch_traj_w64(const RolloutArgs& a, cudaStream_t s, int variant)
+template <bool VAR>
+static cudaError_t traj(const RolloutArgs& a, cudaStream_t s, bool wide)
 {
-    // rollout variants run in the default shape
-    if (uses_variants(a.c)) return launch_traj<64, 32, 1, 16, true, 8>(a, s);
-    switch (variant) {
-    case 1: return launch_traj<64, 16, 8>(a, s);
-    case 2: return launch_traj<64, 32, 8>(a, s);
-    case 3: return launch_traj<64, 32, 2, 5>(a, s);
-    case 4: return launch_traj<64, 32, 1, 10>(a, s);
-    default: return launch_traj<64, 32, 1, 16, false, 8>(a, s);
-    }
+    return wide ? launch_traj_tmem<64, 16, 4, 3, VAR, 8, 8>(a, s) : launch_traj_tmem<64, 32, 4, 4, VAR, 16>(a, s);
 }
 
-// Trajectories with the windowed binned check (fused_kernel; template
-// arguments after the trajectory kernel's: window of states, candidates
-// loaded ahead per lane).  Measured on GB300 at N = 65536, T = 100,
-// M = 8192 (ms per plan step): 0 (default) 12 W2 quads of 16 in shared
-// memory, windows of 8 states: 2.68; 1 10 quads, windows of 16: 2.76;
-// 2 12 quads, windows of 16: 2.73; 3 and 4 with 8 candidates ahead: 2.94 -
-// 2.98 (no register left for them without spills).
+cudaError_t launch_traj_w64(const RolloutArgs& a, cudaStream_t s, int variant)
+{
+    const bool wide = variant == 1 || (variant != 2 && a.N >= 16384);
+    if (uses_variants(a.c)) return traj<true>(a, s, wide);
+    return variant >= 3 ? launch_traj<64, 32, 1, 16, false, 8>(a, s) : traj<false>(a, s, wide);
+}
+
+// Trajectories with the windowed binned check (template arguments after the
+// trajectory kernel's: window of states, candidates loaded ahead per lane).
+// Default: 20 warps per SM in one block, 12 of 16 W2 quads in tensor memory
+// and 4 in shared memory, windows of 8 states; for samples that do not fill
+// those blocks (16 per SM), four-warp blocks with W2 in tensor memory.
+// Measured on GB300 at N = 65536, T = 100, M = 8192 (us): 1993; 16 warps per
+// SM 2018, 24 (10 quads in tensor memory) 1989; shape 3, the earlier default
+// in registers and shared memory (one sample per block), 2458.  (Windows of 4
+// states take 1940, but the library's work counters are defined by windows of
+// 8.)  At N = 2000, T = 50: four-warp blocks 85,
+// 20-warp blocks 95, shape 3 85.
+template <bool VAR>
+static cudaError_t fused(const RolloutArgs& a, cudaStream_t s, bool full)
+{
+    return full ? launch_fused_tmem<64, 32, 20, 1, VAR, 12, 4, 8, 4>(a, s)
+                : launch_fused_tmem<64, 32, 4, 4, VAR, 16, 0, 8, 4>(a, s);
+}
+
 cudaError_t launch_fused_w64(const RolloutArgs& a, cudaStream_t s, int variant)
 {
-    if (uses_variants(a.c)) return launch_fused<64, 32, 1, 16, true, 12, 8, 4>(a, s);
-    switch (variant) {
-    case 1: return launch_fused<64, 32, 1, 16, false, 10, 16, 4>(a, s);
-    case 2: return launch_fused<64, 32, 1, 16, false, 12, 16, 4>(a, s);
-    case 3: return launch_fused<64, 32, 1, 16, false, 12, 16, 8>(a, s);
-    case 4: return launch_fused<64, 32, 1, 16, false, 8, 8, 4>(a, s);
-    default: return launch_fused<64, 32, 1, 16, false, 12, 8, 4>(a, s);
-    }
+    const bool full = variant == 1 || (variant != 2 && a.N >= 16 * a.sm_count);
+    if (uses_variants(a.c)) return fused<true>(a, s, full);
+    return variant >= 3 ? launch_fused<64, 32, 1, 16, false, 12, 8, 4>(a, s) : fused<false>(a, s, full);
 }
 
 }  // namespace npp
