@@ -326,7 +326,63 @@ struct TmemNet {
         }
     }
 
+    // W2 quad `it` of the lane (unit it % U, input quad it / U) to its columns
+    // or shared slot
+    __device__ __forceinline__ void put_w2(int it, const float4& q) {
+        const int j = it % U, qi = it / U;
+        if (KS == 0 || qi < KT) tmem_st4(tm + QC * qi + 4 * j, q);
+        else w2s[(j * KS + (qi - KT)) * G] = make_ulonglong2(f2_pack(q.x, q.y), f2_pack(q.z, q.w));
+    }
+
+    // Explicit parameters: the lane's rows from memory, eight quads' loads in
+    // flight (one at a time, as the sampled ones are made, each would wait
+    // for the one before: 5003 rows at width 32, T = 60, with their check 106
+    // us, so 96).
+    __device__ __forceinline__ void load_mem(const float* m, int gl) {
+        const bool vec = (reinterpret_cast<uintptr_t>(m) & 7u) == 0;
+        const auto quad = [&](int i) {
+            if (vec) {
+                const float2 a = __ldg(reinterpret_cast<const float2*>(m + i));
+                const float2 b = __ldg(reinterpret_cast<const float2*>(m + i + 2));
+                return make_float4(a.x, a.y, b.x, b.y);
+            }
+            return make_float4(m[i], m[i + 1], m[i + 2], m[i + 3]);
+        };
+#pragma unroll
+        for (int j = 0; j < U; ++j) {
+#pragma unroll
+            for (int i = 0; i < NIN; i += 4) {
+                const float4 q = quad((gl * U + j) * NIN + i);
+                w1p[j][i / 2] = f2_pack(q.x, q.y);
+                w1p[j][i / 2 + 1] = f2_pack(q.z, q.w);
+            }
+            b1[j] = m[S::OFF_B1 + gl * U + j];
+            b2[j] = m[S::OFF_B2 + gl * U + j];
+            w3[0][j] = m[S::OFF_W3 + gl * U + j];
+            w3[1][j] = m[S::OFF_W3 + W + gl * U + j];
+        }
+        b3[0] = m[S::OFF_B3]; b3[1] = m[S::OFF_B3 + 1];
+        constexpr int B = 8;
+        static_assert(U * (W / 4) % B == 0, "whole rounds");
+#pragma unroll 1
+        for (int it = 0; it < U * (W / 4); it += B) {
+            float4 q[B];
+#pragma unroll
+            for (int k = 0; k < B; ++k)
+                q[k] = quad(S::OFF_W2 + (gl * U + (it + k) % U) * W + 4 * ((it + k) / U));
+#pragma unroll
+            for (int k = 0; k < B; ++k) put_w2(it + k, q[k]);
+        }
+        tmem_wait_st();
+    }
+
     __device__ __forceinline__ void load(const ThetaSrc& src, int gl) {
+        // explicit rows for all of the warp's samples (uniform: the store to
+        // tensor memory is the whole warp's)
+        if (__all_sync(FULL, src.mem != nullptr)) {
+            load_mem(src.mem, gl);
+            return;
+        }
         // W1's quads, then the biases and W3's rows, by rolled loops (one
         // copy of the sampler's code each) through the columns into registers
 #pragma unroll 1
@@ -360,11 +416,9 @@ struct TmemNet {
         }
 #pragma unroll 1
         for (int it = 0; it < U * (W / 4); ++it) {
-            const int j = it % U, qi = it / U;
-            const float4 q = src.quad(S::OFF_W2 + (gl * U + j) * W + 4 * qi);
+            const float4 q = src.quad(S::OFF_W2 + (gl * U + it % U) * W + 4 * (it / U));
             __syncwarp();
-            if (KS == 0 || qi < KT) tmem_st4(tm + QC * qi + 4 * j, q);
-            else w2s[(j * KS + (qi - KT)) * G] = make_ulonglong2(f2_pack(q.x, q.y), f2_pack(q.z, q.w));
+            put_w2(it, q);
         }
         tmem_wait_st();
     }
