@@ -283,12 +283,12 @@ npp_status run_rollout(npp_handle* h, RolloutArgs& a, cudaStream_t s, bool no_re
         if (h->timing) CUDA_TRY(h, record_event(h->ev[0], s));
         CUDA_TRY(h, cudaEventRecord(h->fork_ev, s));
         CUDA_TRY(h, cudaStreamWaitEvent(h->side, h->fork_ev, 0));
-        CUDA_TRY(h, build_bins_radius(a, h->fp_radius, h->d_bins, h->side));
+        CUDA_TRY(h, build_bins_poly(a, h->fp_radius, h->fp_box, h->d_bins, h->side));
         CUDA_TRY(h, cudaEventRecord(h->join_ev, h->side));
         CUDA_TRY(h, launch_traj(h, a, s));
         if (h->timing) CUDA_TRY(h, record_event(h->ev[1], s));
         CUDA_TRY(h, cudaStreamWaitEvent(s, h->join_ev, 0));
-        CUDA_TRY(h, launch_collide_poly(a, s));
+        CUDA_TRY(h, a.poly.brute ? launch_collide_poly(a, s) : launch_collide_binned(a, s));
         if (h->timing) CUDA_TRY(h, record_event(h->ev[2], s));
         return NPP_OK;
     }
@@ -730,7 +730,7 @@ npp_status npp_set_footprint(npp_handle* h, const float* verts_host, const int32
     const int nv = piece_start_host[n_pieces];
     if (nv > FP_MAX_FACES) return fail(h, NPP_INVALID_ARG, "at most %d vertices in total", FP_MAX_FACES);
     float4 faces[FP_MAX_FACES];
-    double radius = 0.0;
+    double radius = 0.0, box[4] = { 0.0, 0.0, 0.0, 0.0 };
     const double TWO_PI = 6.283185307179586;
     for (int k = 0; k < n_pieces; ++k) {
         const int b = piece_start_host[k], e = piece_start_host[k + 1], n = e - b;
@@ -754,6 +754,11 @@ npp_status npp_set_footprint(npp_handle* h, const float* verts_host, const int32
             faces[b + i] = make_float4((float)nx, (float)ny, (float)(nx * v0[0] + ny * v0[1]),
                                        i == n - 1 ? 1.0f : 0.0f);
             radius = std::fmax(radius, std::sqrt((double)v0[0] * v0[0] + (double)v0[1] * v0[1]));
+            const bool first = b + i == 0;
+            box[0] = first ? v0[0] : std::fmin(box[0], (double)v0[0]);
+            box[1] = first ? v0[0] : std::fmax(box[1], (double)v0[0]);
+            box[2] = first ? v0[1] : std::fmin(box[2], (double)v0[1]);
+            box[3] = first ? v0[1] : std::fmax(box[3], (double)v0[1]);
         }
         if (std::fabs(turn - TWO_PI) > 1e-6)
             return fail(h, NPP_INVALID_ARG, "piece %d winds more than once", k);
@@ -763,6 +768,7 @@ npp_status npp_set_footprint(npp_handle* h, const float* verts_host, const int32
     CUDA_TRY(h, cudaMemcpy(h->d_fp, faces, sizeof(float4) * nv, cudaMemcpyHostToDevice));
     h->fp_faces = nv;
     h->fp_radius = radius;
+    std::memcpy(h->fp_box, box, sizeof box);
     return NPP_OK;
 }
 

@@ -560,11 +560,15 @@ __global__ void __launch_bounds__(256) batch_binned_kernel(const BatchArgs b)
             const float cp = ca.x * isl, sp = ca.y * isl;
             const float along = -ca.z * isl, across = -cb.y * isw;
             const float xc = cp * along - sp * across, yc = sp * along + cp * across;
+            // the box around the rectangle at its recovered centre (the
+            // margin far above the rounding of this reconstruction)
+            const float rx = fmaf(g.hl, fabsf(cp), fmaf(g.hw, fabsf(sp), 0.05f));
+            const float ry = fmaf(g.hl, fabsf(sp), fmaf(g.hw, fabsf(cp), 0.05f));
             const int hq = ok ? h : 0;
             unsigned ntest = 0;
             const bool inside = binned_rows_inside<1>(g, b.bin_cs + s.bin_off + (size_t)hq * BIN_CS_STRIDE,
-                                                      b.bin_pts + s.bpts_off + (size_t)hq * M, ca, cb, xc, yc,
-                                                      b.reach, ok, gl, ntest);
+                                                      b.bin_pts + s.bpts_off + (size_t)hq * M, RectTest{ ca, cb },
+                                                      QueryBox{ xc, yc, fminf(rx, g.reach), fminf(ry, g.reach) }, ok, gl, ntest);
             const unsigned bal = __ballot_sync(FULL, inside);
             unsigned steps_hit = 0;
 #pragma unroll

@@ -5,11 +5,11 @@
 // For every horizon step h the obstacle points at time h Ts (EV frame,
 // p + tau v with the brute-force kernels' arithmetic) are counting-sorted into
 // a uniform grid of BIN_DIM x BIN_DIM cells centred on the vehicle.  A cell is
-// wider than half the radius of the vehicle rectangle's circumscribed disk
-// (plus a rounding margin), so a state's disk overlaps at most 5 x 5 cells
-// (rows of cells are contiguous runs: at most five per query, `cand_rows`); every
-// point inside the rectangle lies in the disk, and cell indices of
-// points and of the query are clamped to the grid the same (monotone) way,
+// wider than half the radius of the vehicle's disk around its reference point
+// (plus a rounding margin), so the box around a state's vehicle overlaps at
+// most 5 x 5 cells (rows of cells are contiguous runs: at most five per query,
+// `cand_rows`); every point inside the vehicle lies in the box, and cell
+// indices of points and of the query are clamped to the grid the same (monotone) way,
 // so the queried cells hold every point that can be inside.  The per-point
 // test is the brute-force one (same coefficients, same fma sequence), hence
 // the collision flags are identical to checking all points.
@@ -45,7 +45,7 @@ __global__ void __launch_bounds__(BIN_THREADS) bin_build_kernel(const RolloutArg
 // once, an 8-lane group per step: a step's candidates are the points of at
 // most five cell rows, each row's cells contiguous in the sorted array; the
 // group's lanes stride through each row's run, one candidate per row and
-// lane loaded ahead (binned_item_inside_rows; longer rows one pass at a time
+// lane loaded ahead (binned_rows_inside; longer rows one pass at a time
 // after them).  The chunk's first colliding step, if any, ends the sample.  Steps
 // are independent given the stored states, so checking a few past the first
 // collision changes nothing; it replaces one chain of two dependent loads
@@ -54,12 +54,18 @@ constexpr int BINNED_WARPS = 8;
 constexpr int BIN_SB = 32 / BIN_ITEM_LANES; // steps per chunk
 constexpr int BIN_GS = BIN_ITEM_LANES;      // lanes per step
 
+template <bool POLY>
 __global__ void __launch_bounds__(BINNED_WARPS * 32, 5) collide_binned_kernel(const RolloutArgs a)
 {
+    __shared__ float4 faces[POLY ? FP_MAX_FACES : 1];
+    if constexpr (POLY) {
+        for (int i = threadIdx.x; i < a.poly.n_faces; i += blockDim.x) faces[i] = a.poly.faces[i];
+        __syncthreads();
+    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int gid = lane / BIN_GS, gl = lane % BIN_GS;
     const BinView& g = a.bins;
-    const int T = a.T, N = a.N, M = a.M;
+    const int T = a.T, N = a.N;
     int n = blockIdx.x * BINNED_WARPS + warp;
     bool valid = n < N;
     if (a.live_in) {
@@ -80,11 +86,22 @@ __global__ void __launch_bounds__(BINNED_WARPS * 32, 5) collide_binned_kernel(co
         for (int h0 = hs; h0 <= he; h0 += BIN_SB) {
             const int h = h0 + gid;
             const bool ok = h <= he;
-            // the rectangle lies in the disk of radius reach around the
-            // reference point (reach covers the centre offset)
             const float4 z = ok ? a.traj[(size_t)h * N + n] : make_float4(0.f, 0.f, 0.f, 0.f);
             nstate += (ok && gl == 0) ? 1u : 0u;
-            const bool inside = binned_item_inside_rows<1>(a.c, g, z, h, ok, gl, ntest);
+            float sp, cp;
+            sincos_r(z.z, sp, cp);
+            const int* cs = g.cell_start + (size_t)(ok ? h : 0) * BIN_CS_STRIDE;
+            const float2* pts = g.pts + (size_t)(ok ? h : 0) * g.M;
+            const QueryBox qb = query_box(g, z.x, z.y, sp, cp);
+            bool inside;
+            if constexpr (POLY) {
+                const PolyTest test = { faces, a.poly.n_faces, a.poly.r2, z.x, z.y, cp, sp };
+                inside = binned_rows_inside<1>(g, cs, pts, test, qb, ok, gl, ntest);
+            } else {
+                RectTest test;
+                coef_rows(a.c, z.x, z.y, sp, cp, test.a, test.b);
+                inside = binned_rows_inside<1>(g, cs, pts, test, qb, ok, gl, ntest);
+            }
             const unsigned bal = __ballot_sync(FULL, inside);
             unsigned steps_hit = 0;
 #pragma unroll
@@ -142,20 +159,9 @@ size_t binned_workspace_bytes(int max_T, int max_M)
     return (size_t)(max_T + 1) * BIN_CS_STRIDE * sizeof(int) + (size_t)(max_T + 1) * max_M * sizeof(float2);
 }
 
-// Cells wider than half the radius of the query disk (circumradius of the
-// rectangle plus |c_off|, plus a margin against rounding of positions of
-// O(100) m), a grid of BIN_DIM^2 cells centred on the vehicle.
-cudaError_t build_bins(RolloutArgs& a, float half_len, float half_wid, float c_off, void* workspace, cudaStream_t s)
+// the grids of geometry g into the workspace (fills a.bins)
+static cudaError_t build_grids(RolloutArgs& a, BinView g, void* workspace, cudaStream_t s)
 {
-    return build_bins_radius(a, std::sqrt((double)half_len * half_len + (double)half_wid * half_wid) +
-                                    std::fabs((double)c_off), workspace, s);
-}
-
-// grids for a footprint inside the disk of the given radius around the
-// reference point
-cudaError_t build_bins_radius(RolloutArgs& a, double radius, void* workspace, cudaStream_t s)
-{
-    BinView g = make_bin_grid_radius(radius);
     int* cell_start = static_cast<int*>(workspace);
     float2* binned = reinterpret_cast<float2*>(cell_start + (size_t)(a.T + 1) * BIN_CS_STRIDE);
     g.cell_start = cell_start;
@@ -170,9 +176,21 @@ cudaError_t build_bins_radius(RolloutArgs& a, double radius, void* workspace, cu
     return e;
 }
 
+cudaError_t build_bins(RolloutArgs& a, float half_len, float half_wid, float c_off, void* workspace, cudaStream_t s)
+{
+    return build_grids(a, make_bin_grid(half_len, half_wid, c_off), workspace, s);
+}
+
+cudaError_t build_bins_poly(RolloutArgs& a, double radius, const double box[4], void* workspace, cudaStream_t s)
+{
+    return build_grids(a, make_bin_grid_box(radius, box), workspace, s);
+}
+
 cudaError_t launch_collide_binned(const RolloutArgs& a, cudaStream_t s)
 {
-    collide_binned_kernel<<<(a.N + BINNED_WARPS - 1) / BINNED_WARPS, BINNED_WARPS * 32, 0, s>>>(a);
+    const int grid = (a.N + BINNED_WARPS - 1) / BINNED_WARPS;
+    if (a.poly.n_faces > 0) collide_binned_kernel<true><<<grid, BINNED_WARPS * 32, 0, s>>>(a);
+    else collide_binned_kernel<false><<<grid, BINNED_WARPS * 32, 0, s>>>(a);
     return cudaGetLastError();
 }
 

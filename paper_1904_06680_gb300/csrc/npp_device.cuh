@@ -353,7 +353,8 @@ constexpr int BIN_CS_STRIDE = BIN_NCELL + 4;    // 16-byte multiple: the float2 
 struct BinView {
     float x0;              // lower-left corner of the grid (EV frame, both axes)
     float inv_cell;
-    float reach;           // query radius
+    float reach;           // radius around the reference point that holds the vehicle, plus a margin
+    float cx, cy, hl, hw;  // a box that holds it too, in its own frame: centre, half extents plus the margin
     const int* cell_start; // null: no grids
     const float2* pts;
     int M;
@@ -378,13 +379,13 @@ __device__ __forceinline__ int bin_cell(float x, const BinView& g)
     return (int)fminf(fmaxf(f, 0.0f), (float)(BIN_DIM - 1));
 }
 
-// The candidate points of a query disk in one step's grid: the cells of the
-// (at most five) cell rows its bounding square overlaps, each row's cells
-// one contiguous run of the cell-sorted points.  Cells are at least half as
-// wide as the query radius, so the square spans at most five cells per axis;
-// indices are clamped monotonically at the grid border, so every point that
-// can lie in the disk is a candidate.
-constexpr int BIN_MAX_ROWS = 5;      // cell rows a query can span (cells >= half the query radius)
+// The candidate points of a query box (half extents rx, ry around (x, y), at
+// most the grid's reach) in one step's grid: the cells of the at most five
+// cell rows it overlaps, each row's cells one contiguous run of the
+// cell-sorted points.  Cells are at least half as wide as the reach, so the
+// box spans at most five cells per axis; indices are clamped monotonically at
+// the grid border, so every point that can lie in the box is a candidate.
+constexpr int BIN_MAX_ROWS = 5;      // cell rows a query can span (cells >= half the reach)
 struct CandRows {
     int b[BIN_MAX_ROWS];             // first sorted point of each row's run
     int e[BIN_MAX_ROWS];             // candidates before the end of each run (inclusive prefix)
@@ -400,11 +401,14 @@ struct CandRows {
     }
 };
 
-__device__ __forceinline__ CandRows cand_rows(const int* __restrict__ cs, const BinView& g, float x, float y,
-                                              float r)
+struct QueryBox {
+    float x, y, rx, ry;
+};
+
+__device__ __forceinline__ CandRows cand_rows(const int* __restrict__ cs, const BinView& g, const QueryBox& q)
 {
-    const int ix0 = bin_cell(x - r, g), ix1 = bin_cell(x + r, g);
-    const int iy0 = bin_cell(y - r, g), iy1 = bin_cell(y + r, g);
+    const int ix0 = bin_cell(q.x - q.rx, g), ix1 = bin_cell(q.x + q.rx, g);
+    const int iy0 = bin_cell(q.y - q.ry, g), iy1 = bin_cell(q.y + q.ry, g);
     CandRows c;
     int acc = 0;
 #pragma unroll
@@ -623,8 +627,10 @@ size_t binned_workspace_bytes(int max_T, int max_M);
 cudaError_t build_bins(RolloutArgs& a, float half_len, float half_wid, float c_off, void* workspace,
                        cudaStream_t s);          // fills a.bins
 cudaError_t launch_collide_binned(const RolloutArgs& a, cudaStream_t s);
-cudaError_t launch_collide_poly(const RolloutArgs& a, cudaStream_t s);
-cudaError_t build_bins_radius(RolloutArgs& a, double radius, void* workspace, cudaStream_t s);
+cudaError_t launch_collide_poly(const RolloutArgs& a, cudaStream_t s);     // every point (a.poly.brute)
+// grids for a general footprint inside the disk of the given radius around
+// the reference point and inside box (xmin, xmax, ymin, ymax) of its frame
+cudaError_t build_bins_poly(RolloutArgs& a, double radius, const double box[4], void* workspace, cudaStream_t s);
 cudaError_t launch_epilogue(const EpilogueArgs& e, cudaStream_t s);
 void set_global_error(const char* msg);
 

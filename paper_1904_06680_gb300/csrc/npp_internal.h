@@ -44,6 +44,7 @@ struct npp_handle {
     float4* d_fp;                        // [FP_MAX_FACES] general footprint faces
     int fp_faces;                        // 0: the rectangle of cfg
     double fp_radius;                    // footprint's largest vertex distance
+    double fp_box[4];                    // its box in the vehicle's frame: xmin, xmax, ymin, ymax
     unsigned* d_work;                    // persistent-kernel work counter
     int sm_count;
     int collide_variant;                 // -1 automatic, else a fixed collision-kernel variant

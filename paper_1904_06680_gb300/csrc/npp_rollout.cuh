@@ -528,9 +528,29 @@ __device__ __forceinline__ int discard_step(const int* vfirst, long long n, int 
     return (hv >= 0 && (fh < 0 || hv < fh)) ? hv : fh;
 }
 
+// The axis-aligned box around the vehicle at (x, y) with heading sine and
+// cosine (sp, cp): its own box (BinView) turned, with 1e-6 of the position
+// against rounding.  It holds every point that can be inside, like the disk
+// around the reference point, with fewer candidates: a 4.5 x 1.8 m rectangle
+// along an axis needs 4.6 x 1.9 m instead of the disk's 5 x 5 m square.
+// (Clamped to the reach, which is never less: make_bin_grid_box.)  Plan steps
+// on GB300, disk / box (us): course 175 / 172, 8192 x 41 states on 855 points
+// 61 / 60, polygons of two pieces (speed limits) 250 / 246 -- and 200 with
+// the box before each polygon test too.
+__device__ __forceinline__ QueryBox query_box(const BinView& g, float x, float y, float sp, float cp)
+{
+    const float m = 1e-6f * (fabsf(x) + fabsf(y));
+    QueryBox q;
+    q.x = fmaf(g.cx, cp, fmaf(-g.cy, sp, x));
+    q.y = fmaf(g.cx, sp, fmaf(g.cy, cp, y));
+    q.rx = fminf(fmaf(g.hl, fabsf(cp), fmaf(g.hw, fabsf(sp), m)), g.reach);
+    q.ry = fminf(fmaf(g.hl, fabsf(sp), fmaf(g.hw, fabsf(cp), m)), g.reach);
+    return q;
+}
+
 // One state of one sample against one step's grid, checked by an 8-lane
 // group of a warp (four such items per warp at a time): the candidates of
-// the at most five cell rows the state's disk overlaps, strided over the
+// the at most five cell rows the state's box overlaps, strided over the
 // group's lanes, each lane first issuing the loads of up to R candidates and
 // then testing them with the brute-force kernels' per-point test (the rest,
 // rarely any, one by one).  Every lane of the warp calls it (warp-wide
@@ -553,9 +573,11 @@ __device__ __forceinline__ bool binned_item_inside(const DevCfg& c, const BinVie
     constexpr int L = BIN_ITEM_LANES;
     float4 ca;
     float2 cb;
-    rows_of_state(c, z, ca, cb);
+    float sp, cp;
+    sincos_r(z.z, sp, cp);
+    coef_rows(c, z.x, z.y, sp, cp, ca, cb);
     CandRows cr = {};
-    if (ok) cr = cand_rows(g.cell_start + (size_t)h * BIN_CS_STRIDE, g, z.x, z.y, g.reach);
+    if (ok) cr = cand_rows(g.cell_start + (size_t)h * BIN_CS_STRIDE, g, query_box(g, z.x, z.y, sp, cp));
     const float2* pts = g.pts + (size_t)(ok ? h : 0) * g.M;
     const int total = cr.total;
     float2 pr[R];
@@ -594,15 +616,14 @@ __device__ __forceinline__ bool binned_item_inside(const DevCfg& c, const BinVie
 // 0.32 against 0.43 ms at the large workload (8 candidates per state), 0.077
 // against 0.078 ms on the course (25); inside the trajectory kernel's
 // window check it costs registers (spills) and is not used there.
-template <int RR>
+template <int RR, class Test>
 __device__ __forceinline__ bool binned_rows_inside(const BinView& g, const int* __restrict__ cs,
-                                                   const float2* __restrict__ pts, const float4& ca,
-                                                   const float2& cb, float qx, float qy, float reach, bool ok,
-                                                   int gl, unsigned& ntest)
+                                                   const float2* __restrict__ pts, const Test& test,
+                                                   const QueryBox& qb, bool ok, int gl, unsigned& ntest)
 {
     constexpr int L = BIN_ITEM_LANES;
     CandRows cr = {};
-    if (ok) cr = cand_rows(cs, g, qx, qy, reach);
+    if (ok) cr = cand_rows(cs, g, qb);
     int len[BIN_MAX_ROWS];
 #pragma unroll
     for (int r = 0; r < BIN_MAX_ROWS; ++r) len[r] = cr.e[r] - (r > 0 ? cr.e[r - 1] : 0);
@@ -621,7 +642,7 @@ __device__ __forceinline__ bool binned_rows_inside(const BinView& g, const int* 
 #pragma unroll
         for (int t = 0; t < RR; ++t)
             if (gl + t * L < len[r]) {
-                inside |= inside_rows(ca, cb, pr[r][t]);
+                inside |= test(pr[r][t]);
                 ++ntest;
             }
         rest = max(rest, len[r] - RR * L);
@@ -632,7 +653,7 @@ __device__ __forceinline__ bool binned_rows_inside(const BinView& g, const int* 
         for (int r = 0; r < BIN_MAX_ROWS; ++r) {
             const int k = RR * L + it * L + gl;
             if (k < len[r]) {
-                inside |= inside_rows(ca, cb, pts[cr.b[r] + k]);
+                inside |= test(pts[cr.b[r] + k]);
                 ++ntest;
             }
         }
@@ -640,18 +661,48 @@ __device__ __forceinline__ bool binned_rows_inside(const BinView& g, const int* 
     return inside;
 }
 
-// the row-wise item check of state z at step h of grid g (its rows
-// recomputed, the query disk around its reference point)
-template <int RR>
-__device__ __forceinline__ bool binned_item_inside_rows(const DevCfg& c, const BinView& g, const float4& z, int h,
-                                                        bool ok, int gl, unsigned& ntest)
+// the per-point tests: the rectangle by its scaled rows, the general footprint
+struct RectTest {
+    float4 a;
+    float2 b;
+    __device__ __forceinline__ bool operator()(float2 p) const { return inside_rows(a, b, p); }
+};
+
+// Whether point p (EV frame at the step's time) is inside the general
+// footprint at pose (x, y) with heading cosine and sine (cp, sp): p moved
+// into the vehicle's frame, q = R(-phi) (p - [x, y]), is inside a convex
+// piece when n . q < b holds strictly for all of its faces (Eq. of the
+// polytope check, Sect. II-D); the footprint is the union of its pieces.
+__device__ __forceinline__ bool poly_inside(const float4* faces, int n_faces, float r2, float2 p, float x,
+                                            float y, float cp, float sp)
 {
-    float4 ca;
-    float2 cb;
-    rows_of_state(c, z, ca, cb);
-    return binned_rows_inside<RR>(g, g.cell_start + (size_t)(ok ? h : 0) * BIN_CS_STRIDE,
-                                  g.pts + (size_t)(ok ? h : 0) * g.M, ca, cb, z.x, z.y, g.reach, ok, gl, ntest);
+    const float dx = p.x - x, dy = p.y - y;
+    const float qx = fmaf(cp, dx, __fmul_rn(sp, dy));
+    const float qy = fmaf(-sp, dx, __fmul_rn(cp, dy));
+    // outside the footprint's bounding disk (r2 is its squared radius,
+    // enlarged beyond any rounding of q): no face test needed
+    if (fmaf(qx, qx, __fmul_rn(qy, qy)) >= r2) return false;
+    bool any = false, in = true;
+    for (int f = 0; f < n_faces; ++f) {
+        const float4 F = faces[f];
+        in = in & (fmaf(F.x, qx, __fmul_rn(F.y, qy)) < F.z);
+        if (F.w != 0.0f) {
+            any = any | in;
+            in = true;
+        }
+    }
+    return any;
 }
+
+struct PolyTest {
+    const float4* faces;
+    int n_faces;
+    float r2, x, y, cp, sp;
+    __device__ __forceinline__ bool operator()(float2 p) const
+    {
+        return poly_inside(faces, n_faces, r2, p, x, y, cp, sp);
+    }
+};
 
 // ------------------------------------------------------------------ bins
 // The grid of one horizon step (time tau) built by one block of THREADS
@@ -712,21 +763,30 @@ __device__ __forceinline__ void build_step_bins(const float4* __restrict__ obs, 
     }
 }
 
-// A grid whose cell exceeds the diameter of the query disk: the rectangle's
-// circumradius plus |c_off|, plus a margin against rounding of positions of
-// O(100) m (host side).
-inline BinView make_bin_grid_radius(double R)
+// The grid's geometry for a vehicle inside the disk of radius R around its
+// reference point and inside box (xmin, xmax, ymin, ymax) of its frame (host
+// side).  The reach is R + 0.05 m (rounding of positions of O(100) m), cells a
+// little wider than half of it, so a query spans at most five cells per axis
+// (measured on GB300: cells half the reach beat cells one and two reaches
+// wide: they cover less area beyond the query).
+inline BinView make_bin_grid_box(double R, const double box[4])
 {
-    // query radius R + 0.05 (rounding of positions of O(100) m); cells a
-    // little wider than half of it, so a query spans at most five cells per
-    // axis (a query square of side 2r over cells of width c covers (2r + c)^2
-    // of candidates on average: 6.25 r^2 here against 16 r^2 for c = 2r;
-    // measured on GB300: c = r/2 beats c = r and c = 2r)
     const double cell = 0.5 * (R + 0.15);
     BinView g;
     g.inv_cell = (float)(1.0 / cell);
     g.x0 = (float)(-0.5 * BIN_DIM * cell);
     g.reach = (float)(R + 0.05);
+    const double hl = 0.5 * (box[1] - box[0]), hw = 0.5 * (box[3] - box[2]);
+    if (hl * hl + hw * hw <= R * R) {
+        g.cx = (float)(0.5 * (box[0] + box[1]));
+        g.cy = (float)(0.5 * (box[2] + box[3]));
+        g.hl = (float)(hl + 0.05);
+        g.hw = (float)(hw + 0.05);
+    } else {
+        // the turned box could exceed the reach: the disk's square instead
+        g.cx = g.cy = 0.0f;
+        g.hl = g.hw = g.reach;
+    }
     g.cell_start = nullptr;
     g.pts = nullptr;
     g.M = 0;
@@ -736,8 +796,9 @@ inline BinView make_bin_grid_radius(double R)
 // the rectangle lies in the disk of its circumradius plus |c_off|
 inline BinView make_bin_grid(float half_len, float half_wid, float c_off)
 {
-    return make_bin_grid_radius(std::sqrt((double)half_len * half_len + (double)half_wid * half_wid) +
-                                std::fabs((double)c_off));
+    const double box[4] = { (double)c_off - half_len, (double)c_off + half_len, -(double)half_wid, (double)half_wid };
+    return make_bin_grid_box(std::sqrt((double)half_len * half_len + (double)half_wid * half_wid) +
+                                 std::fabs((double)c_off), box);
 }
 
 // ------------------------------------------------------------------ traj
