@@ -277,9 +277,12 @@ npp_status run_rollout(npp_handle* h, RolloutArgs& a, cudaStream_t s, bool no_re
         a.poly.faces = h->d_fp;
         a.poly.n_faces = h->fp_faces;
         a.poly.brute = (h->collide_variant >= 0 && h->collide_variant < COLLIDE_BINNED) ? 1 : 0;
-        // enlarged by 1e-3 relative and 1e-6 m^2: larger than any rounding of
-        // a point's squared distance, so no inside point is skipped
-        a.poly.r2 = (float)(h->fp_radius * h->fp_radius * 1.001 + 1e-6);
+        // enlarged by 0.05 m, larger than any rounding of a point's position
+        // in the vehicle's frame, so no inside point is skipped
+        a.poly.cx = (float)(0.5 * (h->fp_box[0] + h->fp_box[1]));
+        a.poly.cy = (float)(0.5 * (h->fp_box[2] + h->fp_box[3]));
+        a.poly.hl = (float)(0.5 * (h->fp_box[1] - h->fp_box[0]) + 0.05);
+        a.poly.hw = (float)(0.5 * (h->fp_box[3] - h->fp_box[2]) + 0.05);
         if (h->timing) CUDA_TRY(h, record_event(h->ev[0], s));
         CUDA_TRY(h, cudaEventRecord(h->fork_ev, s));
         CUDA_TRY(h, cudaStreamWaitEvent(h->side, h->fork_ev, 0));

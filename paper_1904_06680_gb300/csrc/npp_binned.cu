@@ -95,7 +95,7 @@ __global__ void __launch_bounds__(BINNED_WARPS * 32, 5) collide_binned_kernel(co
             const QueryBox qb = query_box(g, z.x, z.y, sp, cp);
             bool inside;
             if constexpr (POLY) {
-                const PolyTest test = { faces, a.poly.n_faces, a.poly.r2, z.x, z.y, cp, sp };
+                const PolyTest test = { a.poly, faces, z.x, z.y, cp, sp };
                 inside = binned_rows_inside<1>(g, cs, pts, test, qb, ok, gl, ntest);
             } else {
                 RectTest test;

@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(POLY_WARPS * 32) collide_poly_kernel(const Rol
                 const int k = base + lane;
                 bool inside = false;
                 if (k < M)
-                    inside = poly_inside(faces, nf, a.poly.r2, pts[k], z.x, z.y, cp, sp);
+                    inside = poly_inside(a.poly, faces, pts[k], z.x, z.y, cp, sp);
                 hit = __any_sync(FULL, inside);
             }
             if (hit) { fh = h; break; }

@@ -673,18 +673,19 @@ struct RectTest {
 // into the vehicle's frame, q = R(-phi) (p - [x, y]), is inside a convex
 // piece when n . q < b holds strictly for all of its faces (Eq. of the
 // polytope check, Sect. II-D); the footprint is the union of its pieces.
-__device__ __forceinline__ bool poly_inside(const float4* faces, int n_faces, float r2, float2 p, float x,
-                                            float y, float cp, float sp)
+// Most candidates fail the footprint's box (enlarged beyond any rounding of
+// q) and need no face: a box turned with the vehicle passes a third of the
+// points that the footprint's disk would.
+__device__ __forceinline__ bool poly_inside(const PolyView& f, const float4* faces, float2 p, float x, float y, float cp,
+                                            float sp)
 {
     const float dx = p.x - x, dy = p.y - y;
     const float qx = fmaf(cp, dx, __fmul_rn(sp, dy));
     const float qy = fmaf(-sp, dx, __fmul_rn(cp, dy));
-    // outside the footprint's bounding disk (r2 is its squared radius,
-    // enlarged beyond any rounding of q): no face test needed
-    if (fmaf(qx, qx, __fmul_rn(qy, qy)) >= r2) return false;
+    if (!(fabsf(qx - f.cx) <= f.hl && fabsf(qy - f.cy) <= f.hw)) return false;
     bool any = false, in = true;
-    for (int f = 0; f < n_faces; ++f) {
-        const float4 F = faces[f];
+    for (int k = 0; k < f.n_faces; ++k) {
+        const float4 F = faces[k];
         in = in & (fmaf(F.x, qx, __fmul_rn(F.y, qy)) < F.z);
         if (F.w != 0.0f) {
             any = any | in;
@@ -693,15 +694,11 @@ __device__ __forceinline__ bool poly_inside(const float4* faces, int n_faces, fl
     }
     return any;
 }
-
 struct PolyTest {
+    const PolyView& f;
     const float4* faces;
-    int n_faces;
-    float r2, x, y, cp, sp;
-    __device__ __forceinline__ bool operator()(float2 p) const
-    {
-        return poly_inside(faces, n_faces, r2, p, x, y, cp, sp);
-    }
+    float x, y, cp, sp;
+    __device__ __forceinline__ bool operator()(float2 p) const { return poly_inside(f, faces, p, x, y, cp, sp); }
 };
 
 // ------------------------------------------------------------------ bins
