@@ -839,8 +839,10 @@ def run_batch(args):
                                      "slices": choice[1], "traj_warps": choice[2]},
                        "l2": "flushed (256 MiB write) between replays"},
             "roofline": roof,
-            # prologue, grids (binned), one trajectory kernel per width, check, epilogue
-            "gpu_launches": (1 + (1 if binned else 0) + n_widths + 1 + 1) * K, "clocks": ck,
+            # grids (binned) or tile order, one trajectory kernel per width, a check per width that does
+            # not check as it rolls out (binned, below 64) or one for all (brute force), epilogue
+            "gpu_launches": (1 + n_widths + (sum(1 for w in set(x["width"] for x in sc) if w < 64) if binned else 1)
+                             + 1) * K, "clocks": ck,
             "cpu_baseline": None if (args.no_cpu_baseline or rank != 0) else batch_cpu_baseline(bt),
             "free_fraction": float(np.mean(fhs < 0)),
             "infeasible_scenes": int((best.cpu().view(S, 8)[:, 1] == 2).sum())}

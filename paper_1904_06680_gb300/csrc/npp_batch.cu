@@ -1,10 +1,14 @@
 // npp_batch.cu -- many independent plan steps (scenes of different N, T, M
 // and network width) in one batch of persistent launches:
-//   prologue      every scene's obstacle points into its EV frame, as pairs;
-//   trajectories  one persistent launch per network width, blocks pulling
-//                 (scene, sample block) items, costliest scenes first;
-//   collisions    one persistent launch over all scenes, blocks of S warps
-//                 pulling (scene, 8-sample) items; a scene's points are
+//   points        every scene's per-step grids (binned check), or its points
+//                 moved into the EV frame as pairs (brute force);
+//   trajectories  one persistent launch per network width, on streams of
+//                 their own so that one width's tail overlaps the next's
+//                 start, warps pulling items of a warp's samples, costliest
+//                 scenes first; width-64 scenes are checked in there (binned);
+//   collisions    binned: a launch per width after its trajectories; brute
+//                 force: one persistent launch over all scenes, blocks of S
+//                 warps pulling (scene, 8-sample) items, a scene's points
 //                 staged in shared memory while the block works on it (read
 //                 from global memory when they do not fit);
 //   epilogue      one block per scene: decode the winner, re-roll it for
@@ -32,7 +36,7 @@ struct SceneDev {
     int N, T, M, width;
     long long obs_off;       // first input point
     long long pair_off;      // first transformed pair
-    long long coef_off;      // first coefficient row
+    long long state_off;     // first stored state
     long long samp_off;      // first sample (costs, first_hit, jfree)
     long long params_off, ctrl_off, traj_off;
     long long tile_off;      // first point tile (32 pairs)
@@ -51,14 +55,12 @@ struct BatchArgs {
     float4* tileP;                   // per tile of 32 pairs: (min x, max x, min y, max y) of its points
     float4* tileV;                   // (min vx, max vx, min vy, max vy)
     float reach;                     // radius around a rectangle's centre that holds it, plus a margin
-    int windowed64;                  // width-64 scenes checked inside their trajectory kernel
     // binned collision check (per scene and horizon step)
     BinView grid;                    // geometry (cell_start, pts, M unused here)
     int* bin_cs;                     // cell tables, scene s at bin_off
     float2* bin_pts;                 // sorted points, scene s at bpts_off
     const long long* bstep_prefix;   // prefix over scenes of T + 1 (grid-build blocks)
-    float4* coefA;
-    float2* coefB;
+    float4* states;                  // [T + 1][N] per scene, EV frame
     float* jfree;
     int* vfirst;                     // first speed-violating step per sample, or null (limits off)
     unsigned long long* keys;        // [S]
@@ -69,6 +71,7 @@ struct BatchArgs {
     const int* torder[3];            // per width: scenes of that width by decreasing cost
     int n_torder[3];
     const long long* citem_prefix;   // prefix of 8-sample items over `order`
+    const long long* witem_prefix[3];  // per width: prefix of 8-sample items over torder
     int resident_pairs;              // pairs that fit in shared memory
     // outputs
     npp_best* best;
@@ -315,36 +318,45 @@ __device__ __forceinline__ float4 live_box(const DevCfg& c, float4 ca, float2 cb
                        __shfl_sync(FULL, ymx, 0));
 }
 
-// KSQ > 0: the last KSQ layer-2 input quads of each lane in shared memory
-// (as the single-scene width-64 kernel: 128 registers and MINB blocks per
-// SM instead of every weight in registers at 250)
-// WIN: the scene's binned check done window by window inside the kernel
+// Trajectories of the scenes of one width: the warps of a resident grid take
+// items of 32 / G consecutive samples of a scene (layer-2 weights in tensor
+// memory, as traj_tmem_kernel and fused_tmem_kernel), so no warp waits for
+// another.  WIN: the scene's binned check done window by window inside
 // (traj_sample_windowed, windows of BATCH_CW states, the scene's grids built
-// before the launch): each sample's cost, first collision and the scene's
-// key are written here, nothing per step is stored
+// before the launch): each sample's cost, first collision and the scene's key
+// are written here, nothing per step is stored.
+// Bound: issue slots and the chain of a step.  48 scenes of all widths on
+// GB300: 12.0 ms with a block per group of samples (which waits for its
+// slowest), weights in registers and the widths one after another, 8.7 with
+// queues of warps, weights in tensor memory and the widths side by side.
 constexpr int BATCH_CW = 8;
-template <int W, int G, int NW, bool VAR = false, int KSQ = 0, int MINB = 1, bool WIN = false>
+template <int W, int G, int NW, int MINB, bool VAR, int KT, int KS, bool WIN>
 __global__ void __launch_bounds__(NW * 32, MINB) batch_traj_kernel(const BatchArgs b, int wi)
 {
-    constexpr int B = TrajKernel<W, G, NW>::B;
-    __shared__ __align__(16) float hx_all[B * W];
-    __shared__ long long qslot;
-    // [LaneNet::SLOTS][NW * 32] floats when W == 32 (KSQ = 0); the shared W2
-    // quads [group][U][KSQ][G] of 16 bytes when KSQ > 0
-    extern __shared__ __align__(16) float stage_all[];
-    const int tid = threadIdx.x;
-    const int bi = tid / G, gl = tid % G;
+    using Net = TmemNet<W, G, KT, KS>;
+    static_assert(NW % 4 == 0 && tmem_cols<Net, NW>() * MINB <= 512, "the blocks of an SM fit its TMEM");
+    extern __shared__ __align__(16) ulonglong2 w2_all[];
+    __shared__ uint32_t tslot;
+    constexpr int NG = 32 / G, CW = WIN ? BATCH_CW : 0;
+    float4* wnd_all = reinterpret_cast<float4*>(w2_all + NW * 32 * Net::U * KS);
+    float* hx_all = reinterpret_cast<float*>(wnd_all + NW * NG * CW);
+    const int tid = threadIdx.x, bi = tid / G, gl = tid % G, warp = tid >> 5, lane = tid & 31;
+    const uint32_t tmem = tmem_alloc<tmem_cols<Net, NW>()>(&tslot);
+    Net net;
+    net.tm = tmem + ((uint32_t)(warp & 3) << 21) + (uint32_t)((warp >> 2) * Net::COLS);
+    net.w2s = w2_all + (size_t)bi * (Net::U * KS * G) + gl;
     const int n_sc = b.n_torder[wi];
-    const long long total = n_sc > 0 ? __ldg(b.titem_prefix[wi] + n_sc) : 0;
+    const long long total = __ldg(b.titem_prefix[wi] + n_sc);
     for (;;) {
-        __syncthreads();
-        if (tid == 0) qslot = (long long)atomicAdd(b.counters + wi, 1u);
-        __syncthreads();
-        const long long item = qslot;
-        if (item >= total) break;
+        unsigned item = 0;
+        if (lane == 0) item = atomicAdd(b.counters + wi, 1u);
+        item = __shfl_sync(FULL, item, 0);
+        if ((long long)item >= total) break;
         const int r = find_slot(b.titem_prefix[wi], n_sc, item);
-        const SceneDev& s = b.scenes[b.torder[wi][r]];
-        const int n = (int)(item - __ldg(b.titem_prefix[wi] + r)) * B + bi;
+        const int si = b.torder[wi][r];
+        const SceneDev& s = b.scenes[si];
+        const int n = (int)((long long)item - __ldg(b.titem_prefix[wi] + r)) * NG + lane / G;
+        const bool valid = n < s.N;
         TrajJob job;
         job.si = scene_step_in(s);
         job.key.k0 = s.k0; job.key.k1 = s.k1; job.key.t_index = s.t_index; job.key.stream_id = 0u;
@@ -352,42 +364,29 @@ __global__ void __launch_bounds__(NW * 32, MINB) batch_traj_kernel(const BatchAr
         job.warm = nullptr;
         job.prop = Proposal{ nullptr, nullptr, 0, 1u };
         job.bins = nullptr;
-        job.stage = stage_all + tid;
+        job.stage = nullptr;
         job.w2s = nullptr;
-        if constexpr (KSQ > 0)
-            job.w2s = reinterpret_cast<ulonglong2*>(stage_all) + (size_t)bi * (Shape<W, G>::U * KSQ * G) + gl;
         job.N = s.N;
         job.T = s.T;
-        job.traj = nullptr;
+        job.traj = WIN ? nullptr : b.states + s.state_off;
         job.ctrl = nullptr;
-        job.rec_stride = 0;
+        job.rec_stride = s.N;
         job.rec_shift = 0;
-        job.coefA = b.coefA;
-        job.coefB = b.coefB;
-        job.coef_base = s.coef_off;
-        job.jfree = b.jfree + s.samp_off;
-        job.vfirst = b.vfirst ? b.vfirst + s.samp_off : nullptr;
-        constexpr int STAGE_TH = (W == 32 && KSQ == 0) ? NW * 32 : 0;     // as traj_kernel
+        job.coefA = nullptr;
+        job.coefB = nullptr;
+        job.coef_base = 0;
+        job.jfree = WIN ? nullptr : b.jfree + s.samp_off;
+        job.vfirst = !WIN && b.vfirst ? b.vfirst + s.samp_off : nullptr;
+        net.load(theta_src<Net::S::NT>(job, n, valid), gl);
         if constexpr (WIN) {
-            const int si = b.torder[wi][r];
             BinView bv = b.grid;
             bv.cell_start = b.bin_cs + s.bin_off;
             bv.pts = b.bin_pts + s.bpts_off;
             bv.M = s.M;
             job.bins = &bv;
-            job.coefA = nullptr;
-            job.coefB = nullptr;
-            job.jfree = nullptr;
-            job.vfirst = nullptr;
-            float4* wnd = reinterpret_cast<float4*>(reinterpret_cast<char*>(stage_all) +
-                                                    NW * 32 * Shape<W, G>::U * KSQ * 16) +
-                          (size_t)(tid / 32) * (32 / G) * BATCH_CW;
             unsigned steps = 0, ntest = 0, nstate = 0;
-            const bool valid = n < s.N;
-            LaneNet<W, G, KSQ> net;
-            load_net<STAGE_TH>(net, job, n, valid, gl);
-            const FusedOut o = traj_sample_windowed<VAR, BATCH_CW, 4>(
-                b.c, job, net, n, valid, gl, hx_all + bi * W, wnd, steps, ntest, nstate);
+            const FusedOut o = traj_sample_windowed<VAR, BATCH_CW, 4>(b.c, job, net, n, valid, gl, hx_all + bi * W,
+                                                                      wnd_all + warp * NG * CW, steps, ntest, nstate);
             if (valid && gl == 0) {
                 unsigned long long key;
                 if (o.first_hit < 0)
@@ -399,11 +398,10 @@ __global__ void __launch_bounds__(NW * 32, MINB) batch_traj_kernel(const BatchAr
                 if (key < *reinterpret_cast<volatile unsigned long long*>(b.keys + si)) atomicMin(b.keys + si, key);
             }
         } else {
-            LaneNet<W, G, KSQ> net;
-            load_net<STAGE_TH>(net, job, n, n < s.N, gl);
-            traj_sample<VAR>(b.c, job, net, n, n < s.N, gl, hx_all + bi * W);
+            traj_sample<VAR>(b.c, job, net, n, valid, gl, hx_all + bi * W);
         }
     }
+    tmem_free<tmem_cols<Net, NW>()>(tmem);
 }
 
 template <int S>
@@ -461,17 +459,13 @@ __global__ void __launch_bounds__(S * 32) batch_collide_kernel(const BatchArgs b
         const int n = n0 + lane;
         const bool mine = lane < cnt;
         unsigned live = (1u << cnt) - 1u;
-        float4 ca = make_float4(0.f, 0.f, 0.f, 0.f);
-        float2 cb = make_float2(0.f, 0.f);
-        if (mine) { ca = b.coefA[s.coef_off + n]; cb = b.coefB[s.coef_off + n]; }
+        float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (mine) z = b.states[s.state_off + n];
         for (int h = 0; h <= T; ++h) {
-            const float4 cur_a = ca;
-            const float2 cur_b = cb;
-            if (mine && h < T) {
-                const long long idx = s.coef_off + (long long)(h + 1) * N + n;
-                ca = b.coefA[idx];
-                cb = b.coefB[idx];
-            }
+            float4 cur_a;
+            float2 cur_b;
+            rows_of_state(b.c, z, cur_a, cur_b);
+            if (mine && h < T) z = b.states[s.state_off + (long long)(h + 1) * N + n];
             const unsigned gone = __ballot_sync(FULL, lane < 8 && *(volatile int*)&dead_at[lane] <= h);
             live &= ~gone;
             if (live == 0u || ntiles <= warp) break;
@@ -523,52 +517,40 @@ __global__ void __launch_bounds__(1024) batch_bin_build_kernel(const BatchArgs b
                           cnt, run_tot);
 }
 
-// Binned check of an 8-sample item per block, one warp per sample, over the
-// stored inequality rows: four steps at once, eight lanes per step, each
-// cell row's run of candidates taken directly (binned_rows_inside, as the
-// single-scene check); the query disk around the rectangle's centre
-// recovered from its rows (as in live_box).  The chunk's first colliding
-// step ends the sample; one key minimum per block.
-__global__ void __launch_bounds__(256) batch_binned_kernel(const BatchArgs b)
+// Binned check of the scenes of one width, an 8-sample item per block, one
+// warp per sample over its stored states: four steps at once, eight lanes per
+// step, each cell row's run of candidates taken directly (as
+// collide_binned_kernel).  The chunk's first colliding step ends the sample;
+// one key minimum per block.
+__global__ void __launch_bounds__(256) batch_binned_kernel(const BatchArgs b, int wi)
 {
     __shared__ unsigned long long red[8];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int gid = lane / BIN_ITEM_LANES, gl = lane % BIN_ITEM_LANES;
     constexpr int SB = 32 / BIN_ITEM_LANES;            // steps per chunk
     const long long item = blockIdx.x;
-    const int r = find_slot(b.citem_prefix, b.S, item);
-    const int si = b.order[r];
+    const int r = find_slot(b.witem_prefix[wi], b.n_torder[wi], item);
+    const int si = b.torder[wi][r];
     const SceneDev& s = b.scenes[si];
-    if (b.windowed64 && s.width == 64) return;       // checked inside the trajectory kernel (block-uniform)
     const int T = s.T, N = s.N, M = s.M;
-    const int n = (int)(item - __ldg(b.citem_prefix + r)) * 8 + warp;
+    const int n = (int)(item - __ldg(b.witem_prefix[wi] + r)) * 8 + warp;
     const BinView& g = b.grid;
-    const float isl = 1.0f / (2.0f * b.c.ihl), isw = 1.0f / (2.0f * b.c.ihw);
     unsigned long long key = ~0ull;
     if (n < N) {
         int fh = -1;
         for (int h0 = 0; h0 <= T; h0 += SB) {
             const int h = h0 + gid;
             const bool ok = h <= T;
-            float4 ca = make_float4(0.f, 0.f, 0.f, 0.f);
-            float2 cb = make_float2(0.f, 0.f);
-            if (ok) {
-                const long long idx = s.coef_off + (long long)h * N + n;
-                ca = b.coefA[idx];
-                cb = b.coefB[idx];
-            }
-            const float cp = ca.x * isl, sp = ca.y * isl;
-            const float along = -ca.z * isl, across = -cb.y * isw;
-            const float xc = cp * along - sp * across, yc = sp * along + cp * across;
-            // the box around the rectangle at its recovered centre (the
-            // margin far above the rounding of this reconstruction)
-            const float rx = fmaf(g.hl, fabsf(cp), fmaf(g.hw, fabsf(sp), 0.05f));
-            const float ry = fmaf(g.hl, fabsf(sp), fmaf(g.hw, fabsf(cp), 0.05f));
             const int hq = ok ? h : 0;
+            const float4 z = ok ? b.states[s.state_off + (long long)h * N + n] : make_float4(0.f, 0.f, 0.f, 0.f);
+            float sp, cp;
+            sincos_r(z.z, sp, cp);
+            RectTest test;
+            coef_rows(b.c, z.x, z.y, sp, cp, test.a, test.b);
             unsigned ntest = 0;
             const bool inside = binned_rows_inside<1>(g, b.bin_cs + s.bin_off + (size_t)hq * BIN_CS_STRIDE,
-                                                      b.bin_pts + s.bpts_off + (size_t)hq * M, RectTest{ ca, cb },
-                                                      QueryBox{ xc, yc, fminf(rx, g.reach), fminf(ry, g.reach) }, ok, gl, ntest);
+                                                      b.bin_pts + s.bpts_off + (size_t)hq * M, test,
+                                                      query_box(g, z.x, z.y, sp, cp), ok, gl, ntest);
             const unsigned bal = __ballot_sync(FULL, inside);
             unsigned steps_hit = 0;
 #pragma unroll
@@ -597,7 +579,7 @@ __global__ void __launch_bounds__(256) batch_binned_kernel(const BatchArgs b)
     if (threadIdx.x == 0) {
         unsigned long long k = red[0];
         for (int w = 1; w < 8; ++w) k = red[w] < k ? red[w] : k;
-        atomicMin(b.keys + si, k);
+        if (k < *reinterpret_cast<volatile unsigned long long*>(b.keys + si)) atomicMin(b.keys + si, k);
     }
 }
 
@@ -720,10 +702,12 @@ struct npp_batch {
     float2* d_bin_pts;
     long long* d_bstep_prefix;
     long long bin_blocks;    // sum over scenes of T + 1
-    long long total_items;   // sum over scenes of ceil(N / 8)
+    long long* d_witem_prefix[3];
+    long long witems[3];     // per width: sum over its scenes of ceil(N / 8)
+    cudaStream_t side[2];    // the smaller widths' trajectories and checks
+    cudaEvent_t fork, join[2];
     int binned;              // collision check: 0 brute force (tile-culled), 1 per-step bins
-    float4* d_coefA;
-    float2* d_coefB;
+    float4* d_states;
     float* d_jfree;
     int* d_vfirst;           // [samples] when the handle's speed limits are on
     unsigned long long* d_keys;
@@ -731,9 +715,9 @@ struct npp_batch {
     int resident_pairs;
     int max_pairs;
     long long total_pairs, total_rows, total_samples;
-    int grid_traj[3], grid_collide;
+    int grid_collide;
     int slices;              // warps per collision item (point slices): 2, 4, 8
-    int traj_warps;          // warps per trajectory block: 4, 8
+    int traj_warps;          // warps per trajectory block: 4, 8 (20 at width 64 with its check)
     int smem_optin;
 };
 
@@ -747,8 +731,14 @@ void free_batch(npp_batch* B)
     void* ptrs[] = { B->d_scenes, B->d_order, B->d_citem_prefix, B->d_torder[0], B->d_torder[1],
                      B->d_torder[2], B->d_titem_prefix[0], B->d_titem_prefix[1], B->d_titem_prefix[2],
                      B->d_pXY, B->d_pV, B->d_tileP, B->d_tileV, B->d_bin_cs, B->d_bin_pts, B->d_bstep_prefix,
-                     B->d_coefA, B->d_coefB, B->d_jfree, B->d_vfirst, B->d_keys, B->d_counters };
+                     B->d_witem_prefix[0], B->d_witem_prefix[1], B->d_witem_prefix[2],
+                     B->d_states, B->d_jfree, B->d_vfirst, B->d_keys, B->d_counters };
     for (void* p : ptrs) if (p) cudaFree(p);
+    for (int i = 0; i < 2; ++i) {
+        if (B->side[i]) cudaStreamDestroy(B->side[i]);
+        if (B->join[i]) cudaEventDestroy(B->join[i]);
+    }
+    if (B->fork) cudaEventDestroy(B->fork);
     delete B;
 }
 
@@ -771,7 +761,7 @@ npp_status upload_scenes(npp_batch* B)
         d.bin_off = bcs; bcs += (long long)(s.T + 1) * BIN_CS_STRIDE;
         d.bpts_off = bpts; bpts += (long long)(s.T + 1) * s.M;
         bstep[i + 1] = bstep[i] + s.T + 1;
-        d.coef_off = rows; rows += (long long)s.N * (s.T + 1);
+        d.state_off = rows; rows += (long long)s.N * (s.T + 1);
         d.samp_off = samp; samp += s.N;
         d.params_off = par; par += n_theta_w(s.width);
         d.ctrl_off = ctl; ctl += s.T;
@@ -801,36 +791,9 @@ cudaError_t collide_grid(npp_batch* B, int* grid)
     return e;
 }
 
-template <int W, int G>
-constexpr int batch_stage_bytes(int nw) { return W == 32 ? LaneNet<W, G>::SLOTS * nw * 32 * (int)sizeof(float) : 0; }
-
-// width 64: 8 of 16 layer-2 input quads per lane in shared memory, 16 warps
-// per SM (the single-scene default; 250 registers and 8 warps per SM with
-// every weight in registers)
-constexpr int BATCH_KSQ64 = 8;
-constexpr int batch_w2s_bytes64(int nw) { return nw * 32 * 2 * BATCH_KSQ64 * 16; }
-// with the windowed check: the W2 quads of 12 inputs per lane in shared
-// memory (registers for the check, as the single-scene kernel) and the
-// warps' windows of states
-constexpr int BATCH_KSQ64W = 12;
-constexpr int batch_w64w_bytes(int nw) { return nw * 32 * 2 * BATCH_KSQ64W * 16 + nw * BATCH_CW * 16; }
-
-template <int NW>
-void traj_grids(npp_batch* B)
-{
-    int nt = 0;
-    const int s16 = batch_stage_bytes<16, 8>(NW), s32 = batch_stage_bytes<32, 16>(NW);
-    ensure_smem(batch_traj_kernel<16, 8, NW>, s16);
-    ensure_smem(batch_traj_kernel<32, 16, NW, false, 0, 16 / NW>, s32);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nt, batch_traj_kernel<16, 8, NW>, NW * 32, s16);
-    B->grid_traj[0] = B->h->sm_count * std::max(1, nt);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nt, batch_traj_kernel<32, 16, NW, false, 0, 16 / NW>, NW * 32, s32);
-    B->grid_traj[1] = B->h->sm_count * std::max(1, nt);
-    auto k64 = batch_traj_kernel<64, 32, NW, false, BATCH_KSQ64, 16 / NW>;
-    ensure_smem(k64, batch_w2s_bytes64(NW));
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nt, k64, NW * 32, batch_w2s_bytes64(NW));
-    B->grid_traj[2] = B->h->sm_count * std::max(1, nt);
-}
+// samples a warp takes at once, by width (and, at width 64, by whether its
+// check runs inside)
+int item_samples(const npp_batch* B, int wi) { return wi == 0 ? 8 : wi == 1 ? 4 : B->binned ? 1 : 2; }
 
 // work order (costliest scenes first), item prefixes for the current block
 // shapes, persistent grids
@@ -849,13 +812,17 @@ npp_status plan_work(npp_batch* B)
     CUDA_TRY(h, cudaMemcpy(B->d_citem_prefix, cpre.data(), sizeof(long long) * (S + 1), cudaMemcpyHostToDevice));
     const int widths[3] = { 16, 32, 64 };
     for (int w = 0; w < 3; ++w) {
-        const int Bsz = B->traj_warps * 32 / (widths[w] / 2);
+        const int Bsz = item_samples(B, w);
         std::vector<int> v;
         for (int r = 0; r < S; ++r) if (sc[order[r]].width == widths[w]) v.push_back(order[r]);
         std::stable_sort(v.begin(), v.end(), [&](int a, int b) {
             return (double)sc[a].N * sc[a].T > (double)sc[b].N * sc[b].T; });
         std::vector<long long> pre(v.size() + 1, 0);
         for (size_t r = 0; r < v.size(); ++r) pre[r + 1] = pre[r] + (sc[v[r]].N + Bsz - 1) / Bsz;
+        std::vector<long long> wpre(v.size() + 1, 0);
+        for (size_t r = 0; r < v.size(); ++r) wpre[r + 1] = wpre[r] + (sc[v[r]].N + 7) / 8;
+        B->witems[w] = wpre[v.size()];
+        CUDA_TRY(h, cudaMemcpy(B->d_witem_prefix[w], wpre.data(), sizeof(long long) * wpre.size(), cudaMemcpyHostToDevice));
         B->n_torder[w] = (int)v.size();
         if (!v.empty()) CUDA_TRY(h, cudaMemcpy(B->d_torder[w], v.data(), sizeof(int) * v.size(), cudaMemcpyHostToDevice));
         CUDA_TRY(h, cudaMemcpy(B->d_titem_prefix[w], pre.data(), sizeof(long long) * pre.size(), cudaMemcpyHostToDevice));
@@ -867,7 +834,6 @@ npp_status plan_work(npp_batch* B)
     default: e = collide_grid<4>(B, &B->grid_collide); break;
     }
     if (e != cudaSuccess) return fail(h, NPP_CUDA_ERROR, "batch collision set-up: %s", cudaGetErrorString(e));
-    if (B->traj_warps == 4) traj_grids<4>(B); else traj_grids<8>(B);
     return NPP_OK;
 }
 
@@ -878,34 +844,38 @@ void launch_batch_collide(npp_batch* B, const BatchArgs& b, cudaStream_t s)
     batch_collide_kernel<S><<<B->grid_collide, BatchCollide<S>::THREADS, smem, s>>>(b);
 }
 
-template <int NW, bool VAR>
-void launch_batch_traj_v(npp_batch* B, const BatchArgs& b, cudaStream_t s)
+template <int W, int G, int NW, int MINB, bool VAR, int KT, int KS, bool WIN>
+cudaError_t launch_traj_items(npp_batch* B, const BatchArgs& b, int wi, cudaStream_t s)
 {
-    if (B->n_torder[0]) {
-        ensure_smem(batch_traj_kernel<16, 8, NW, VAR>, batch_stage_bytes<16, 8>(NW));
-        batch_traj_kernel<16, 8, NW, VAR><<<B->grid_traj[0], NW * 32, batch_stage_bytes<16, 8>(NW), s>>>(b, 0);
-    }
-    if (B->n_torder[1]) {
-        ensure_smem(batch_traj_kernel<32, 16, NW, VAR, 0, 16 / NW>, batch_stage_bytes<32, 16>(NW));
-        batch_traj_kernel<32, 16, NW, VAR, 0, 16 / NW><<<B->grid_traj[1], NW * 32, batch_stage_bytes<32, 16>(NW), s>>>(b, 1);
-    }
-    if (B->n_torder[2] && b.windowed64) {
-        auto k64 = batch_traj_kernel<64, 32, NW, VAR, BATCH_KSQ64W, 16 / NW, true>;
-        ensure_smem(k64, batch_w64w_bytes(NW));
-        k64<<<B->grid_traj[2], NW * 32, batch_w64w_bytes(NW), s>>>(b, 2);
-    } else if (B->n_torder[2]) {
-        auto k64 = batch_traj_kernel<64, 32, NW, VAR, BATCH_KSQ64, 16 / NW>;
-        ensure_smem(k64, batch_w2s_bytes64(NW));
-        k64<<<B->grid_traj[2], NW * 32, batch_w2s_bytes64(NW), s>>>(b, 2);
+    auto fn = batch_traj_kernel<W, G, NW, MINB, VAR, KT, KS, WIN>;
+    constexpr int smem = tmem_block_bytes<W, G, NW, KS, WIN ? BATCH_CW : 0>();
+    cudaError_t e = ensure_smem(fn, smem);
+    if (e != cudaSuccess) return e;
+    fn<<<MINB * B->h->sm_count, NW * 32, smem, s>>>(b, wi);
+    return cudaGetLastError();
+}
+
+// the launch shapes of the single-scene kernels, in blocks of NW warps
+template <int NW, bool VAR>
+cudaError_t launch_batch_traj_w(npp_batch* B, const BatchArgs& b, int wi, cudaStream_t s)
+{
+    switch (wi) {
+    case 0: return launch_traj_items<16, 4, NW, 16 / NW, VAR, 4, 0, false>(B, b, 0, s);
+    case 1: return launch_traj_items<32, 8, NW, 16 / NW, VAR, 8, 0, false>(B, b, 1, s);
+    default:
+        if (!B->binned) return launch_traj_items<64, 16, 4, 3, VAR, 8, 8, false>(B, b, 2, s);
+        if (NW == 4) return launch_traj_items<64, 32, 4, 4, VAR, 16, 0, true>(B, b, 2, s);
+        return launch_traj_items<64, 32, 20, 1, VAR, 12, 4, true>(B, b, 2, s);
     }
 }
 
 // rollout variants (body-frame features, speed limits) in their own kernels
-template <int NW>
-void launch_batch_traj(npp_batch* B, const BatchArgs& b, cudaStream_t s)
+cudaError_t launch_batch_traj(npp_batch* B, const BatchArgs& b, int wi, cudaStream_t s)
 {
-    if (uses_variants(b.c)) launch_batch_traj_v<NW, true>(B, b, s);
-    else launch_batch_traj_v<NW, false>(B, b, s);
+    const bool var = uses_variants(b.c);
+    if (B->traj_warps == 4)
+        return var ? launch_batch_traj_w<4, true>(B, b, wi, s) : launch_batch_traj_w<4, false>(B, b, wi, s);
+    return var ? launch_batch_traj_w<8, true>(B, b, wi, s) : launch_batch_traj_w<8, false>(B, b, wi, s);
 }
 
 }  // namespace
@@ -918,7 +888,7 @@ npp_status npp_batch_create(npp_handle* h, const npp_scene* scenes, int32_t S, n
     *out = nullptr;
     if (h->fp_faces > 0)
         return fail(h, NPP_UNSUPPORTED, "batch: a general footprint is checked by the single-scene entry points only");
-    long long pairs = 0, rows = 0, samples = 0, tiles_total = 0, bin_ints = 0, bin_pts = 0, items = 0;
+    long long pairs = 0, rows = 0, samples = 0, tiles_total = 0, bin_ints = 0, bin_pts = 0;
     int max_pairs = 0;
     for (int i = 0; i < S; ++i) {
         const npp_scene& s = scenes[i];
@@ -935,7 +905,6 @@ npp_status npp_batch_create(npp_handle* h, const npp_scene* scenes, int32_t S, n
         tiles_total += ((s.M + 1) / 2 + 31) / 32;
         bin_ints += (long long)(s.T + 1) * BIN_CS_STRIDE;
         bin_pts += (long long)(s.T + 1) * s.M;
-        items += (s.N + 7) / 8;
         rows += (long long)s.N * (s.T + 1);
         samples += s.N;
         max_pairs = std::max(max_pairs, (s.M + 1) / 2);
@@ -958,7 +927,6 @@ npp_status npp_batch_create(npp_handle* h, const npp_scene* scenes, int32_t S, n
     B->slices = 4;
     B->traj_warps = 8;
     B->binned = 1;
-    B->total_items = items;
     cudaError_t e = cudaSuccess;
     auto A = [&](void** p, size_t bytes) { if (e == cudaSuccess) e = cudaMalloc(p, bytes > 0 ? bytes : 16); };
     A((void**)&B->d_scenes, sizeof(SceneDev) * S);
@@ -967,6 +935,7 @@ npp_status npp_batch_create(npp_handle* h, const npp_scene* scenes, int32_t S, n
     for (int w = 0; w < 3; ++w) {
         A((void**)&B->d_torder[w], sizeof(int) * S);
         A((void**)&B->d_titem_prefix[w], sizeof(long long) * (S + 1));
+        A((void**)&B->d_witem_prefix[w], sizeof(long long) * (S + 1));
     }
     A((void**)&B->d_pXY, sizeof(float4) * std::max(1LL, pairs));
     A((void**)&B->d_pV, sizeof(float4) * std::max(1LL, pairs));
@@ -975,12 +944,16 @@ npp_status npp_batch_create(npp_handle* h, const npp_scene* scenes, int32_t S, n
     A((void**)&B->d_bin_cs, sizeof(int) * std::max(1LL, bin_ints));
     A((void**)&B->d_bin_pts, sizeof(float2) * std::max(1LL, bin_pts));
     A((void**)&B->d_bstep_prefix, sizeof(long long) * (S + 1));
-    A((void**)&B->d_coefA, sizeof(float4) * rows);
-    A((void**)&B->d_coefB, sizeof(float2) * rows);
+    A((void**)&B->d_states, sizeof(float4) * rows);
     A((void**)&B->d_jfree, sizeof(float) * samples);
     if (h->cfg.v_limits) A((void**)&B->d_vfirst, sizeof(int) * samples);
     A((void**)&B->d_keys, sizeof(unsigned long long) * S);
     A((void**)&B->d_counters, 64);
+    for (int i = 0; i < 2 && e == cudaSuccess; ++i) {
+        e = cudaStreamCreateWithFlags(&B->side[i], cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&B->join[i], cudaEventDisableTiming);
+    }
+    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&B->fork, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         free_batch(B);
         return fail(h, NPP_CUDA_ERROR, "batch allocation failed: %s", cudaGetErrorString(e));
@@ -1049,12 +1022,10 @@ npp_status npp_plan_batch(npp_batch* B, const float* obs_dev, const npp_batch_ou
     b.reach = (float)(std::sqrt((double)h->cfg.half_len * h->cfg.half_len + (double)h->cfg.half_wid * h->cfg.half_wid)
                       + std::fabs((double)h->cfg.c_off) + 0.1);
     b.grid = make_bin_grid(h->cfg.half_len, h->cfg.half_wid, h->cfg.c_off);
-    b.windowed64 = B->binned ? 1 : 0;
     b.bin_cs = B->d_bin_cs;
     b.bin_pts = B->d_bin_pts;
     b.bstep_prefix = B->d_bstep_prefix;
-    b.coefA = B->d_coefA;
-    b.coefB = B->d_coefB;
+    b.states = B->d_states;
     b.jfree = B->d_jfree;
     b.vfirst = B->d_vfirst;
     b.keys = B->d_keys;
@@ -1063,6 +1034,7 @@ npp_status npp_plan_batch(npp_batch* B, const float* obs_dev, const npp_batch_ou
     for (int w = 0; w < 3; ++w) {
         b.titem_prefix[w] = B->d_titem_prefix[w];
         b.torder[w] = B->d_torder[w];
+        b.witem_prefix[w] = B->d_witem_prefix[w];
         b.n_torder[w] = B->n_torder[w];
     }
     b.citem_prefix = B->d_citem_prefix;
@@ -1079,25 +1051,44 @@ npp_status npp_plan_batch(npp_batch* B, const float* obs_dev, const npp_batch_ou
     }
     CUDA_TRY(h, cudaMemsetAsync(B->d_keys, 0xff, sizeof(unsigned long long) * B->S, s));
     CUDA_TRY(h, cudaMemsetAsync(B->d_counters, 0, 64, s));
-    if (B->max_pairs > 0) {
+    if (!B->binned && B->max_pairs > 0) {
         const int smem = SORT_KEYS * (int)sizeof(int);
         CUDA_TRY(h, ensure_smem(batch_prologue_kernel, smem));
         batch_prologue_kernel<<<B->S, SORT_THREADS, smem, s>>>(b);
         CUDA_TRY(h, cudaGetLastError());
     }
-    // with the binned check the grids come first: the width-64 scenes are
-    // checked inside their trajectory kernel (windowed), the others after
     if (B->binned && B->bin_blocks > 0) {
         const int smem = BIN_NCELL * (int)sizeof(int);
         CUDA_TRY(h, ensure_smem(batch_bin_build_kernel, smem));
         batch_bin_build_kernel<<<(unsigned)B->bin_blocks, 1024, smem, s>>>(b);
         CUDA_TRY(h, cudaGetLastError());
     }
-    if (B->traj_warps == 4) launch_batch_traj<4>(B, b, s); else launch_batch_traj<8>(B, b, s);
-    CUDA_TRY(h, cudaGetLastError());
+    // the widths on three streams (fork and join by events; under stream
+    // capture three graph branches), width 64, the longest, on the caller's:
+    // a width's blocks move in as another's leave, and a binned check runs
+    // as soon as its width's trajectories are in.  With timing on, the
+    // stages follow one another instead.
+    const bool fork = !h->timing;
+    if (fork) CUDA_TRY(h, cudaEventRecord(B->fork, s));
+    for (int w = 2; w >= 0; --w) {
+        if (!B->n_torder[w]) continue;
+        cudaStream_t sw = fork && w < 2 ? B->side[w] : s;
+        if (sw != s) CUDA_TRY(h, cudaStreamWaitEvent(sw, B->fork, 0));
+        CUDA_TRY(h, launch_batch_traj(B, b, w, sw));
+        if (fork && B->binned && w < 2) {
+            batch_binned_kernel<<<(unsigned)B->witems[w], 256, 0, sw>>>(b, w);
+            CUDA_TRY(h, cudaGetLastError());
+        }
+        if (sw != s) CUDA_TRY(h, cudaEventRecord(B->join[w], sw));
+    }
+    if (fork)
+        for (int w = 0; w < 2; ++w)
+            if (B->n_torder[w]) CUDA_TRY(h, cudaStreamWaitEvent(s, B->join[w], 0));
     if (h->timing) CUDA_TRY(h, record_event(h->ev[1], s));
     if (B->binned) {
-        batch_binned_kernel<<<(unsigned)B->total_items, 256, 0, s>>>(b);
+        if (!fork)
+            for (int w = 0; w < 2; ++w)
+                if (B->n_torder[w]) batch_binned_kernel<<<(unsigned)B->witems[w], 256, 0, s>>>(b, w);
     } else {
         switch (B->slices) {
         case 2: launch_batch_collide<2>(B, b, s); break;
