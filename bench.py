@@ -295,7 +295,7 @@ def algorithmic_work(first_hit, T, M, W):
 
 
 # source files whose code each profiled kernel is built from
-_ROLLOUT = ("npp_rollout.cuh", "npp_device.cuh", "npp_async.cuh", "npp_tmem.cuh")
+_ROLLOUT = ("npp_rollout.cuh", "npp_device.cuh", "npp_async.cuh", "npp_tmem.cuh", "npp_launch.cuh")
 KERNEL_SOURCES = tuple(
     (kind + "<%d" % w, _ROLLOUT + ("npp_rollout_w%d.cu" % w,))      # each width's own translation unit
     for kind in ("traj_kernel", "fused_kernel", "traj_tmem_kernel", "fused_tmem_kernel") for w in (16, 32, 64)) + (
@@ -512,8 +512,8 @@ def run_npp(args):
     nch = 1
     if binned and not poly and not fused:
         nch = min(int(options.get("chunks", 0)) or (2 if W == 64 else 1), T)
-    # per sampling time: plan step kernels, epilogue, vehicle and obstacle advance
-    launches_per_step = (2 if fused else 1 + 2 * nch if binned and not poly else 3 if poly else 2) + 3
+    # per sampling time: plan step kernels, epilogue, vehicle and obstacle advance (one up to 4096 points)
+    launches_per_step = (2 if fused else 1 + 2 * nch if binned and not poly else 3 if poly else 2) + 2 + (M > 4096)
     # default launch shapes; the fifth template argument is the variant flag
     # (off: no speed limits, features in the EV frame at t)
     var = int(bool(p.get("v_limits", 0) or p.get("feature_frame", 0)))
@@ -1092,8 +1092,8 @@ def run_mission(args):
             tm = npp.npp_loop_last_timing(L)
             if t >= args.warmup or k > 0:
                 step_ms.append(tm["total"])
-            # trajectories, collision check (+ grid build when binned), epilogue, vehicle, points
-            launches += 5 if states_auto(M, N, W) else 6
+            # trajectories, collision check (+ grid build when binned), epilogue, vehicle and points (one up to 4096)
+            launches += (4 if states_auto(M, N, W) else 5) + (M > 4096)
             st = npp.npp_loop_read(L)
             if st["done"]:
                 done_at = st["t"]

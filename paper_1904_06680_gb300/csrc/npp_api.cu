@@ -12,6 +12,7 @@
 #include "../../include/npp.h"
 #include "npp_device.cuh"
 #include "npp_internal.h"
+#include "npp_launch.cuh"
 
 using namespace npp;
 
@@ -53,7 +54,10 @@ __global__ void epilogue_kernel(const EpilogueArgs e)
         skey.t_index = e.dyn->t_index;
         warm_ok = e.dyn->warm_valid != 0 || e.warm_force != 0;
     }
-    const unsigned long long key = *e.best_key;
+    float s0, c0;
+    sincosf(phi0, &s0, &c0);
+    wait_for_previous();                   // the check
+    const unsigned long long key = *reinterpret_cast<const volatile unsigned long long*>(e.best_key);
     const int idx = (int)(key & 0xffffffffull);
     const bool dead = (key >> 63) != 0;
     const unsigned hi = (unsigned)((key >> 32) & 0x7fffffffu);
@@ -72,8 +76,6 @@ __global__ void epilogue_kernel(const EpilogueArgs e)
         b->first_hit = fh;
         b->reserved[0] = b->reserved[1] = b->reserved[2] = b->reserved[3] = 0;
     }
-    float s0, c0;
-    sincosf(phi0, &s0, &c0);
     if (e.trajectory) {
         for (int h = threadIdx.x; h <= e.T; h += blockDim.x) {
             const float4 z = e.traj[(size_t)min(h, last) * e.N + idx];
@@ -146,8 +148,7 @@ void set_global_error(const char* msg) { g_err = msg; }
 // The winner epilogue for callers outside this file (one block of 256).
 cudaError_t launch_epilogue(const EpilogueArgs& e, cudaStream_t s)
 {
-    epilogue_kernel<<<1, 256, 0, s>>>(e);
-    return cudaGetLastError();
+    return launch_dependent(epilogue_kernel, 1, 256, 0, s, e);
 }
 }  // namespace npp
 
@@ -345,6 +346,7 @@ npp_status run_rollout(npp_handle* h, RolloutArgs& a, cudaStream_t s, bool no_re
         return NPP_OK;
     }
     if (v == COLLIDE_STATES) {
+        a.reset_key = a.best_key;
         if (h->timing) CUDA_TRY(h, record_event(h->ev[0], s));
         CUDA_TRY(h, launch_traj(h, a, s));
         if (h->timing) CUDA_TRY(h, record_event(h->ev[1], s));
@@ -366,6 +368,7 @@ npp_status run_rollout(npp_handle* h, RolloutArgs& a, cudaStream_t s, bool no_re
         a.grid_collide = h->sm_count * h->occ_blocks;
     }
     CUDA_TRY(h, cudaMemsetAsync(h->d_work, 0, sizeof(unsigned), s));
+    a.reset_key = a.best_key;
     if (h->timing) CUDA_TRY(h, record_event(h->ev[0], s));
     CUDA_TRY(h, launch_traj(h, a, s));
     if (h->timing) CUDA_TRY(h, record_event(h->ev[1], s));
@@ -563,7 +566,6 @@ static npp_status plan_step_impl(npp_handle* h, const npp_state* state, const np
     a.ctrl = out->sample_ctrl ? reinterpret_cast<float2*>(out->sample_ctrl) : h->d_ctrl;
     a.jfree = h->d_jfree;
     a.best_key = h->d_key;
-    CUDA_TRY(h, cudaMemsetAsync(h->d_key, 0xff, sizeof(unsigned long long), s));
     const bool records = out->sample_traj != nullptr || out->sample_ctrl != nullptr;
     if ((st = run_rollout(h, a, s, !records)) != NPP_OK) return st;
 

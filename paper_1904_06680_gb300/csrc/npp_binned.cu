@@ -33,6 +33,11 @@ __global__ void __launch_bounds__(BIN_THREADS) bin_build_kernel(const RolloutArg
     extern __shared__ int cnt[];             // [BIN_NCELL]
     __shared__ int run_tot[BIN_THREADS];
     const int h = blockIdx.x;
+    if (h == 0 && threadIdx.x == 0) {
+        // start of the plan step's minimum and sample queue
+        if (a.best_key) *a.best_key = ~0ull;
+        if (a.work) *a.work = 0u;
+    }
     const StepIn si = step_in(a);
     float s0, c0;
     sincosf(si.phi0, &s0, &c0);
@@ -58,6 +63,7 @@ template <bool POLY>
 __global__ void __launch_bounds__(BINNED_WARPS * 32, 5) collide_binned_kernel(const RolloutArgs a)
 {
     __shared__ float4 faces[POLY ? FP_MAX_FACES : 1];
+    start_next();
     if constexpr (POLY) {
         for (int i = threadIdx.x; i < a.poly.n_faces; i += blockDim.x) faces[i] = a.poly.faces[i];
         __syncthreads();

@@ -33,6 +33,7 @@ __global__ void __launch_bounds__(STATES_WARPS * 32) collide_states_kernel(const
     extern __shared__ __align__(16) float4 pairs[];              // XY_q at 2 q, V_q at 2 q + 1
     const int tid = threadIdx.x, lane = tid & 31;
     const int T = a.T, N = a.N, npairs = (a.M + 1) / 2;
+    start_next();
     {
         const StepIn si = step_in(a);
         float s0, c0;
@@ -50,6 +51,7 @@ __global__ void __launch_bounds__(STATES_WARPS * 32) collide_states_kernel(const
         }
     }
     __syncthreads();
+    wait_for_previous();                                         // the trajectories
     const int sl = lane % S, ph = lane / S;                      // sample and step of this lane
     const int n = (blockIdx.x * STATES_WARPS + (tid >> 5)) * S + sl;
     const bool valid = n < N;
@@ -117,8 +119,8 @@ template <int P>
 static cudaError_t launch_states(const RolloutArgs& a, cudaStream_t s)
 {
     constexpr int per_block = STATES_WARPS * (32 / P);
-    collide_states_kernel<P><<<(a.N + per_block - 1) / per_block, STATES_WARPS * 32, (a.M + 1) / 2 * 32, s>>>(a);
-    return cudaGetLastError();
+    return launch_dependent(collide_states_kernel<P>, (a.N + per_block - 1) / per_block, STATES_WARPS * 32,
+                            (size_t)((a.M + 1) / 2 * 32), s, a);
 }
 
 // One sample per warp, 32 steps a round, except for many samples with few

@@ -535,6 +535,7 @@ struct RolloutArgs {
     float4* coefA;                     // [T+1][N] (A, B, -C, D) scaled inequality rows
     float2* coefB;                     // [T+1][N] (E, -F)
     unsigned long long* best_key;      // packed (class, cost, index) minimum
+    unsigned long long* reset_key;     // the minimum, for the trajectory kernel to start (null: started elsewhere)
     unsigned* work;                    // work-queue counter of the persistent collision kernel
     int grid_collide;                  // persistent grid size
     int sm_count;                      // SMs of the device

@@ -17,6 +17,7 @@
 #include "../../include/npp.h"
 #include "npp_device.cuh"
 #include "npp_internal.h"
+#include "npp_launch.cuh"
 
 using namespace npp;
 
@@ -196,12 +197,12 @@ __global__ void mission_init_kernel(LoopDev* d, const float4* __restrict__ ref)
 // Obstacle points at the current sampling time t (the state kernel has
 // advanced t): p0 + tau v, tau = t Ts; with hide, points outside the range
 // field at t are moved far away (at rest), so no plan step sees them.
-__global__ void advance_obstacles_kernel(const LoopDev* d, const float4* __restrict__ obs0,
-                                         float4* __restrict__ obs, int M, float Ts)
+__device__ __forceinline__ void advance_points(const LoopDev* d, const float4* __restrict__ obs0,
+                                               float4* __restrict__ obs, int M, float Ts, int first, int stride)
 {
     const float tau = (float)d->t * Ts;
     const Pose v = { d->px, d->py, d->pphi, d->pv, d->cphi, d->sphi };
-    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < M; j += gridDim.x * blockDim.x) {
+    for (int j = first; j < M; j += stride) {
         const float4 o = obs0[j];
         const float px = fmaf(tau, o.z, o.x), py = fmaf(tau, o.w, o.y);
         if (d->hide && !in_field(v, d->field, px, py)) obs[j] = make_float4(HIDDEN_POINT, HIDDEN_POINT, 0.0f, 0.0f);
@@ -209,14 +210,20 @@ __global__ void advance_obstacles_kernel(const LoopDev* d, const float4* __restr
     }
 }
 
+__global__ void advance_obstacles_kernel(const LoopDev* d, const float4* __restrict__ obs0,
+                                         float4* __restrict__ obs, int M, float Ts)
+{
+    advance_points(d, obs0, obs, M, Ts, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
 // Steps 6 and 7 of Alg. 1: one sampling time of the simulated vehicle (the
 // kinematic bicycle of Sect. IV, FP64, explicit Euler on the old state) under
 // the winner's first applied control; waypoint switch or mission update;
 // log row (x, y, phi, v, a0, a1, best cost, goal index).  One warp: every
 // lane computes the same vehicle step, lane 0 writes.
-__global__ void advance_state_kernel(LoopDev* d, const float* __restrict__ controls,
-                                     const npp_best* __restrict__ best, const float4* __restrict__ wps,
-                                     float* __restrict__ log, int max_log, PlantCfg pc)
+__device__ __forceinline__ void advance_vehicle(LoopDev* d, const float* controls, const npp_best* best,
+                                                const float4* __restrict__ wps, float* __restrict__ log, int max_log,
+                                                const PlantCfg& pc)
 {
     const int lane = threadIdx.x & 31;
     const double a0 = controls[0], a1 = controls[1];
@@ -264,6 +271,26 @@ __global__ void advance_state_kernel(LoopDev* d, const float* __restrict__ contr
     d->warm_valid = 1;
 }
 
+// The vehicle's step by the block's first warp, then, for obs not null, the
+// points at the new time by the whole block: one launch instead of two per
+// sampling time where one block moves the points as fast as several
+// (ADVANCE_ONE_BLOCK points or fewer).
+constexpr int ADVANCE_THREADS = 512;
+constexpr int ADVANCE_ONE_BLOCK = 4096;
+__global__ void __launch_bounds__(ADVANCE_THREADS)
+advance_kernel(LoopDev* d, const float* controls, const npp_best* best, const float4* __restrict__ wps,
+               float* __restrict__ log, int max_log, PlantCfg pc, const float4* __restrict__ obs0,
+               float4* __restrict__ obs, int M)
+{
+    // (controls and best come from the kernel before: no __restrict__, so no
+    // read of them moves above the wait)
+    wait_for_previous();                   // the winner epilogue
+    if (threadIdx.x < 32) advance_vehicle(d, controls, best, wps, log, max_log, pc);
+    if (!obs) return;
+    __syncthreads();
+    advance_points(d, obs0, obs, M, (float)pc.Ts, threadIdx.x, ADVANCE_THREADS);
+}
+
 void free_loop(npp_loop* L)
 {
     if (!L) return;
@@ -301,7 +328,6 @@ npp_status enqueue_step(npp_loop* L, uint64_t seed)
     a.dyn = L->d_dyn;
     a.costs = L->d_costs;
     a.first_hit = L->d_fh;
-    CUDA_TRY(h, cudaMemsetAsync(h->d_key, 0xff, sizeof(unsigned long long), s));
     npp_status st = run_rollout(h, a, s, true);
     if (st != NPP_OK) return st;
     EpilogueArgs e;
@@ -331,7 +357,6 @@ npp_status enqueue_step(npp_loop* L, uint64_t seed)
         ar.prop = Proposal{ L->d_warm, L->d_sigma, L->N, (uint32_t)r };
         ar.warm = L->d_warm;
         ar.warm_force = 1;
-        CUDA_TRY(h, cudaMemsetAsync(h->d_key, 0xff, sizeof(unsigned long long), s));
         st = run_rollout(h, ar, s, true);
         if (st != NPP_OK) {
             h->timing = timing;
@@ -350,10 +375,11 @@ npp_status enqueue_step(npp_loop* L, uint64_t seed)
     PlantCfg pc;
     pc.lf = h->cfg.lf; pc.lr = h->cfg.lr; pc.delta_max = h->cfg.delta_max;
     pc.u_min = h->cfg.u_min; pc.u_max = h->cfg.u_max; pc.Ts = h->cfg.Ts;
-    advance_state_kernel<<<1, 32, 0, s>>>(L->d_dyn, L->d_controls, L->d_best, L->d_wp, L->d_log,
-                                         L->max_log, pc);
-    CUDA_TRY(h, cudaGetLastError());
-    if (L->M > 0) {
+    const bool one = L->M > 0 && L->M <= ADVANCE_ONE_BLOCK;
+    CUDA_TRY(h, launch_dependent(advance_kernel, 1, one ? ADVANCE_THREADS : 32, 0, s, L->d_dyn, L->d_controls,
+                                 L->d_best, L->d_wp, L->d_log, L->max_log, pc, L->d_obs0,
+                                 one ? L->d_obs : nullptr, L->M));
+    if (L->M > 0 && !one) {
         advance_obstacles_kernel<<<(L->M + 255) / 256, 256, 0, s>>>(L->d_dyn, L->d_obs0, L->d_obs, L->M,
                                                                      (float)pc.Ts);
         CUDA_TRY(h, cudaGetLastError());

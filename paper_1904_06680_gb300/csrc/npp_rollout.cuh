@@ -34,6 +34,7 @@
 #include "npp_device.cuh"
 #include "npp_async.cuh"
 #include "npp_tmem.cuh"
+#include "npp_launch.cuh"
 
 namespace npp {
 
@@ -1174,6 +1175,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) traj_kernel(const RolloutArgs a
     extern __shared__ __align__(16) float stage_all[];
     const int tid = threadIdx.x;
     const int b = tid / G, gl = tid % G;
+    if (a.reset_key && blockIdx.x == 0 && tid == 0) *a.reset_key = ~0ull;
     int n = blockIdx.x * B + b;
     bool valid = n < a.N;
     if (a.live_in) {
@@ -1365,6 +1367,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) traj_tmem_kernel(const RolloutA
     float* hx_all = reinterpret_cast<float*>(w2_all + NW * 32 * Net::U * KS);
     const int tid = threadIdx.x, b = tid / G, gl = tid % G, warp = tid >> 5;
     const uint32_t tmem = tmem_alloc<tmem_cols<Net, NW>()>(&tslot);
+    start_next();
+    if (a.reset_key && blockIdx.x == 0 && tid == 0) *a.reset_key = ~0ull;
     int n = blockIdx.x * B + b;
     bool valid = n < a.N;
     bool idle = false;
@@ -1394,7 +1398,8 @@ __global__ void __launch_bounds__(NW * 32, MINB) traj_tmem_kernel(const RolloutA
 
 // Trajectories with the windowed check (as fused_kernel): the warps of a
 // resident grid take samples from a queue, so that a warp whose sample ends
-// early starts another at once (a.work: the samples taken so far).
+// early starts another at once (a.work: the samples taken so far, started by
+// the grid build).
 template <int W, int G, int NW, int MINB, bool VAR, int KT, int KS, int CW, int R>
 __global__ void __launch_bounds__(NW * 32, MINB) fused_tmem_kernel(const RolloutArgs a)
 {
@@ -1407,6 +1412,7 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_tmem_kernel(const Rollout
     float* hx_all = reinterpret_cast<float*>(wnd_all + NW * NG * CW);
     const int tid = threadIdx.x, b = tid / G, gl = tid % G, warp = tid >> 5, lane = tid & 31;
     const uint32_t tmem = tmem_alloc<tmem_cols<Net, NW>()>(&tslot);
+    start_next();
     TrajJob job = traj_job<W, G>(a);
     job.jfree = nullptr;
     job.vfirst = nullptr;
@@ -2083,7 +2089,6 @@ cudaError_t launch_fused_tmem(const RolloutArgs& a, cudaStream_t stream)
     auto fn = fused_tmem_kernel<W, G, NW, MINB, VAR, KT, KS, CW, R>;
     constexpr int B = NW * 32 / G, smem = tmem_block_bytes<W, G, NW, KS, CW>();
     cudaError_t e = ensure_smem(fn, smem);
-    if (e == cudaSuccess) e = cudaMemsetAsync(a.work, 0, sizeof(unsigned), stream);
     if (e != cudaSuccess) return e;
     fn<<<min((a.N + B - 1) / B, MINB * a.sm_count), NW * 32, smem, stream>>>(a);
     return cudaGetLastError();
