@@ -300,6 +300,7 @@ KERNEL_SOURCES = tuple(
     (kind + "<%d" % w, _ROLLOUT + ("npp_rollout_w%d.cu" % w,))      # each width's own translation unit
     for kind in ("traj_kernel", "fused_kernel", "traj_tmem_kernel", "fused_tmem_kernel") for w in (16, 32, 64)) + (
     ("bin_build_kernel", _ROLLOUT + ("npp_binned.cu",)),
+    ("collide_grid_kernel", _ROLLOUT + ("npp_binned.cu",)),
     ("collide_binned_kernel", _ROLLOUT + ("npp_binned.cu",)),
     ("collide_poly_kernel", _ROLLOUT + ("npp_poly.cu",)),
     ("collide_", _ROLLOUT + ("npp_collide.cu",)),
@@ -571,7 +572,8 @@ def run_npp(args):
         # cells a state overlaps, which has no fixed algorithmic count; the
         # MLP rollout is the work every plan step must do
         tname = "traj" + shape
-        cname = "bin_build_kernel + " + ("collide_poly_kernel" if poly else "collide_binned_kernel")
+        cname = "bin_build_kernel + " + ("collide_binned_kernel" if poly or nch > 1 or N < 1024 or M > 8702
+                                         else "collide_grid_kernel")
         fps_t = res["fma_t"] / (traj_ms / 1e3)
         coll = {"ms_per_step": collide_ms / K}
         if not poly and res["states"] > 0:

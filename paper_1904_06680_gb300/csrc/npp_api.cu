@@ -320,14 +320,21 @@ npp_status run_rollout(npp_handle* h, RolloutArgs& a, cudaStream_t s, bool no_re
             // stream capture this makes two graph branches)
             CUDA_TRY(h, cudaEventRecord(h->fork_ev, s));
             CUDA_TRY(h, cudaStreamWaitEvent(h->side, h->fork_ev, 0));
+            const int K = chunk_count(h, a, no_records);
+            const bool grid = K == 1 && grid_auto(a.M, a.N, a.T);
+            if (grid) {
+                a.first = h->d_first;
+                a.done = h->d_first + h->cfg.max_N;
+            }
             CUDA_TRY(h, build_bins(a, h->cfg.half_len, h->cfg.half_wid, h->cfg.c_off, h->d_bins, h->side));
             CUDA_TRY(h, cudaEventRecord(h->join_ev, h->side));
-            const int K = chunk_count(h, a, no_records);
             if (K > 1) return run_chunked(h, a, s, K);
             CUDA_TRY(h, launch_traj(h, a, s));
             if (h->timing) CUDA_TRY(h, record_event(h->ev[1], s));
             CUDA_TRY(h, cudaStreamWaitEvent(s, h->join_ev, 0));
-            CUDA_TRY(h, launch_collide_binned(a, s));
+            CUDA_TRY(h, grid ? launch_collide_grid(a, s) : launch_collide_binned(a, s));
+            a.first = nullptr;
+            a.done = nullptr;
             a.counts = nullptr;
             if (h->timing) CUDA_TRY(h, record_event(h->ev[2], s));
             return NPP_OK;
@@ -492,6 +499,7 @@ npp_status npp_create(npp_handle** out, const npp_config* cfg, int32_t device)
     A((void**)&h->d_fault, sizeof(unsigned));
     A((void**)&h->d_live, (size_t)2 * cfg->max_N * sizeof(int));
     A((void**)&h->d_live_n, NPP_MAX_CHUNKS * sizeof(int));
+    A((void**)&h->d_first, ((size_t)cfg->max_N + GRID_MAX_CHUNKS) * sizeof(int));
     A((void**)&h->d_carry, (size_t)cfg->max_N * sizeof(float4));
     A(&h->d_bins, binned_workspace_bytes(cfg->max_T, cfg->max_M));
     if (cfg->max_M > max_points) {
@@ -528,7 +536,7 @@ npp_status npp_destroy(npp_handle* h)
     cudaSetDevice(h->device);
     if (h->stream) cudaStreamSynchronize(h->stream);
     void* ptrs[] = { h->d_key, h->d_traj, h->d_ctrl, h->d_jfree, h->d_vfirst, h->d_fp, h->d_work, h->d_counts,
-                     h->d_live, h->d_live_n, h->d_carry,
+                     h->d_live, h->d_live_n, h->d_first, h->d_carry,
                      h->d_pXY, h->d_fault, h->d_bins,
                      h->d_obs, h->d_warm, h->d_sigma, h->d_best, h->d_params, h->d_controls, h->d_trajectory,
                      h->d_costs, h->d_fh };

@@ -38,6 +38,12 @@ __global__ void __launch_bounds__(BIN_THREADS) bin_build_kernel(const RolloutArg
         if (a.best_key) *a.best_key = ~0ull;
         if (a.work) *a.work = 0u;
     }
+    if (a.first) {
+        // start of the grid check: no collision known, no step finished
+        for (int i = h * BIN_THREADS + threadIdx.x; i < a.N; i += gridDim.x * BIN_THREADS) a.first[i] = 0x7fffffff;
+        if (h == 0)
+            for (int i = threadIdx.x; i < GRID_MAX_CHUNKS; i += BIN_THREADS) a.done[i] = 0;
+    }
     const StepIn si = step_in(a);
     float s0, c0;
     sincosf(si.phi0, &s0, &c0);
@@ -155,6 +161,123 @@ __global__ void __launch_bounds__(BINNED_WARPS * 32, 5) collide_binned_kernel(co
         atomicMin(a.best_key, key);
 }
 
+// ------------------------------------------------------------------ one step's grid in shared memory
+// Block (x, h) checks a chunk of the samples at step h: the step's grid
+// (cell starts as 16-bit offsets, 32 KB, and its M points) is copied into
+// shared memory once, then every lane takes one state at a time -- its rows,
+// the cell rows of its query and their runs of points, two at a time -- and a
+// collision lowers the sample's first colliding step.  Blocks start in the
+// order of their steps, so a sample that collided early is mostly skipped at
+// later steps.  The chunk's last block to finish turns the first steps into
+// costs and keys.  The candidates and the per-point test are the
+// warp-per-sample kernel's, so the same flags.
+//
+// Why: there, a warp's four states at a time each wait for two dependent L2
+// reads (cell bounds, then points; every step has its own grid, so they miss
+// L1), and eight lanes repeat a state's query arithmetic.
+// Bound: shared-memory bank conflicts and lanes waiting for the longest run
+// of their warp.  Measured on GB300 (check after the trajectories, us,
+// against the warp-per-sample kernel): course (16384 x 41 states, 2000
+// points) 42 / 54, 5003 x 61 states 25 / 32, 8192 x 41 (855 points) 21 / 27,
+// large (65536 x 101, 8192 points) 207 / 306; a handful of samples 11 / 7.
+// (With polygons, whose test is long, lanes diverge: 316 / 134.)
+constexpr int GRID_THREADS = 512;
+constexpr int GRID_CS_BYTES = (BIN_NCELL + 8) * 2;
+
+__global__ void __launch_bounds__(GRID_THREADS, 2) collide_grid_kernel(const RolloutArgs a, int chunk)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    unsigned short* cs = reinterpret_cast<unsigned short*>(smem_raw);
+    float2* pts = reinterpret_cast<float2*>(smem_raw + GRID_CS_BYTES);
+    __shared__ int last;
+    __shared__ unsigned long long red[GRID_THREADS / 32];
+    const int tid = threadIdx.x, h = blockIdx.y;
+    const int T = a.T, N = a.N, M = a.M;
+    const int n0 = blockIdx.x * chunk, n1 = min(N, n0 + chunk);
+    const BinView& g = a.bins;
+    start_next();
+    {
+        const int4* src = reinterpret_cast<const int4*>(g.cell_start + (size_t)h * BIN_CS_STRIDE);
+        ushort4* dst = reinterpret_cast<ushort4*>(cs);
+        for (int i = tid; i < BIN_NCELL / 4; i += GRID_THREADS) {
+            const int4 v = src[i];
+            dst[i] = make_ushort4((unsigned short)v.x, (unsigned short)v.y, (unsigned short)v.z, (unsigned short)v.w);
+        }
+        const float2* p = g.pts + (size_t)h * M;
+        for (int i = tid; i < M; i += GRID_THREADS) pts[i] = p[i];
+        if (tid == 0) cs[BIN_NCELL] = (unsigned short)M;
+    }
+    __syncthreads();
+    unsigned ntest = 0, nstate = 0;
+    for (int n = n0 + tid; n < n1; n += GRID_THREADS) {
+        if (__ldcg(a.first + n) <= h) continue;
+        const float4 z = a.traj[(size_t)h * N + n];
+        float sp, cp;
+        sincos_r(z.z, sp, cp);
+        RectTest test;
+        coef_rows(a.c, z.x, z.y, sp, cp, test.a, test.b);
+        const QueryBox q = query_box(g, z.x, z.y, sp, cp);
+        const int ix0 = bin_cell(q.x - q.rx, g), ix1 = bin_cell(q.x + q.rx, g);
+        const int iy0 = bin_cell(q.y - q.ry, g), iy1 = min(bin_cell(q.y + q.ry, g), iy0 + BIN_MAX_ROWS - 1);
+        bool hit = false;
+        for (int iy = iy0; iy <= iy1 && !hit; ++iy) {
+            const int b = cs[iy * BIN_DIM + ix0], e = cs[iy * BIN_DIM + ix1 + 1];
+            ntest += e - b;
+            // two points a pass (an odd run's last point twice)
+            for (int i = b; i < e; i += 2) hit |= test(pts[i]) | test(pts[min(i + 1, e - 1)]);
+        }
+        ++nstate;
+        if (hit) atomicMin(a.first + n, h);
+    }
+    if (a.counts) {
+        unsigned long long t = ntest, s = nstate;
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            t += __shfl_xor_sync(FULL, t, off);
+            s += __shfl_xor_sync(FULL, s, off);
+        }
+        if ((tid & 31) == 0) {
+            atomicAdd(a.counts, t);
+            atomicAdd(a.counts + 1, s);
+        }
+    }
+    // the chunk's last block: every first colliding step is in
+    __threadfence();
+    __syncthreads();
+    if (tid == 0) last = atomicAdd(a.done + blockIdx.x, 1) == T;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    unsigned long long best = ~0ull;
+    for (int n = n0 + tid; n < n1; n += GRID_THREADS) {
+        const int f = __ldcg(a.first + n);
+        const int fh = discard_step(a.vfirst, n, f <= T ? f : -1);
+        float J = __int_as_float(0x7f800000);
+        unsigned long long key;
+        if (fh < 0) {
+            J = a.jfree[n];
+            key = ((unsigned long long)__float_as_uint(J) << 32) | (unsigned)n;
+        } else {
+            key = (1ull << 63) | ((unsigned long long)(T - fh) << 32) | (unsigned)n;
+        }
+        if (a.costs) a.costs[n] = J;
+        if (a.first_hit) a.first_hit[n] = fh;
+        best = key < best ? key : best;
+    }
+    if (!a.best_key) return;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const unsigned long long o = __shfl_xor_sync(FULL, best, off);
+        best = o < best ? o : best;
+    }
+    if ((tid & 31) == 0) red[tid >> 5] = best;
+    __syncthreads();
+    if (tid == 0) {
+        for (int w = 1; w < GRID_THREADS / 32; ++w) best = red[w] < best ? red[w] : best;
+        atomicMin(a.best_key, best);
+    }
+}
+
 }  // namespace
 
 namespace npp {
@@ -190,6 +313,24 @@ cudaError_t build_bins(RolloutArgs& a, float half_len, float half_wid, float c_o
 cudaError_t build_bins_poly(RolloutArgs& a, double radius, const double box[4], void* workspace, cudaStream_t s)
 {
     return build_grids(a, make_bin_grid_box(radius, box), workspace, s);
+}
+
+// points that leave two blocks per SM (the offsets are 16-bit)
+int collide_grid_points() { return (100 * 1024 - GRID_CS_BYTES) / 8; }
+
+cudaError_t launch_collide_grid(const RolloutArgs& a, cudaStream_t s)
+{
+    // chunks of the samples so that the (chunk, step) blocks are about three
+    // per SM: fewer would leave SMs idle, more would copy the grids oftener
+    const int want = max(1, 3 * a.sm_count / (a.T + 1));
+    int chunk = (a.N + want - 1) / want;
+    chunk = (chunk + GRID_THREADS - 1) / GRID_THREADS * GRID_THREADS;
+    const dim3 grid((a.N + chunk - 1) / chunk, a.T + 1);
+    const int smem = GRID_CS_BYTES + a.M * (int)sizeof(float2);
+    const cudaError_t e = cudaFuncSetAttribute(collide_grid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    collide_grid_kernel<<<grid, GRID_THREADS, smem, s>>>(a, chunk);
+    return cudaGetLastError();
 }
 
 cudaError_t launch_collide_binned(const RolloutArgs& a, cudaStream_t s)

@@ -565,6 +565,8 @@ struct RolloutArgs {
     int* live_n_out;
     float4* carry;
     PolyView poly;                     // general footprint (polygon checks)
+    int* first;                        // [N] first colliding step so far (grid check; null: another check)
+    int* done;                         // [GRID_MAX_CHUNKS] steps finished per sample chunk
 };
 
 __device__ __forceinline__ StepIn step_in(const RolloutArgs& a)
@@ -627,6 +629,11 @@ int collide_max_points(int smem_limit);
 size_t binned_workspace_bytes(int max_T, int max_M);
 cudaError_t build_bins(RolloutArgs& a, float half_len, float half_wid, float c_off, void* workspace,
                        cudaStream_t s);          // fills a.bins
+// the rectangle's binned check with a step's grid in shared memory (M <=
+// collide_grid_points()); the grid build starts `first` and `done`
+constexpr int GRID_MAX_CHUNKS = 1024;
+int collide_grid_points();
+cudaError_t launch_collide_grid(const RolloutArgs& a, cudaStream_t s);
 cudaError_t launch_collide_binned(const RolloutArgs& a, cudaStream_t s);
 cudaError_t launch_collide_poly(const RolloutArgs& a, cudaStream_t s);     // every point (a.poly.brute)
 // grids for a general footprint inside the disk of the given radius around

@@ -26,6 +26,12 @@ inline bool states_auto(int M, int N, int width)
     return M < (width == 64 ? 128 : N <= 1024 ? 257 : 160);
 }
 
+// Whether the rectangle's binned check over all steps takes a step's grid into
+// shared memory: enough samples to pay for the copies (from 1024; below, the
+// warp-per-sample kernel's latency is less), points that leave two blocks per
+// SM, and steps within a launch's grid.
+inline bool grid_auto(int M, int N, int T) { return N >= 1024 && M <= npp::collide_grid_points() && T < 65535; }
+
 // most step chunks of one plan step, and the stage events they need
 constexpr int NPP_MAX_CHUNKS = 8;
 constexpr int NPP_CHUNK_EVENTS = 2 * NPP_MAX_CHUNKS + 1;
@@ -58,6 +64,7 @@ struct npp_handle {
     int last_chunks;                     // chunks of the last timed plan step (its stage events)
     int* d_live;                         // [2][max_N] samples still collision-free between chunks
     int* d_live_n;                       // [NPP_MAX_CHUNKS] their counts
+    int* d_first;                        // [max_N] first colliding steps, then the chunk counters (grid check)
     float4* d_carry;                     // [max_N] values carried from chunk to chunk
     int loop_restarts;                   // hill-climb rounds per sampling time of new loops (1: none)
     float loop_sigma;                    // their perturbation scale
