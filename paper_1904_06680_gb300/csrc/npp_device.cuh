@@ -463,6 +463,16 @@ __device__ __forceinline__ float tanh_r(float x)
     return fmaf(-2.0f, sfu_rcp(e + 1.0f), 1.0f);
 }
 
+// tanh_r of two values side by side (each rounding as above)
+__device__ __forceinline__ void tanh_r2(float& x0, float& x1)
+{
+    const float2 t = f2_unpack(f2_mul(f2_pack(x0, x1), f2_both(2.88539008177792681f)));
+    const float2 e = f2_unpack(f2_add(f2_pack(sfu_ex2(t.x), sfu_ex2(t.y)), f2_both(1.0f)));
+    const float2 r = f2_unpack(f2_fma(f2_both(-2.0f), f2_pack(sfu_rcp(e.x), sfu_rcp(e.y)), f2_both(1.0f)));
+    x0 = r.x;
+    x1 = r.y;
+}
+
 // tan z = sin z / cos z for the steering angle (|z| <= delta_max < pi/2)
 __device__ __forceinline__ float tan_r(float z)
 {

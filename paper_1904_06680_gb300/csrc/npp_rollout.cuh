@@ -581,13 +581,24 @@ __device__ __forceinline__ bool binned_item_inside(const DevCfg& c, const BinVie
     if (ok) cr = cand_rows(g.cell_start + (size_t)h * BIN_CS_STRIDE, g, query_box(g, z.x, z.y, sp, cp));
     const float2* pts = g.pts + (size_t)(ok ? h : 0) * g.M;
     const int total = cr.total;
+    // most states have few candidates, many none: no load for the warp's four
+    // items, or one per lane, before the general case
+    const int most = __reduce_max_sync(FULL, total);
+    if (most == 0) return false;
+    bool inside = false;
+    if (most <= L) {
+        if (gl < total) {
+            inside = inside_rows(ca, cb, pts[cr.index(gl)]);
+            ++ntest;
+        }
+        return inside;
+    }
     float2 pr[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) {
         const int k = gl + r * L;
         pr[r] = k < total ? pts[cr.index(k)] : make_float2(0.f, 0.f);
     }
-    bool inside = false;
 #pragma unroll
     for (int r = 0; r < R; ++r)
         if (gl + r * L < total) {
@@ -596,7 +607,7 @@ __device__ __forceinline__ bool binned_item_inside(const DevCfg& c, const BinVie
         }
     constexpr int PRE = R * L;
     const int rest = total > PRE ? (total - PRE + L - 1) / L : 0;
-    const int maxr = __reduce_max_sync(FULL, rest);
+    const int maxr = most > PRE ? (most - PRE + L - 1) / L : 0;
     for (int it = 0; it < maxr; ++it) {
         const int k = PRE + it * L + gl;
         if (it < rest && k < total) {
@@ -927,8 +938,10 @@ __device__ __forceinline__ float2 control_step(const DevCfg& c, const Net& net, 
 #pragma unroll
         for (int i = 1; i < NIN / 2; ++i) q = f2_fma(net.w1p[j][i], sp2[i], q);
         const float2 qq = f2_unpack(q);
-        h1[j] = tanh_r(__fadd_rn(__fadd_rn(qq.x, qq.y), net.b1[j]));
+        h1[j] = __fadd_rn(__fadd_rn(qq.x, qq.y), net.b1[j]);
     }
+#pragma unroll
+    for (int j = 0; j < U; j += 2) tanh_r2(h1[j], h1[j + 1]);
 #pragma unroll
     for (int j = 0; j < U; ++j) hrow[gl * U + j] = h1[j];
     __syncwarp();
@@ -947,23 +960,29 @@ __device__ __forceinline__ float2 control_step(const DevCfg& c, const Net& net, 
     }
     // layer 3: a fixed pairwise tree over the hidden units -- leaves
     // w_2i h_2i + w_2i+1 h_2i+1 (one fma), then sums of neighbours -- so
-    // the value does not depend on how many units a lane holds
+    // the value does not depend on how many units a lane holds.  From the
+    // first exchange on, even lanes carry output 0's sums and odd lanes
+    // output 1's (each lane sends the other's), so a level is one shuffle and
+    // one sum and each lane evaluates one tanh; the last exchange gives every
+    // lane both outputs.
     float h2[U];
 #pragma unroll
-    for (int j = 0; j < U; ++j) h2[j] = tanh_r(acc2[j]);
+    for (int j = 0; j < U; ++j) h2[j] = acc2[j];
+#pragma unroll
+    for (int j = 0; j < U; j += 2) tanh_r2(h2[j], h2[j + 1]);
     float p0 = fmaf(net.w3[0][1], h2[1], __fmul_rn(net.w3[0][0], h2[0]));
     float p1 = fmaf(net.w3[1][1], h2[1], __fmul_rn(net.w3[1][0], h2[0]));
     if constexpr (U == 4) {
         p0 = __fadd_rn(p0, fmaf(net.w3[0][3], h2[3], __fmul_rn(net.w3[0][2], h2[2])));
         p1 = __fadd_rn(p1, fmaf(net.w3[1][3], h2[3], __fmul_rn(net.w3[1][2], h2[2])));
     }
+    const bool odd = gl & 1;
+    float ps = __fadd_rn(odd ? p1 : p0, __shfl_xor_sync(FULL, odd ? p0 : p1, 1));
 #pragma unroll
-    for (int off = 1; off < G; off <<= 1) {
-        p0 = __fadd_rn(p0, __shfl_xor_sync(FULL, p0, off));
-        p1 = __fadd_rn(p1, __shfl_xor_sync(FULL, p1, off));
-    }
-    const float ar0 = tanh_r(__fadd_rn(net.b3[0], p0));
-    const float ar1 = tanh_r(__fadd_rn(net.b3[1], p1));
+    for (int off = 2; off < G; off <<= 1) ps = __fadd_rn(ps, __shfl_xor_sync(FULL, ps, off));
+    const float ar = tanh_r(__fadd_rn(odd ? net.b3[1] : net.b3[0], ps));
+    const float ao = __shfl_xor_sync(FULL, ar, 1);
+    const float ar0 = odd ? ao : ar, ar1 = odd ? ar : ao;
     float a0 = fminf(fmaxf(ar0, __fsub_rn(ap0, c.r_rate)), __fadd_rn(ap0, c.r_rate));
     a0 = fminf(fmaxf(a0, -1.0f), 1.0f);
     const float a1 = ar1;
