@@ -174,6 +174,15 @@ struct LaneNet {
         }
     }
 
+    // layer 2's biases and layer 3's rows
+    struct Tail { float b2[U], w3[2][U]; };
+    __device__ __forceinline__ Tail tail() const {
+        Tail t;
+#pragma unroll
+        for (int j = 0; j < U; ++j) { t.b2[j] = b2[j]; t.w3[0][j] = w3[0][j]; t.w3[1][j] = w3[1][j]; }
+        return t;
+    }
+
     // nothing to fetch ahead of a step (TmemNet has)
     struct Ahead {};
     __device__ __forceinline__ Ahead fetch_ahead() const { return {}; }
@@ -297,14 +306,20 @@ struct LaneNet {
 // Why: a sample's weights decide how many samples an SM holds, and the
 // rollout step is a serial chain (layers, tanh, shuffle tree, Euler step), so
 // resident samples are what fills the pipes.
-template <int W_, int G_, int KT, int KS = 0>
+//
+// LEAN: b2 and W3's rows stay in 16 more columns, read once per step after
+// layer 2, and layer 2's columns come through one buffer: about 100 registers
+// a thread at four units a lane instead of 128, so 20 warps fit an SM.
+template <int W_, int G_, int KT, int KS = 0, bool LEAN = false>
 struct TmemNet {
     static constexpr int W = W_, G = G_;
     using S = Shape<W, G>;
     static constexpr int U = S::U;
     static constexpr int QC = 4 * U;              // columns of one input quad
-    static constexpr int COLS = QC * KT;          // TMEM columns of one warp
+    static constexpr int COLS = QC * KT + (LEAN ? 16 : 0);   // TMEM columns of one warp
+    static constexpr int TAIL = LEAN ? QC * KT : U * NIN;    // b1, b2 and W3's rows (staged there if not LEAN)
     static constexpr int QPR = 16 / QC;           // input quads per 16-column read
+    static_assert(!LEAN || U == 4, "four-unit columns");
     static_assert(KT % QPR == 0 && KT + KS == W / 4, "whole 16-column reads");
     static_assert(COLS >= (U == 2 ? 32 : 64), "the registers' parameters are staged through the columns");
     unsigned long long w1p[U][NIN / 2];
@@ -363,6 +378,11 @@ struct TmemNet {
             w3[1][j] = m[S::OFF_W3 + W + gl * U + j];
         }
         b3[0] = m[S::OFF_B3]; b3[1] = m[S::OFF_B3 + 1];
+        if constexpr (LEAN) {
+            tmem_st4(tm + TAIL + U, make_float4(b2[0], b2[1], b2[2], b2[3]));
+            tmem_st4(tm + TAIL + 2 * U, make_float4(w3[0][0], w3[0][1], w3[0][2], w3[0][3]));
+            tmem_st4(tm + TAIL + 3 * U, make_float4(w3[1][0], w3[1][1], w3[1][2], w3[1][3]));
+        }
         constexpr int B = 8;
         static_assert(U * (W / 4) % B == 0, "whole rounds");
 #pragma unroll 1
@@ -395,7 +415,7 @@ struct TmemNet {
 #pragma unroll 1
         for (int k = 0; k < 4; ++k) {
             const int off = k == 0 ? S::OFF_B1 : k == 1 ? S::OFF_B2 : k == 2 ? S::OFF_W3 : S::OFF_W3 + W;
-            put_units(src, off + gl * U, tm + U * NIN + k * U);
+            put_units(src, off + gl * U, tm + TAIL + k * U);
         }
         const float2 o = src.pair(S::OFF_B3);
         b3[0] = o.x; b3[1] = o.y;
@@ -404,7 +424,7 @@ struct TmemNet {
         Tmem16 a[U / 2], b;
 #pragma unroll
         for (int k = 0; k < U / 2; ++k) tmem_ld16(tm + 16 * k, a[k]);
-        tmem_ld16(tm + U * NIN, b);
+        tmem_ld16(tm + TAIL, b);
 #pragma unroll
         for (int k = 0; k < U / 2; ++k) tmem_wait_ld(a[k]);
         tmem_wait_ld(b);
@@ -424,6 +444,22 @@ struct TmemNet {
         tmem_wait_st();
     }
 
+    struct Tail { float b2[U], w3[2][U]; };
+    __device__ __forceinline__ Tail tail() const {
+        Tail t;
+        if constexpr (LEAN) {
+            Tmem16 b;
+            tmem_ld16(tm + TAIL, b);
+            tmem_wait_ld(b);
+#pragma unroll
+            for (int j = 0; j < U; ++j) { t.b2[j] = b.f(U + j); t.w3[0][j] = b.f(2 * U + j); t.w3[1][j] = b.f(3 * U + j); }
+        } else {
+#pragma unroll
+            for (int j = 0; j < U; ++j) { t.b2[j] = b2[j]; t.w3[0][j] = w3[0][j]; t.w3[1][j] = w3[1][j]; }
+        }
+        return t;
+    }
+
     // the first 16 columns, read while layer 1 runs
     struct Ahead { Tmem16 w; };
     __device__ __forceinline__ Ahead fetch_ahead() const {
@@ -436,13 +472,14 @@ struct TmemNet {
     // their way while these are multiplied
     __device__ __forceinline__ void layer2(const float4* hrow4, Ahead& f, unsigned long long (&p01)[U],
                                            unsigned long long (&p23)[U]) const {
-        Tmem16 buf[2];
+        Tmem16 buf[LEAN ? 1 : 2];
         buf[0] = f.w;
 #pragma unroll
         for (int c = 0; c < KT / QPR; ++c) {
-            Tmem16& w = buf[c & 1];
+            Tmem16& w = buf[LEAN ? 0 : c & 1];
+            if (LEAN && c > 0) tmem_ld16(tm + 16 * c, w);
             tmem_wait_ld(w);
-            if (c + 1 < KT / QPR) tmem_ld16(tm + 16 * (c + 1), buf[(c + 1) & 1]);
+            if (!LEAN && c + 1 < KT / QPR) tmem_ld16(tm + 16 * (c + 1), buf[(c + 1) & 1]);
 #pragma unroll
             for (int q = 0; q < QPR; ++q) {
                 const float4 hv = hrow4[QPR * c + q];
@@ -952,11 +989,12 @@ __device__ __forceinline__ float2 control_step(const DevCfg& c, const Net& net, 
     for (int j = 0; j < U; ++j) p01[j] = p23[j] = 0ull;
     net.layer2(reinterpret_cast<const float4*>(hrow), ahead, p01, p23);
     __syncwarp();
+    const typename Net::Tail tl = net.tail();
     float acc2[U];
 #pragma unroll
     for (int j = 0; j < U; ++j) {
         const float2 q01 = f2_unpack(p01[j]), q23 = f2_unpack(p23[j]);
-        acc2[j] = __fadd_rn(__fadd_rn(__fadd_rn(q01.x, q01.y), __fadd_rn(q23.x, q23.y)), net.b2[j]);
+        acc2[j] = __fadd_rn(__fadd_rn(__fadd_rn(q01.x, q01.y), __fadd_rn(q23.x, q23.y)), tl.b2[j]);
     }
     // layer 3: a fixed pairwise tree over the hidden units -- leaves
     // w_2i h_2i + w_2i+1 h_2i+1 (one fma), then sums of neighbours -- so
@@ -970,11 +1008,11 @@ __device__ __forceinline__ float2 control_step(const DevCfg& c, const Net& net, 
     for (int j = 0; j < U; ++j) h2[j] = acc2[j];
 #pragma unroll
     for (int j = 0; j < U; j += 2) tanh_r2(h2[j], h2[j + 1]);
-    float p0 = fmaf(net.w3[0][1], h2[1], __fmul_rn(net.w3[0][0], h2[0]));
-    float p1 = fmaf(net.w3[1][1], h2[1], __fmul_rn(net.w3[1][0], h2[0]));
+    float p0 = fmaf(tl.w3[0][1], h2[1], __fmul_rn(tl.w3[0][0], h2[0]));
+    float p1 = fmaf(tl.w3[1][1], h2[1], __fmul_rn(tl.w3[1][0], h2[0]));
     if constexpr (U == 4) {
-        p0 = __fadd_rn(p0, fmaf(net.w3[0][3], h2[3], __fmul_rn(net.w3[0][2], h2[2])));
-        p1 = __fadd_rn(p1, fmaf(net.w3[1][3], h2[3], __fmul_rn(net.w3[1][2], h2[2])));
+        p0 = __fadd_rn(p0, fmaf(tl.w3[0][3], h2[3], __fmul_rn(tl.w3[0][2], h2[2])));
+        p1 = __fadd_rn(p1, fmaf(tl.w3[1][3], h2[3], __fmul_rn(tl.w3[1][2], h2[2])));
     }
     const bool odd = gl & 1;
     float ps = __fadd_rn(odd ? p1 : p0, __shfl_xor_sync(FULL, odd ? p0 : p1, 1));
@@ -1375,10 +1413,10 @@ constexpr int tmem_block_bytes()
 }
 
 // Trajectories, one sample per group (as traj_kernel).
-template <int W, int G, int NW, int MINB, bool VAR, int KT, int KS>
+template <int W, int G, int NW, int MINB, bool VAR, int KT, int KS, bool LEAN>
 __global__ void __launch_bounds__(NW * 32, MINB) traj_tmem_kernel(const RolloutArgs a)
 {
-    using Net = TmemNet<W, G, KT, KS>;
+    using Net = TmemNet<W, G, KT, KS, LEAN>;
     static_assert(NW % 4 == 0 && tmem_cols<Net, NW>() * MINB <= 512, "the blocks of an SM fit its TMEM");
     extern __shared__ __align__(16) ulonglong2 w2_all[];
     __shared__ uint32_t tslot;
@@ -2091,10 +2129,10 @@ inline bool rollout_wide(const RolloutArgs& a, int block)
     return (a.N + block - 1) / block > a.sm_count * 7 / 8;
 }
 
-template <int W, int G, int NW, int MINB, bool VAR, int KT, int KS = 0>
+template <int W, int G, int NW, int MINB, bool VAR, int KT, int KS = 0, bool LEAN = false>
 cudaError_t launch_traj_tmem(const RolloutArgs& a, cudaStream_t stream)
 {
-    auto fn = traj_tmem_kernel<W, G, NW, MINB, VAR, KT, KS>;
+    auto fn = traj_tmem_kernel<W, G, NW, MINB, VAR, KT, KS, LEAN>;
     constexpr int B = NW * 32 / G, smem = tmem_block_bytes<W, G, NW, KS, 0>();
     cudaError_t e = ensure_smem(fn, smem);
     if (e != cudaSuccess) return e;

@@ -6,6 +6,11 @@
 //     sample, so the faster one where samples fill the SMs
 //   2 two units a lane, four samples a warp: more warps from the same
 //     samples and a shorter chain per step, so the faster one below
+//   1's samples in 20-warp blocks (LEAN) where they fill 20 warps per SM but
+//     not 16 (N in 16 .. 20 x 8 x SMs), a second wave otherwise: N = 20480,
+//     T = 200: 225 -> 190; N = 24320, T = 40: 81 -> 71.  In one wave of 16
+//     or in several the 16-warp shape is the faster (16384 samples, T = 40:
+//     56 / 61; 30000: 91 / 113).
 //   3, 4 every weight in registers <16, 8, 4, 4>
 // Measured on GB300 (trajectories, us; 1 / 2 / the earlier default in
 // registers): road N = 20480, T = 200: 223 / 248 / 280; course N = 16384,
@@ -17,6 +22,9 @@ namespace npp {
 template <bool VAR>
 static cudaError_t traj(const RolloutArgs& a, cudaStream_t s, bool wide)
 {
+    // samples that 16 warps per SM take in a wave and a bit, and 20 in one
+    const int per = 8 * a.sm_count;
+    if (wide && a.N > 16 * per && a.N <= 20 * per) return launch_traj_tmem<16, 4, 20, 1, VAR, 4, 0, true>(a, s);
     return wide ? launch_traj_tmem<16, 4, 4, 4, VAR, 4>(a, s) : launch_traj_tmem<16, 8, 4, 6, VAR, 4>(a, s);
 }
 
