@@ -11,13 +11,20 @@
 // (BF16, K-major, 128-byte swizzle).  The weight gradients read the
 // activations row-major as they are (MN-major operands), so nothing is
 // stored transposed.  Measured on GB300: training step at batch 8192 (all
-// launches) 187 -> 87 us; a forward pass of 300 rows with the encoding of
+// launches) 187 -> 75 us; a forward pass of 300 rows with the encoding of
 // their scenes 61 -> 33 us.
+//
+// In a training step each kernel starts while the one before it runs
+// (programmatic dependent launch), on the SMs that one leaves idle: the
+// backward pass fills 64 of 152 at batch 8192, and dW3 needs nothing of it.
+// A kernel lets the next one start only after its own wait, so what lies two
+// launches back is complete; see the waits.  A step so 87 -> 75 us.
 //
 // Every CTA: one TMA producer lane, one MMA-issuing lane, eight epilogue
 // warps (two per TMEM lane quarter, each half of the columns).  All waits
 // are bounded; on a timeout the CTA records an error, stops issuing, waits
 // (bounded) for its copies, frees its TMEM and returns.
+#include "npp_launch.cuh"
 #include "npp_mlp.cuh"
 #include "npp_tcgen05.cuh"
 
@@ -216,6 +223,7 @@ mlp_forward_kernel(const __grid_constant__ MlpForwardMaps maps, const MlpForward
                 : o >= MLP_NTH ? 0.0f : f.b3[i < 2 * MLP_HID + MLP_D3 / 2 ? o : MLP_NTH + o];
     }
     const uint32_t tmem = pipe_init(p);        // a block barrier: the biases are in
+    start_next();
     const int tiles = (f.n + TILE_M - 1) / TILE_M, units = tiles * f.groups, tpu = 4 / f.groups;
 
     if (warp == 0 && lane == 0) {
@@ -469,6 +477,8 @@ mlp_backward_kernel(const __grid_constant__ MlpBackwardMaps maps, const MlpBackw
     Pipe<BW_STAGES>& p = *reinterpret_cast<Pipe<BW_STAGES>*>(ring + BW_STAGES * BW_STAGE);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const uint32_t tmem = pipe_init(p);
+    wait_for_previous();                       // the forward pass
+    start_next();
     const int tiles = f.n / TILE_M;
     constexpr int NK = MLP_D3 / 64 + MLP_HID / 64;         // K blocks of the two products
 
@@ -611,10 +621,17 @@ mlp_grad_kernel(const __grid_constant__ MlpGradMaps maps, const MlpGrads f)
     };
 
     if (warp == 0 && lane == 0) {
+        // dW3's operands are the forward pass's, complete before the backward
+        // pass let this kernel start; the others wait for the backward pass
         int g = 0;
-        bool go = true;
+        bool go = true, waited = false;
         for (int u = blockIdx.x; u < units && go; u += gridDim.x) {
             const Unit x = unit(u);
+            if (x.k != 0 && !waited) {
+                wait_for_previous();
+                start_next();
+                waited = true;
+            }
             for (int kb = x.k0; kb < x.k1; ++kb) {
                 if (!(go = stage_free(p, g))) break;
                 const int s = g % GR_STAGES;
@@ -625,6 +642,10 @@ mlp_grad_kernel(const __grid_constant__ MlpGradMaps maps, const MlpGrads f)
                     tma_load_2d(st + A_BLOCK + c * 8192, &maps.b[x.k], c * 64, kb * 64, &p.full[s]);
                 ++g;
             }
+        }
+        if (!waited) {
+            wait_for_previous();
+            start_next();
         }
         p.flags[1] = g;
     } else if (warp == 1 && lane == 0) {
@@ -728,8 +749,7 @@ cudaError_t launch_mlp_backward(const MlpBackwardMaps& m, const MlpBackward& b, 
 {
     cudaError_t e = smem_opt(mlp_backward_kernel, BW_SMEM);
     if (e != cudaSuccess) return e;
-    mlp_backward_kernel<<<std::min(b.n / TILE_M, mlp_sm_count()), THREADS, BW_SMEM, s>>>(m, b);
-    return cudaGetLastError();
+    return launch_dependent(mlp_backward_kernel, std::min(b.n / TILE_M, mlp_sm_count()), THREADS, BW_SMEM, s, m, b);
 }
 
 cudaError_t launch_mlp_grads(const MlpGradMaps& m, const MlpGrads& g, cudaStream_t s)
@@ -737,8 +757,7 @@ cudaError_t launch_mlp_grads(const MlpGradMaps& m, const MlpGrads& g, cudaStream
     cudaError_t e = smem_opt(mlp_grad_kernel, GR_SMEM);
     if (e != cudaSuccess) return e;
     const int units = gr_tiles(0) * g.splits[0] + gr_tiles(1) * g.splits[1] + gr_tiles(2) * g.splits[2];
-    mlp_grad_kernel<<<std::min(units, mlp_sm_count()), THREADS, GR_SMEM, s>>>(m, g);
-    return cudaGetLastError();
+    return launch_dependent(mlp_grad_kernel, std::min(units, mlp_sm_count()), THREADS, GR_SMEM, s, m, g);
 }
 
 }  // namespace npp

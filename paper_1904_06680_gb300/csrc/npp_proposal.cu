@@ -27,8 +27,9 @@
 
 #include "../../include/npp_proposal.h"
 #include "npp_gemm.cuh"
-#include "npp_mlp.cuh"
 #include "npp_internal.h"
+#include "npp_launch.cuh"
+#include "npp_mlp.cuh"
 
 using namespace npp;
 
@@ -171,7 +172,10 @@ __device__ __forceinline__ float adam_step(const Adam& a, float g, float w, floa
 // Blocks 0 .. UPD_B - 1: UPD_COLS biases each, the longest; then four weights
 // a thread; the last block the loss.
 // Bound: L2 reads of the partials (40 MB at batch 8192) and of the batch's
-// gradients for the bias sums.  One launch instead of four (split sum, bias
+// gradients for the bias sums.  The weight gradients' kernel lets this one
+// start once the backward pass is complete, so the biases and the loss, which
+// need no more than that, are done while it runs; the weights wait for it.
+// One launch instead of four (split sum, bias
 // gradients, Adam, BF16 copies: 36 us of a 187 us step at batch 8192).
 struct UpdateArgs {
     float *w, *m, *v, *g;
@@ -244,18 +248,19 @@ __global__ void __launch_bounds__(UPD_THREADS) update_kernel(const UpdateArgs a)
         int i = (blockIdx.x - UPD_B) * UPD_THREADS + tid;
         const int k = i < n1 ? 0 : i < n1 + n2 ? 1 : 2;
         i -= k == 0 ? 0 : k == 1 ? n1 : n1 + n2;
+        wait_for_previous();                     // the weight gradients
         const size_t size = k == 0 ? n1 : k == 1 ? n2 : n3;
         const size_t off = k == 0 ? OFF_W1 : k == 1 ? OFF_W2 : OFF_W3;
         const float4* p = reinterpret_cast<const float4*>(a.part[k]) + i;
         const int S = a.splits[k];
         float4 g = make_float4(0.f, 0.f, 0.f, 0.f);
         int z = 0;
-        for (; z + 8 <= S; z += 8) {             // eight loads in flight, added in slice order
-            float4 t[8];
+        for (; z + 16 <= S; z += 16) {           // sixteen loads in flight, added in slice order
+            float4 t[16];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) t[u] = p[(size_t)(z + u) * size];
+            for (int u = 0; u < 16; ++u) t[u] = p[(size_t)(z + u) * size];
 #pragma unroll
-            for (int u = 0; u < 8; ++u) { g.x += t[u].x; g.y += t[u].y; g.z += t[u].z; g.w += t[u].w; }
+            for (int u = 0; u < 16; ++u) { g.x += t[u].x; g.y += t[u].y; g.z += t[u].z; g.w += t[u].w; }
         }
         for (; z < S; ++z) {
             const float4 t = p[(size_t)z * size];
@@ -583,8 +588,7 @@ npp_status npp_proposal_train_step(npp_proposal* P, const float* x_dev, const fl
         u.adam = { lr, P->cfg.beta1, P->cfg.beta2, P->cfg.eps,
                    (float)(1.0 - std::pow((double)P->cfg.beta1, P->t)),
                    (float)(1.0 - std::pow((double)P->cfg.beta2, P->t)) };
-        update_kernel<<<UPD_B + UPD_W + 1, UPD_THREADS, 0, s>>>(u);
-        e = cudaGetLastError();
+        e = launch_dependent(update_kernel, UPD_B + UPD_W + 1, UPD_THREADS, 0, s, u);
     }
     if (e != cudaSuccess) return perr(NPP_CUDA_ERROR, std::string("proposal train step: ") + cudaGetErrorString(e));
     return NPP_OK;
