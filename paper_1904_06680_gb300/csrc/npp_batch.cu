@@ -123,7 +123,7 @@ __device__ __forceinline__ int sort_key(float px, float py, float vx, float vy)
 
 __global__ void __launch_bounds__(SORT_THREADS) batch_prologue_kernel(const BatchArgs b)
 {
-    extern __shared__ int cnt[];                       // [SORT_KEYS]
+    extern __shared__ __align__(16) int cnt[];         // [SORT_KEYS]
     __shared__ int run_tot[SORT_THREADS];
     const SceneDev& s = b.scenes[blockIdx.x];
     const int M = s.M;
@@ -504,8 +504,8 @@ __global__ void __launch_bounds__(S * 32) batch_collide_kernel(const BatchArgs b
 // Grids of every scene and horizon step: block b -> (scene, h).
 __global__ void __launch_bounds__(1024) batch_bin_build_kernel(const BatchArgs b)
 {
-    extern __shared__ int cnt[];             // [BIN_NCELL]
-    __shared__ int run_tot[1024];
+    extern __shared__ __align__(16) int cnt[];       // [BIN_NCELL]
+    __shared__ int run_tot[32];
     const long long blk = blockIdx.x;
     const int si = find_slot(b.bstep_prefix, b.S, blk);
     const SceneDev& s = b.scenes[si];

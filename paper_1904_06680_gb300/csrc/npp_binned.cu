@@ -30,8 +30,8 @@ constexpr int BIN_THREADS = 1024;
 __global__ void __launch_bounds__(BIN_THREADS) bin_build_kernel(const RolloutArgs a, BinView g, int* __restrict__ cell_start,
                                                                 float2* __restrict__ binned)
 {
-    extern __shared__ int cnt[];             // [BIN_NCELL]
-    __shared__ int run_tot[BIN_THREADS];
+    extern __shared__ __align__(16) int cnt[];       // [BIN_NCELL]
+    __shared__ int run_tot[BIN_THREADS / 32];
     const int h = blockIdx.x;
     if (h == 0 && threadIdx.x == 0) {
         // start of the plan step's minimum and sample queue
