@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(1024) batch_bin_build_kernel(const BatchArgs b
     const int h = (int)(blk - __ldg(b.bstep_prefix + si));
     float sn, cs;
     sincosf(s.phi0, &sn, &cs);
-    build_step_bins<1024>(b.obs + s.obs_off, s.M, s.x0, s.y0, sn, cs, (float)h * b.c.Ts, b.grid,
+    build_step_bins<1024, int>(b.obs + s.obs_off, s.M, s.x0, s.y0, sn, cs, (float)h * b.c.Ts, b.grid,
                           b.bin_cs + s.bin_off + (size_t)h * BIN_CS_STRIDE, b.bin_pts + s.bpts_off + (size_t)h * s.M,
                           cnt, run_tot);
 }

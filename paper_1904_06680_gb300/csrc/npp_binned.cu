@@ -47,8 +47,13 @@ __global__ void __launch_bounds__(BIN_THREADS) bin_build_kernel(const RolloutArg
     const StepIn si = step_in(a);
     float s0, c0;
     sincosf(si.phi0, &s0, &c0);
-    build_step_bins<BIN_THREADS>(a.obs, a.M, si.x0, si.y0, s0, c0, (float)h * a.c.Ts, g,
-                                 cell_start + (size_t)h * BIN_CS_STRIDE, binned + (size_t)h * a.M, cnt, run_tot);
+    int* cs = cell_start + (size_t)h * BIN_CS_STRIDE;
+    float2* out = binned + (size_t)h * a.M;
+    if (a.first)
+        build_step_bins<BIN_THREADS>(a.obs, a.M, si.x0, si.y0, s0, c0, (float)h * a.c.Ts, g,
+                                     reinterpret_cast<unsigned short*>(cs), out, cnt, run_tot);
+    else
+        build_step_bins<BIN_THREADS>(a.obs, a.M, si.x0, si.y0, s0, c0, (float)h * a.c.Ts, g, cs, out, cnt, run_tot);
 }
 
 // One warp per sample over its stored states (each step's inequality rows
@@ -180,8 +185,23 @@ __global__ void __launch_bounds__(BINNED_WARPS * 32, 5) collide_binned_kernel(co
 // against the warp-per-sample kernel): course (16384 x 41 states, 2000
 // points) 42 / 54, 5003 x 61 states 25 / 32, 8192 x 41 (855 points) 21 / 27,
 // large (65536 x 101, 8192 points) 207 / 306; a handful of samples 11 / 7.
-// (With polygons, whose test is long, lanes diverge: 316 / 134.)
+// (With polygons, whose test is long, lanes diverge: 316 / 134.)  The build
+// writes this check's cell starts as 16 bits, and they and the points come by
+// asynchronous copies, all in flight (32-bit starts through registers: plan
+// steps of 2048 samples, T = 40, 41.1 us, now 39.0; 3000 x 201 states 118.0,
+// now 114.7).
 constexpr int GRID_THREADS = 512;
+static_assert(BIN_NCELL * 2 % (16 * GRID_THREADS) == 0, "whole rounds of 16-byte copies");
+
+// BYTES (8 or 16) from global into shared memory without a register between
+template <int BYTES>
+__device__ __forceinline__ void copy_async(void* dst, const void* src)
+{
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
+    if constexpr (BYTES == 16) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+    else asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 constexpr int GRID_CS_BYTES = (BIN_NCELL + 8) * 2;
 
 __global__ void __launch_bounds__(GRID_THREADS, 2) collide_grid_kernel(const RolloutArgs a, int chunk)
@@ -197,15 +217,17 @@ __global__ void __launch_bounds__(GRID_THREADS, 2) collide_grid_kernel(const Rol
     const BinView& g = a.bins;
     start_next();
     {
-        const int4* src = reinterpret_cast<const int4*>(g.cell_start + (size_t)h * BIN_CS_STRIDE);
-        ushort4* dst = reinterpret_cast<ushort4*>(cs);
-        for (int i = tid; i < BIN_NCELL / 4; i += GRID_THREADS) {
-            const int4 v = src[i];
-            dst[i] = make_ushort4((unsigned short)v.x, (unsigned short)v.y, (unsigned short)v.z, (unsigned short)v.w);
+        // every copy in flight at once
+        const char* src = reinterpret_cast<const char*>(g.cell_start + (size_t)h * BIN_CS_STRIDE);
+#pragma unroll
+        for (int i = 0; i < BIN_NCELL * 2 / 16 / GRID_THREADS; ++i) {
+            const int o = (i * GRID_THREADS + tid) * 16;
+            copy_async<16>(smem_raw + o, src + o);
         }
         const float2* p = g.pts + (size_t)h * M;
-        for (int i = tid; i < M; i += GRID_THREADS) pts[i] = p[i];
+        for (int i = tid; i < M; i += GRID_THREADS) copy_async<8>(pts + i, p + i);
         if (tid == 0) cs[BIN_NCELL] = (unsigned short)M;
+        copy_async_wait();
     }
     __syncthreads();
     unsigned ntest = 0, nstate = 0;

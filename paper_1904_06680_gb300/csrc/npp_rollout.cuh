@@ -754,14 +754,15 @@ struct PolyTest {
 // The grid of one horizon step (time tau) built by one block of THREADS
 // threads: counting sort of the extrapolated EV-frame points by cell (counts
 // in shared memory cnt[BIN_NCELL], exclusive scan, scatter).  Writes the
-// step's cell-start table cs[BIN_NCELL + 1] and the sorted points out[M].
+// step's cell-start table cs[BIN_NCELL + 1] (CS: 32 bits, or 16 for the check
+// that copies it into shared memory) and the sorted points out[M].
 // Bound: latency of the points' two reads and the barriers.  The scan takes
 // consecutive fours across a warp: a thread scanning a run of 16 cells for
 // itself met 16-way bank conflicts in two passes.  GB300, 41 steps of 2000
 // points 12.5 -> 7 us, 101 of 8192 22 -> 11.
-template <int THREADS>
+template <int THREADS, typename CS>
 __device__ __forceinline__ void build_step_bins(const float4* __restrict__ obs, int M, float x0, float y0, float s0,
-                                                float c0, float tau, const BinView& g, int* __restrict__ cs,
+                                                float c0, float tau, const BinView& g, CS* __restrict__ cs,
                                                 float2* __restrict__ out, int* cnt, int* run_tot)
 {
     // the cells by fours (cnt and cs are 16-byte aligned): a warp owns CELLS
@@ -803,14 +804,17 @@ __device__ __forceinline__ void build_step_bins(const float4* __restrict__ obs, 
     if (lane == 0) run_tot[warp] = run;
     __syncthreads();
     const int before = __reduce_add_sync(FULL, lane < warp ? run_tot[lane] : 0);
-    int4* out4 = reinterpret_cast<int4*>(cs + warp * CELLS) + lane;
 #pragma unroll
     for (int r = 0; r < ROUNDS; ++r) {
         const int4 q = make_int4(v[r].x + before, v[r].y + before, v[r].z + before, v[r].w + before);
         mine[32 * r] = q;
-        out4[32 * r] = q;
+        if constexpr (sizeof(CS) == 4)
+            reinterpret_cast<int4*>(cs + warp * CELLS)[lane + 32 * r] = q;
+        else
+            reinterpret_cast<ushort4*>(cs + warp * CELLS)[lane + 32 * r] =
+                make_ushort4((unsigned short)q.x, (unsigned short)q.y, (unsigned short)q.z, (unsigned short)q.w);
     }
-    if (threadIdx.x == 0) cs[BIN_NCELL] = M;
+    if (threadIdx.x == 0) cs[BIN_NCELL] = (CS)M;
     __syncthreads();
     // scatter (order within a cell is arbitrary; the test is an OR)
     for (int j = threadIdx.x; j < M; j += THREADS) {
