@@ -342,11 +342,16 @@ int collide_grid_points() { return (100 * 1024 - GRID_CS_BYTES) / 8; }
 
 cudaError_t launch_collide_grid(const RolloutArgs& a, cudaStream_t s)
 {
-    // chunks of the samples so that the (chunk, step) blocks are about three
-    // per SM: fewer would leave SMs idle, more would copy the grids oftener
+    // chunks of the samples: (chunk, step) blocks about three per SM, each of
+    // two states a thread at most -- fewer blocks would leave SMs idle, more
+    // would copy the grids oftener, and longer chunks leave the last blocks
+    // running alone (four or ten states a thread: 20000 x 101 states 227 us
+    // the plan step, now 185; 40000 x 61 242, now 217; one: 8192 x 41 54, not
+    // 52)
     const int want = max(1, 3 * a.sm_count / (a.T + 1));
-    int chunk = (a.N + want - 1) / want;
-    chunk = (chunk + GRID_THREADS - 1) / GRID_THREADS * GRID_THREADS;
+    const auto whole = [](int n) { return (n + GRID_THREADS - 1) / GRID_THREADS * GRID_THREADS; };
+    const int chunk = max(min(whole((a.N + want - 1) / want), 2 * GRID_THREADS),
+                          whole((a.N + GRID_MAX_CHUNKS - 1) / GRID_MAX_CHUNKS));
     const dim3 grid((a.N + chunk - 1) / chunk, a.T + 1);
     const int smem = GRID_CS_BYTES + a.M * (int)sizeof(float2);
     const cudaError_t e = cudaFuncSetAttribute(collide_grid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
