@@ -524,9 +524,9 @@ def run_npp(args):
                               {16: "<16,8,4,6,%d,4,0>", 32: "<32,16,4,5,%d,8,0>", 64: "<64,32,4,4,%d,16,0>"})[W] % var
     if fused:
         # [0] grid build, [1] the trajectory kernel with the windowed check
-        full = N >= 16 * sms
+        full = N >= 160 * sms
         fshape = {16: "_kernel<16,8,4,4,%d,0,16,4>", 32: "_kernel<32,16,4,5,%d,5,8,4>",
-                  64: "_tmem_kernel<64,32,20,1,%d,12,4,8,4>" if full else "_tmem_kernel<64,32,4,4,%d,16,0,8,4>"}[W] % var
+                  64: "_tmem_kernel<64,32,24,1,%d,10,6,8,4>" if full else "_tmem_kernel<64,32,4,4,%d,16,0,8,4>"}[W] % var
         fname = "fused" + fshape
         fps = res["fma_t"] / (collide_ms / 1e3)
         rolled = res["rolled"] if res["rolled"] > 0 else float(N) * T * K

@@ -429,7 +429,7 @@ npp_status npp_plan_batch(npp_batch* B, const float* obs_dev, const npp_batch_ou
  * item's live samples are skipped; "slices" = warps that share one 8-sample
  * brute-force item, each on an interleaved share of the point tiles (2, 4 or
  * 8; default 4); "traj_warps" = warps per trajectory block (4 or 8; default 8;
- * with the binned check of width 64, 8 stands for one block of 20 per SM).
+ * with the binned check of width 64, 8 stands for one block of 24 per SM).
  * Synchronous (re-plans the work lists). */
 npp_status npp_batch_set_option(npp_batch* B, const char* name, int32_t value);
 

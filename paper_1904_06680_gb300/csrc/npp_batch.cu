@@ -717,7 +717,7 @@ struct npp_batch {
     long long total_pairs, total_rows, total_samples;
     int grid_collide;
     int slices;              // warps per collision item (point slices): 2, 4, 8
-    int traj_warps;          // warps per trajectory block: 4, 8 (20 at width 64 with its check)
+    int traj_warps;          // warps per trajectory block: 4, 8 (24 at width 64 with its check)
     int smem_optin;
 };
 
@@ -865,7 +865,7 @@ cudaError_t launch_batch_traj_w(npp_batch* B, const BatchArgs& b, int wi, cudaSt
     default:
         if (!B->binned) return launch_traj_items<64, 16, 4, 3, VAR, 8, 8, false>(B, b, 2, s);
         if (NW == 4) return launch_traj_items<64, 32, 4, 4, VAR, 16, 0, true>(B, b, 2, s);
-        return launch_traj_items<64, 32, 20, 1, VAR, 12, 4, true>(B, b, 2, s);
+        return launch_traj_items<64, 32, 24, 1, VAR, 10, 6, true>(B, b, 2, s);
     }
 }
 

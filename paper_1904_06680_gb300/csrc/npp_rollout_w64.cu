@@ -31,25 +31,27 @@ cudaError_t launch_traj_w64(const RolloutArgs& a, cudaStream_t s, int variant)
 
 // Trajectories with the windowed binned check (template arguments after the
 // trajectory kernel's: window of states, candidates loaded ahead per lane).
-// Default: 20 warps per SM in one block, 12 of 16 W2 quads in tensor memory
-// and 4 in shared memory, windows of 8 states; for samples that do not fill
-// those blocks (16 per SM), four-warp blocks with W2 in tensor memory.
-// Measured on GB300 at N = 65536, T = 100, M = 8192 (us): 1993; 16 warps per
-// SM 2018, 24 (10 quads in tensor memory) 1989; shape 3, the earlier default
-// in registers and shared memory (one sample per block), 2458.  (Windows of 4
-// states take 1940, but the library's work counters are defined by windows of
-// 8.)  At N = 2000, T = 50: four-warp blocks 85,
-// 20-warp blocks 95, shape 3 85.
+// Default: 24 warps per SM in one block, 10 of 16 W2 quads in tensor memory
+// and 6 in shared memory, windows of 8 states; below 160 samples per SM
+// four-warp blocks, 16 warps per SM, with all of W2 in tensor memory: a
+// sample runs through faster, which counts until the queue is long.
+// Measured on GB300 (us): N = 65536, T = 100, M = 8192: 16 warps per SM 2018, 20
+// (12 quads) 1993, 24 1976; shape 3, the earlier default in registers and
+// shared memory (one sample per block), 2458; two samples a warp, 12 warps,
+// 2350.  Plan steps with 24 / 16 warps, T = 50, M = 4000: N = 2432 125 / 102,
+// 4800 173 / 154, 9000 244 / 235, 24000 529 / 528, 48000 992 / 1001.
+// (Windows of 4 states take 3 % less, but the library's work counters are
+// defined by windows of 8.)
 template <bool VAR>
 static cudaError_t fused(const RolloutArgs& a, cudaStream_t s, bool full)
 {
-    return full ? launch_fused_tmem<64, 32, 20, 1, VAR, 12, 4, 8, 4>(a, s)
+    return full ? launch_fused_tmem<64, 32, 24, 1, VAR, 10, 6, 8, 4>(a, s)
                 : launch_fused_tmem<64, 32, 4, 4, VAR, 16, 0, 8, 4>(a, s);
 }
 
 cudaError_t launch_fused_w64(const RolloutArgs& a, cudaStream_t s, int variant)
 {
-    const bool full = variant == 1 || (variant != 2 && a.N >= 16 * a.sm_count);
+    const bool full = variant == 1 || (variant != 2 && a.N >= 160 * a.sm_count);
     if (uses_variants(a.c)) return fused<true>(a, s, full);
     return variant >= 3 ? launch_fused<64, 32, 1, 16, false, 12, 8, 4>(a, s) : fused<false>(a, s, full);
 }
