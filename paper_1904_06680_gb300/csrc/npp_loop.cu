@@ -113,9 +113,8 @@ __device__ __forceinline__ bool reached(const Pose& v, const float* eps, const f
 {
     double dxi, deta;
     ev_of(v, g.x, g.y, dxi, deta);
-    const double dphi = remainder((double)g.z - v.pphi, 2.0 * M_PI);
-    return fabs(dxi) <= eps[0] && fabs(deta) <= eps[1] && fabs(dphi) <= eps[2] &&
-           fabs((double)g.w - v.pv) <= eps[3];
+    if (!(fabs(dxi) <= eps[0] && fabs(deta) <= eps[1])) return false;
+    return fabs(remainder((double)g.z - v.pphi, 2.0 * M_PI)) <= eps[2] && fabs((double)g.w - v.pv) <= eps[3];
 }
 
 // the last setpoint from idx on, up to stop, that the range field holds
@@ -244,14 +243,22 @@ __device__ __forceinline__ void advance_vehicle(LoopDev* d, const float* control
     const double L = pc.lf + pc.lr;
     const double delta = pc.delta_max * a0;
     const double u = pc.u_min + 0.5 * (a1 + 1.0) * (pc.u_max - pc.u_min);
-    const double beta = atan(pc.lr * tan(delta) / L);
+    // one cosine and one sine for the three angles, on lanes 0, 1 and 2 (the
+    // step is a chain of FP64 calls: seven of them one after another took 4 us
+    // more)
+    const double td = tan(delta);
+    const double beta = atan(pc.lr * td / L);
     Pose p;
-    p.px = x + pc.Ts * v * cos(ph + beta) / cos(beta);
-    p.py = y + pc.Ts * v * sin(ph + beta) / cos(beta);
-    p.pphi = ph + pc.Ts * v * tan(delta) / L;
+    p.pphi = ph + pc.Ts * v * td / L;
+    const double ang = lane == 1 ? beta : lane == 2 ? p.pphi : ph + beta;
+    const double ca = cos(ang), sa = sin(ang);
+    p.c = __shfl_sync(FULL, ca, 2);
+    p.s = __shfl_sync(FULL, sa, 2);
+    const double along = __shfl_sync(FULL, ca, 0), across = __shfl_sync(FULL, sa, 0);
+    const double move = pc.Ts * v * ((lane & 1) ? across : along) / __shfl_sync(FULL, ca, 1);
+    p.px = x + __shfl_sync(FULL, move, 0);
+    p.py = y + __shfl_sync(FULL, move, 1);
     p.pv = v + pc.Ts * u;
-    p.c = cos(p.pphi);
-    p.s = sin(p.pphi);
     if (d->mission) {
         mission_update(d, p, wps);
     } else if (lane == 0 && !d->done && reached(p, d->eps, wps[d->waypoint])) {
