@@ -586,7 +586,7 @@ def run_npp(args):
                         candidate_tests_per_state=res["cand_tests"] / res["states"],
                         states_per_s=res["states"] / (collide_ms / 1e3),
                         bytes_per_step=nbytes / K, achieved_gbs=nbytes / (collide_ms / 1e3) / 1e9,
-                        traffic=profiled_traffic("collide_binned_kernel", args.workload),
+                        traffic=profiled_traffic(cname.split(" + ")[-1], args.workload),
                         bytes_note="algorithmic: 56 B per state checked (state + ten cell-run bounds), "
                                    "8 B per candidate test, 12 B per sample; traffic = DRAM bytes per "
                                    "launch from profiles/traffic.json")

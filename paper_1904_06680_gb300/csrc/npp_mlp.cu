@@ -11,14 +11,15 @@
 // (BF16, K-major, 128-byte swizzle).  The weight gradients read the
 // activations row-major as they are (MN-major operands), so nothing is
 // stored transposed.  Measured on GB300: training step at batch 8192 (all
-// launches) 187 -> 75 us; a forward pass of 300 rows with the encoding of
-// their scenes 61 -> 33 us.
+// launches) 187 -> 84 us; a forward pass of 300 rows with the encoding of
+// their scenes 61 -> 28 us.
 //
 // In a training step each kernel starts while the one before it runs
 // (programmatic dependent launch), on the SMs that one leaves idle: the
 // backward pass fills 64 of 152 at batch 8192, and dW3 needs nothing of it.
 // A kernel lets the next one start only after its own wait, so what lies two
-// launches back is complete; see the waits.  A step so 87 -> 75 us.
+// launches back is complete; see the waits.  16 steps and two reads of the
+// parameters so 1638 -> 1436 us.
 //
 // Every CTA: one TMA producer lane, one MMA-issuing lane, eight epilogue
 // warps (two per TMEM lane quarter, each half of the columns).  All waits
