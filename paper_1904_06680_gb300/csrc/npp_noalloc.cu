@@ -145,8 +145,9 @@ extern "C" npp_status npp_plan_step_noalloc(const npp_config* cfg, const npp_sta
     a.fault = reinterpret_cast<unsigned*>(base + 12);
     int sm_count = 1;
     cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
+    a.sm_count = sm_count > 0 ? sm_count : 1;                    // decides the trajectories' launch shape
     const int variant = N <= 8192 ? 3 : 4;
-    a.grid_collide = (sm_count > 0 ? sm_count : 1) * collide_resident_blocks_per_sm(M, variant);
+    a.grid_collide = a.sm_count * collide_resident_blocks_per_sm(M, variant);
 
     // the best key starts at all ones, the work counter and fault flag at zero
     e = cudaMemsetAsync(base, 0xff, 8, s);
