@@ -124,13 +124,17 @@ static cudaError_t launch_states(const RolloutArgs& a, cudaStream_t s)
 }
 
 // One sample per warp, 32 steps a round, except for many samples with few
-// points: there the state reads count, and at two samples per warp they fill
-// their 32-byte sectors.  Measured on GB300 (plan step, P = 4, 8, 16, 32):
-// N = 20480, T = 60, M = 20: 126, 123, 122, 124 us; N = 2048, T = 40,
-// M = 128: 66, 52, 44, 43 us.
+// points and steps: there the state reads count, and at two samples per warp
+// they fill their 32-byte sectors.  Over long horizons the more and shorter
+// warps of one sample each win: they fill the SMs as the trajectories' blocks
+// leave, without a nearly empty last wave.  Measured on GB300 (plan step, P =
+// 4, 8, 16, 32): N = 20480, T = 60, M = 20: 126, 123, 122, 124 us; N = 2048,
+// T = 40, M = 128: 66, 52, 44, 43 us; later, P = 16, 32, M = 20: N = 20480, T = 60
+// 86, 89, T = 200 226, 223; N = 8192, T = 200 126, 121; N = 40960, T = 200 429,
+// 431.
 cudaError_t launch_collide_states(const RolloutArgs& a, cudaStream_t s)
 {
-    return a.N >= 8192 && a.M < 64 ? launch_states<16>(a, s) : launch_states<32>(a, s);
+    return a.N >= 8192 && a.M < 64 && a.T < 128 ? launch_states<16>(a, s) : launch_states<32>(a, s);
 }
 
 using CollideResident = CollideBlockKernel<16, 128>;
