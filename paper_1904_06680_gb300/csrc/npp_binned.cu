@@ -354,7 +354,10 @@ cudaError_t launch_collide_grid(const RolloutArgs& a, cudaStream_t s)
                           whole((a.N + GRID_MAX_CHUNKS - 1) / GRID_MAX_CHUNKS));
     const dim3 grid((a.N + chunk - 1) / chunk, a.T + 1);
     const int smem = GRID_CS_BYTES + a.M * (int)sizeof(float2);
-    const cudaError_t e = cudaFuncSetAttribute(collide_grid_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    // the setting belongs to the kernel and the device, whichever thread or
+    // handle launches: always the largest size, never this call's (another
+    // thread's larger launch between this and its own setting would fail)
+    const cudaError_t e = ensure_smem(collide_grid_kernel, GRID_CS_BYTES + collide_grid_points() * (int)sizeof(float2));
     if (e != cudaSuccess) return e;
     collide_grid_kernel<<<grid, GRID_THREADS, smem, s>>>(a, chunk);
     return cudaGetLastError();
