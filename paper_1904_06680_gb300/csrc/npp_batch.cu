@@ -713,12 +713,12 @@ struct npp_batch {
     unsigned long long* d_keys;
     unsigned* d_counters;
     int resident_pairs;
+    int most_pairs;          // that fit in shared memory, whatever the batch
     int max_pairs;
     long long total_pairs, total_rows, total_samples;
     int grid_collide;
     int slices;              // warps per collision item (point slices): 2, 4, 8
     int traj_warps;          // warps per trajectory block: 4, 8 (24 at width 64 with its check)
-    int smem_optin;
 };
 
 namespace {
@@ -782,7 +782,7 @@ template <int S>
 cudaError_t collide_grid(npp_batch* B, int* grid)
 {
     const int smem = B->resident_pairs * 32 + BatchCollide<S>::fixed_bytes();
-    cudaError_t e = ensure_smem(batch_collide_kernel<S>, smem);
+    cudaError_t e = ensure_smem(batch_collide_kernel<S>, B->most_pairs * 32 + BatchCollide<S>::fixed_bytes());
     int nb = 0;
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, batch_collide_kernel<S>,
@@ -920,10 +920,8 @@ npp_status npp_batch_create(npp_handle* h, const npp_scene* scenes, int32_t S, n
     B->max_pairs = max_pairs;
     int smem_optin = 0;
     cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-    const int cap = (smem_optin - BatchCollide<MAX_SLICES>::fixed_bytes()) / 32;
-    B->resident_pairs = std::min(max_pairs, cap);
-
-    B->smem_optin = smem_optin;
+    B->most_pairs = (smem_optin - BatchCollide<MAX_SLICES>::fixed_bytes()) / 32;
+    B->resident_pairs = std::min(max_pairs, B->most_pairs);
     B->slices = 4;
     B->traj_warps = 8;
     B->binned = 1;

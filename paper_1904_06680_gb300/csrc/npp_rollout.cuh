@@ -2097,12 +2097,26 @@ __global__ void __launch_bounds__(P * S * 32, MINB) collide_slice_kernel(const R
 // ------------------------------------------------------------------ launchers
 // opt in to more than 48 KB of dynamic shared memory for kernel fn (a host
 // call; repeated on every launch that needs it, since the setting is per
-// function and per device)
+// function and per device).  `most` is the largest size any call asks of fn,
+// never one call's own: the setting is shared, and a smaller one would make
+// another thread's launch, or a later one of another batch, fail.
 template <typename KernelFn>
-inline cudaError_t ensure_smem(KernelFn fn, int smem)
+inline cudaError_t ensure_smem(KernelFn fn, int most)
+{
+    if (most <= 48 * 1024) return cudaSuccess;
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+}
+
+// the same for a collision kernel (shape K) whose call holds its points in
+// `smem` bytes: all that fit the current device
+template <typename K, typename KernelFn>
+inline cudaError_t ensure_points_smem(KernelFn fn, int smem)
 {
     if (smem <= 48 * 1024) return cudaSuccess;
-    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    int dev = 0, optin = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    return e == cudaSuccess ? ensure_smem(fn, K::smem_bytes(collide_max_points(optin))) : e;
 }
 
 // Whether a configuration turns on a rollout variant (VAR kernels).
@@ -2173,7 +2187,7 @@ cudaError_t launch_collide_block(const RolloutArgs& a, cudaStream_t stream)
 {
     using K = CollideBlockKernel<NW, SBMAX>;
     const int smem = K::smem_bytes(a.M);
-    cudaError_t e = ensure_smem(collide_block_kernel<NW, SBMAX, MINB>, smem);
+    cudaError_t e = ensure_points_smem<K>(collide_block_kernel<NW, SBMAX, MINB>, smem);
     if (e != cudaSuccess) return e;
     const int grid = max(1, min((a.N + 7) / 8, a.grid_collide));
     collide_block_kernel<NW, SBMAX, MINB><<<grid, K::THREADS, smem, stream>>>(a);
@@ -2186,7 +2200,7 @@ int collide_block_blocks_per_sm(int M)
     using K = CollideBlockKernel<NW, SBMAX>;
     int nb = 0;
     const int smem = K::smem_bytes(M);
-    if (ensure_smem(collide_block_kernel<NW, SBMAX, MINB>, smem) != cudaSuccess) return 1;
+    if (ensure_points_smem<K>(collide_block_kernel<NW, SBMAX, MINB>, smem) != cudaSuccess) return 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, collide_block_kernel<NW, SBMAX, MINB>,
                                                   K::THREADS, smem);
     return nb > 0 ? nb : 1;
@@ -2197,7 +2211,7 @@ cudaError_t launch_collide_warp(const RolloutArgs& a, cudaStream_t stream)
 {
     using K = CollideWarpKernel<NW>;
     const int smem = K::smem_bytes(a.M);
-    cudaError_t e = ensure_smem(collide_warp_kernel<NW, MINB>, smem);
+    cudaError_t e = ensure_points_smem<K>(collide_warp_kernel<NW, MINB>, smem);
     if (e != cudaSuccess) return e;
     const int nwarps_needed = (a.N + 7) / 8;
     const int grid = min((nwarps_needed + NW - 1) / NW, a.grid_collide);
@@ -2211,7 +2225,7 @@ int collide_warp_blocks_per_sm(int M)
     using K = CollideWarpKernel<NW>;
     int nb = 0;
     const int smem = K::smem_bytes(M);
-    if (ensure_smem(collide_warp_kernel<NW, MINB>, smem) != cudaSuccess) return 1;
+    if (ensure_points_smem<K>(collide_warp_kernel<NW, MINB>, smem) != cudaSuccess) return 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, collide_warp_kernel<NW, MINB>, K::THREADS, smem);
     return nb > 0 ? nb : 1;
 }
@@ -2258,7 +2272,7 @@ cudaError_t launch_collide_slice(const RolloutArgs& a, cudaStream_t stream)
 {
     using K = CollideSliceKernel<S, P>;
     const int smem = K::smem_bytes(a.M);
-    cudaError_t e = ensure_smem(collide_slice_kernel<S, MINB, false, P>, smem);
+    cudaError_t e = ensure_points_smem<K>(collide_slice_kernel<S, MINB, false, P>, smem);
     if (e != cudaSuccess) return e;
     const int grid = max(1, min(((a.N + 7) / 8 + P - 1) / P, a.grid_collide));
     collide_slice_kernel<S, MINB, false, P><<<grid, K::THREADS, smem, stream>>>(a);
@@ -2271,7 +2285,7 @@ int collide_slice_blocks_per_sm(int M)
     using K = CollideSliceKernel<S, P>;
     int nb = 0;
     const int smem = K::smem_bytes(M);
-    if (ensure_smem(collide_slice_kernel<S, MINB, false, P>, smem) != cudaSuccess) return 1;
+    if (ensure_points_smem<K>(collide_slice_kernel<S, MINB, false, P>, smem) != cudaSuccess) return 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, collide_slice_kernel<S, MINB, false, P>, K::THREADS, smem);
     return nb > 0 ? nb : 1;
 }
