@@ -121,6 +121,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
         mbar_init_fence();
     }
     if (warp == 0) {
+        __syncwarp();                          // after lane 0's set-up
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(smem_u32(tmem_slot)), "r"(2 * BN) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -196,7 +197,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUte
         for (int u = blockIdx.x; u < units; u += gridDim.x, ++i) {
             const int b = i & 1;
             const bool ok = mbar_wait(&tfull[b], (i >> 1) & 1);
-            if (!__all_sync(0xffffffffu, ok) || *reinterpret_cast<volatile int*>(&flags[0])) {
+            // (one answer for the warp, whose lanes the vote brings together:
+            // the accumulator reads are the whole warp's)
+            if (!__all_sync(0xffffffffu, ok && !*reinterpret_cast<volatile int*>(&flags[0]))) {
                 atomicExch(&flags[0], 1);
                 break;
             }
@@ -275,6 +278,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__
         mbar_init_fence();
     }
     if (warp == 0) {
+        __syncwarp();                          // after lane 0's set-up
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(smem_u32(tmem_slot)), "r"(512) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
@@ -346,7 +350,9 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap ta, const __grid_constant__
         for (int u = pair; u < units; u += pairs, ++i) {
             const int b = i & 1;
             const bool ok = mbar_wait_cluster(&tfull[b], (i >> 1) & 1);
-            if (!__all_sync(0xffffffffu, ok) || *reinterpret_cast<volatile int*>(&flags[0])) {
+            // (one answer for the warp, whose lanes the vote brings together:
+            // the accumulator reads are the whole warp's)
+            if (!__all_sync(0xffffffffu, ok && !*reinterpret_cast<volatile int*>(&flags[0]))) {
                 atomicExch(&flags[0], 1);
                 break;
             }

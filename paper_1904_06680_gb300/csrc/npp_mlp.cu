@@ -73,6 +73,7 @@ __device__ __forceinline__ uint32_t pipe_init(Pipe<STAGES>& p)
         mbar_init_fence();
     }
     if (warp == 0) {
+        __syncwarp();                          // after lane 0's set-up
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(smem_u32(&p.tmem)), "r"(512) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
@@ -107,6 +108,12 @@ __device__ __forceinline__ void pipe_end(Pipe<STAGES>& p, uint32_t tmem, int* er
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
     }
 }
+
+// Epilogue side, after a wait: whether every lane's was in time and nothing
+// aborted, the same answer for the whole warp.  The vote also brings its lanes
+// together: the accumulator reads that follow are the whole warp's.
+template <int STAGES>
+__device__ __forceinline__ bool epilogue_go(Pipe<STAGES>& p, bool ok) { return __all_sync(0xffffffffu, ok && !aborted(p)); }
 
 // Producer side: the next stage, free; false to stop.
 template <int STAGES>
@@ -328,7 +335,7 @@ mlp_forward_kernel(const __grid_constant__ MlpForwardMaps maps, const MlpForward
             for (int l = 0; l < 2 && go; ++l, ++layer) {
                 const int b = layer & 1;
                 const bool ok = mbar_wait(&p.tfull[b], (layer >> 1) & 1);
-                if (!__all_sync(0xffffffffu, ok) || aborted(p)) { atomicExch(&p.flags[0], 1); go = false; break; }
+                if (!epilogue_go(p, ok)) { atomicExch(&p.flags[0], 1); go = false; break; }
                 tc_fence_after();
                 uint32_t pos[4] = { 0u, 0u, 0u, 0u };      // positive activations of this lane's 128 columns
 #pragma unroll
@@ -358,7 +365,7 @@ mlp_forward_kernel(const __grid_constant__ MlpForwardMaps maps, const MlpForward
                 float2 th[16];
                 if constexpr (TRAIN) fetch_rows(f.theta, tvec, m0 + q * 32, f.n, p0, lane, th);
                 const bool ok = mbar_wait(&p.tfull[b], (layer >> 1) & 1);
-                if (!__all_sync(0xffffffffu, ok) || aborted(p)) { atomicExch(&p.flags[0], 1); go = false; break; }
+                if (!epilogue_go(p, ok)) { atomicExch(&p.flags[0], 1); go = false; break; }
                 tc_fence_after();
                 float loss = 0.0f;
                 const float scale = 1.0f / ((float)f.n * (float)MLP_NTH);
@@ -369,8 +376,8 @@ mlp_forward_kernel(const __grid_constant__ MlpForwardMaps maps, const MlpForward
                     float sd[TRAIN ? 1 : 32];
                     if constexpr (TRAIN) {
                         rows_to_scratch(sc, lane, th);
-                        __syncwarp();
                         if (ch == 0) fetch_rows(f.theta, tvec, m0 + q * 32, f.n, p0 + 32, lane, th);
+                        __syncwarp();
                     }
 #pragma unroll
                     for (int s = 0; s < 2; ++s) {
@@ -560,7 +567,7 @@ mlp_backward_kernel(const __grid_constant__ MlpBackwardMaps maps, const MlpBackw
                 const uint4 mk = __ldg(f.mask + ((size_t)(1 - l) * f.n + row) * 2 + half);
                 const uint32_t pos[4] = { mk.x, mk.y, mk.z, mk.w };
                 const bool ok = mbar_wait(&p.tfull[b], (layer >> 1) & 1);
-                if (!__all_sync(0xffffffffu, ok) || aborted(p)) { atomicExch(&p.flags[0], 1); go = false; break; }
+                if (!epilogue_go(p, ok)) { atomicExch(&p.flags[0], 1); go = false; break; }
                 tc_fence_after();
 #pragma unroll
                 for (int ch = 0; ch < 8; ++ch) {
@@ -682,7 +689,7 @@ mlp_grad_kernel(const __grid_constant__ MlpGradMaps maps, const MlpGrads f)
             const Unit x = unit(u);
             const int b = i & 1;
             const bool ok = mbar_wait(&p.tfull[b], (i >> 1) & 1);
-            if (!__all_sync(0xffffffffu, ok) || aborted(p)) { atomicExch(&p.flags[0], 1); break; }
+            if (!epilogue_go(p, ok)) { atomicExch(&p.flags[0], 1); break; }
             tc_fence_after();
             const int rows = x.k == 0 ? MLP_D3 : MLP_HID;
             float* out = f.part[x.k] + ((size_t)x.z * rows + x.m0 + q * 32 + lane) * x.bn;

@@ -153,6 +153,9 @@ __device__ __forceinline__ void mma_commit(uint64_t* bar)
                  ::"r"(smem_u32(bar)) : "memory");
 }
 
+// sixteen accumulator columns of the warp's 32 rows; the read is the whole
+// warp's (.sync.aligned): after code that parts its lanes (waits, guarded
+// accesses), callers __syncwarp
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v)
 {
     uint32_t r[16];

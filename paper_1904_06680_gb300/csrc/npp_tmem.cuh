@@ -1,7 +1,8 @@
 // npp_tmem.cuh -- tensor memory (256 KB per SM: 128 lanes x 512 columns of 32
 // bits) as plain per-warp storage, as inline PTX.  A warp reaches the 32
 // lanes of its quarter (warp index modulo 4); one column is one 32-bit value
-// per thread.
+// per thread.  Every instruction here but the fences is the whole warp's
+// (.sync.aligned): after code that parts its lanes, callers __syncwarp first.
 #pragma once
 
 #include <cstdint>
