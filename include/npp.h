@@ -524,9 +524,13 @@ npp_status npp_last_timing(npp_handle* h, float* stage_ms, int32_t n);
  * of the first round of a closed loop's sampling time created with timing
  * on): [0] candidate point tests (each one evaluation of the rectangle's
  * inequalities), [1] states checked, [2] sample-steps the trajectory kernel
- * rolled out (N T in one launch, fewer with the step chunks).  Zero when
- * that step used another collision check.  Synchronises the device; needs
- * timing enabled; writes up to n (at most 3) values. */
+ * rolled out (N T in one launch, fewer with the step chunks).  The same from
+ * run to run: where the check takes a step's samples together (from 1024
+ * samples, in one launch), [1] are the states up to each sample's first
+ * collision, [0] the points of the cells their boxes overlap, and a timed step
+ * ends with a kernel that counts them, after the last event.  Zero when that
+ * step used another collision check.  Synchronises the device; needs timing
+ * enabled; writes up to n (at most 3) values. */
 npp_status npp_last_counts(npp_handle* h, uint64_t* counts, int32_t n);
 
 #ifdef __cplusplus

@@ -269,7 +269,14 @@ npp_status run_rollout(npp_handle* h, RolloutArgs& a, cudaStream_t s, bool no_re
     a.coefB = nullptr;
     a.work = h->d_work;
     a.sm_count = h->sm_count;
+    a.first = nullptr;
+    a.done = nullptr;
+    a.counts = nullptr;
     if (h->timing) h->last_chunks = 1;
+    // measurement counters (candidate tests, states checked, sample-steps
+    // rolled out): zero unless the rectangle's binned check runs
+    const bool count = h->timing && h->counting;
+    if (count) CUDA_TRY(h, cudaMemsetAsync(h->d_counts, 0, 4 * sizeof(unsigned long long), s));
     if (h->fp_faces > 0) {
         // general footprint: grids sized by its radius (side stream, as
         // below), trajectories without the rectangle's rows, polygon check
@@ -309,12 +316,7 @@ npp_status run_rollout(npp_handle* h, RolloutArgs& a, cudaStream_t s, bool no_re
         if (h->timing) CUDA_TRY(h, record_event(h->ev[0], s));
         const bool fuse = no_records && (h->fuse == 1 || (h->fuse < 0 && h->cfg.width == 64));
         if (!fuse) {
-            if (h->timing) {
-                // measurement counters (candidate tests, states checked,
-                // sample-steps rolled out)
-                CUDA_TRY(h, cudaMemsetAsync(h->d_counts, 0, 4 * sizeof(unsigned long long), s));
-                a.counts = h->d_counts;
-            }
+            if (count) a.counts = h->d_counts;
             // the grids depend only on the points: build them on the side
             // stream while the trajectories run (fork/join events; under
             // stream capture this makes two graph branches)
@@ -333,18 +335,13 @@ npp_status run_rollout(npp_handle* h, RolloutArgs& a, cudaStream_t s, bool no_re
             if (h->timing) CUDA_TRY(h, record_event(h->ev[1], s));
             CUDA_TRY(h, cudaStreamWaitEvent(s, h->join_ev, 0));
             CUDA_TRY(h, grid ? launch_collide_grid(a, s) : launch_collide_binned(a, s));
-            a.first = nullptr;
-            a.done = nullptr;
-            a.counts = nullptr;
+            if (!grid) a.counts = nullptr;       // else count_work's
             if (h->timing) CUDA_TRY(h, record_event(h->ev[2], s));
             return NPP_OK;
         }
         // fused: the grids first, then the trajectories with the windowed
         // check inside (timing: [0] the grid build, [1] the fused kernel)
-        if (h->timing) {
-            CUDA_TRY(h, cudaMemsetAsync(h->d_counts, 0, 4 * sizeof(unsigned long long), s));
-            a.counts = h->d_counts;
-        }
+        if (count) a.counts = h->d_counts;
         CUDA_TRY(h, build_bins(a, h->cfg.half_len, h->cfg.half_wid, h->cfg.c_off, h->d_bins, s));
         if (h->timing) CUDA_TRY(h, record_event(h->ev[1], s));
         CUDA_TRY(h, launch_fused(h, a, s));
@@ -384,6 +381,11 @@ npp_status run_rollout(npp_handle* h, RolloutArgs& a, cudaStream_t s, bool no_re
     return NPP_OK;
 }
 
+
+cudaError_t count_work(const RolloutArgs& a, cudaStream_t s)
+{
+    return a.counts && a.first ? launch_count_grid(a, s) : cudaSuccess;
+}
 
 static SamplerKey make_key(uint64_t seed, uint32_t t_index, uint32_t stream_id)
 {
@@ -594,6 +596,7 @@ static npp_status plan_step_impl(npp_handle* h, const npp_state* state, const np
     e.trajectory = out->trajectory;
     CUDA_TRY(h, launch_epilogue(e, s));
     if (h->timing) CUDA_TRY(h, record_event(h->ev[3], s));
+    CUDA_TRY(h, count_work(a, s));
     return NPP_OK;
 }
 
@@ -725,6 +728,7 @@ npp_status npp_rollout_params(npp_handle* h, const npp_state* state, const npp_g
     a.best_key = nullptr;
     if ((st = run_rollout(h, a, s, !sample_traj_dev && !sample_ctrl_dev)) != NPP_OK) return st;
     if (h->timing) CUDA_TRY(h, record_event(h->ev[3], s));
+    CUDA_TRY(h, count_work(a, s));
     return NPP_OK;
 }
 
@@ -825,7 +829,7 @@ npp_status npp_inject_fault(npp_handle* h)
 npp_status npp_set_timing(npp_handle* h, int32_t enable)
 {
     if (!h) return fail(nullptr, NPP_INVALID_ARG, "handle is NULL");
-    h->timing = enable != 0;
+    h->timing = h->counting = enable != 0;
     return NPP_OK;
 }
 

@@ -204,6 +204,20 @@ __device__ __forceinline__ void copy_async(void* dst, const void* src)
 __device__ __forceinline__ void copy_async_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 constexpr int GRID_CS_BYTES = (BIN_NCELL + 8) * 2;
 
+// the cells a query box overlaps
+struct QueryCells {
+    int ix0, ix1, iy0, iy1;
+};
+__device__ __forceinline__ QueryCells query_cells(const BinView& g, const QueryBox& q)
+{
+    QueryCells c;
+    c.ix0 = bin_cell(q.x - q.rx, g);
+    c.ix1 = bin_cell(q.x + q.rx, g);
+    c.iy0 = bin_cell(q.y - q.ry, g);
+    c.iy1 = min(bin_cell(q.y + q.ry, g), c.iy0 + BIN_MAX_ROWS - 1);
+    return c;
+}
+
 __global__ void __launch_bounds__(GRID_THREADS, 2) collide_grid_kernel(const RolloutArgs a, int chunk)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -230,7 +244,6 @@ __global__ void __launch_bounds__(GRID_THREADS, 2) collide_grid_kernel(const Rol
         copy_async_wait();
     }
     __syncthreads();
-    unsigned ntest = 0, nstate = 0;
     for (int n = n0 + tid; n < n1; n += GRID_THREADS) {
         if (__ldcg(a.first + n) <= h) continue;
         const float4 z = a.traj[(size_t)h * N + n];
@@ -238,30 +251,14 @@ __global__ void __launch_bounds__(GRID_THREADS, 2) collide_grid_kernel(const Rol
         sincos_r(z.z, sp, cp);
         RectTest test;
         coef_rows(a.c, z.x, z.y, sp, cp, test.a, test.b);
-        const QueryBox q = query_box(g, z.x, z.y, sp, cp);
-        const int ix0 = bin_cell(q.x - q.rx, g), ix1 = bin_cell(q.x + q.rx, g);
-        const int iy0 = bin_cell(q.y - q.ry, g), iy1 = min(bin_cell(q.y + q.ry, g), iy0 + BIN_MAX_ROWS - 1);
+        const QueryCells q = query_cells(g, query_box(g, z.x, z.y, sp, cp));
         bool hit = false;
-        for (int iy = iy0; iy <= iy1 && !hit; ++iy) {
-            const int b = cs[iy * BIN_DIM + ix0], e = cs[iy * BIN_DIM + ix1 + 1];
-            ntest += e - b;
+        for (int iy = q.iy0; iy <= q.iy1 && !hit; ++iy) {
+            const int b = cs[iy * BIN_DIM + q.ix0], e = cs[iy * BIN_DIM + q.ix1 + 1];
             // two points a pass (an odd run's last point twice)
             for (int i = b; i < e; i += 2) hit |= test(pts[i]) | test(pts[min(i + 1, e - 1)]);
         }
-        ++nstate;
         if (hit) atomicMin(a.first + n, h);
-    }
-    if (a.counts) {
-        unsigned long long t = ntest, s = nstate;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) {
-            t += __shfl_xor_sync(FULL, t, off);
-            s += __shfl_xor_sync(FULL, s, off);
-        }
-        if ((tid & 31) == 0) {
-            atomicAdd(a.counts, t);
-            atomicAdd(a.counts + 1, s);
-        }
     }
     // the chunk's last block: every first colliding step is in
     __threadfence();
@@ -297,6 +294,34 @@ __global__ void __launch_bounds__(GRID_THREADS, 2) collide_grid_kernel(const Rol
     if (tid == 0) {
         for (int w = 1; w < GRID_THREADS / 32; ++w) best = red[w] < best ? red[w] : best;
         atomicMin(a.best_key, best);
+    }
+}
+
+// The grid check's work counters, from its results: a sample's states up to
+// its first collision (all without one) and the points in the cells their
+// boxes overlap.  The check itself cannot count: which states of a collided
+// sample it still meets depends on the order in which the steps' blocks run.
+// Timed plan steps only, after the last event.
+constexpr int COUNT_THREADS = 256;
+__global__ void __launch_bounds__(COUNT_THREADS) count_grid_kernel(const RolloutArgs a)
+{
+    const int n = blockIdx.x * COUNT_THREADS + threadIdx.x, h = blockIdx.y;
+    const BinView& g = a.bins;
+    unsigned tests = 0, states = 0;
+    if (n < a.N && h <= a.first[n]) {
+        const unsigned short* cs = reinterpret_cast<const unsigned short*>(g.cell_start + (size_t)h * BIN_CS_STRIDE);
+        const float4 z = a.traj[(size_t)h * a.N + n];
+        float sp, cp;
+        sincos_r(z.z, sp, cp);
+        const QueryCells q = query_cells(g, query_box(g, z.x, z.y, sp, cp));
+        for (int iy = q.iy0; iy <= q.iy1; ++iy) tests += cs[iy * BIN_DIM + q.ix1 + 1] - cs[iy * BIN_DIM + q.ix0];
+        states = 1;
+    }
+    tests = __reduce_add_sync(FULL, tests);
+    states = __reduce_add_sync(FULL, states);
+    if ((threadIdx.x & 31) == 0 && states) {
+        atomicAdd(a.counts, (unsigned long long)tests);
+        atomicAdd(a.counts + 1, (unsigned long long)states);
     }
 }
 
@@ -360,6 +385,12 @@ cudaError_t launch_collide_grid(const RolloutArgs& a, cudaStream_t s)
     const cudaError_t e = ensure_smem(collide_grid_kernel, GRID_CS_BYTES + collide_grid_points() * (int)sizeof(float2));
     if (e != cudaSuccess) return e;
     collide_grid_kernel<<<grid, GRID_THREADS, smem, s>>>(a, chunk);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_count_grid(const RolloutArgs& a, cudaStream_t s)
+{
+    count_grid_kernel<<<dim3((a.N + COUNT_THREADS - 1) / COUNT_THREADS, a.T + 1), COUNT_THREADS, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -644,6 +644,7 @@ cudaError_t build_bins(RolloutArgs& a, float half_len, float half_wid, float c_o
 constexpr int GRID_MAX_CHUNKS = 1024;
 int collide_grid_points();
 cudaError_t launch_collide_grid(const RolloutArgs& a, cudaStream_t s);
+cudaError_t launch_count_grid(const RolloutArgs& a, cudaStream_t s);   // its work, after it
 cudaError_t launch_collide_binned(const RolloutArgs& a, cudaStream_t s);
 cudaError_t launch_collide_poly(const RolloutArgs& a, cudaStream_t s);     // every point (a.poly.brute)
 // grids for a general footprint inside the disk of the given radius around

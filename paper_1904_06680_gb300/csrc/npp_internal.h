@@ -85,7 +85,8 @@ struct npp_handle {
     cudaStream_t stream;
     cudaStream_t side;                   // concurrent branch of a plan step (grid build)
     cudaEvent_t fork_ev, join_ev;
-    bool timing;
+    bool timing;                         // stage events
+    bool counting;                       // work counters (with timing; a loop created without it has events only)
     cudaEvent_t ev[4];                   // start, after trajectories, after collisions, end
     cudaEvent_t cev[NPP_CHUNK_EVENTS];   // chunked step: before trajectories k (2k), before check k
                                          // (2k + 1), after the last check (2K)
@@ -123,6 +124,9 @@ cudaError_t stage_times(const cudaEvent_t* ev, const cudaEvent_t* cev, int nch, 
 // rolling a sample out after its first collision (the winner's rows, up to
 // its first collision, are always complete)
 npp_status run_rollout(npp_handle* h, npp::RolloutArgs& a, cudaStream_t s, bool no_records);
+// the work counters that run_rollout(a) leaves to be taken from its results;
+// the caller queues it after its last event
+cudaError_t count_work(const npp::RolloutArgs& a, cudaStream_t s);
 
 #define CUDA_TRY(h, call)                                                                  \
     do {                                                                                   \

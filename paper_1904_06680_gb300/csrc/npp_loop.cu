@@ -352,6 +352,8 @@ npp_status enqueue_step(npp_loop* L, uint64_t seed)
     e.trajectory = L->d_trajectory;
     e.dyn = L->d_dyn;
     CUDA_TRY(h, launch_epilogue(e, s));
+    // the first round's counters, before other rounds overwrite its states
+    if (L->restarts > 1) CUDA_TRY(h, count_work(a, s));
     // restart rounds: the winner so far is sample 0 (warm start, valid even
     // at the loop's first step), every other sample a perturbation of it on
     // the round's own Philox stream; the winner's parameters, controls and
@@ -392,6 +394,7 @@ npp_status enqueue_step(npp_loop* L, uint64_t seed)
         CUDA_TRY(h, cudaGetLastError());
     }
     CUDA_TRY(h, record_event(L->ev[3], s));
+    if (L->restarts == 1) CUDA_TRY(h, count_work(a, s));
     return NPP_OK;
 }
 
