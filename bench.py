@@ -54,6 +54,7 @@ DEFAULT_FUSE = -1                # the library's default of the "fuse" option (-
 FP32_LANES_PER_SM = 128          # FP32 FMA lanes per SM (4 schedulers x 32) on sm_100-class parts
 SM_MAX_MHZ_NOMINAL = 2070.0      # GB300 maximum SM clock, used only when the device does not report it
 BIN_DIM = 128                    # cells per side of the library's per-step grids (the grid build's table size)
+GRID_POINTS = (100 * 1024 - 2 * (BIN_DIM * BIN_DIM + 8)) // 8   # most points of a step's grid in shared memory (library)
 
 
 def parse():
@@ -263,6 +264,72 @@ def states_auto(M, N, W):
     check of a few points (the same rule as its states_auto; else the binned
     check)."""
     return M < (128 if W == 64 else 257 if N <= 1024 else 160)
+
+
+def kernel_shape(width, lanes, warps, blocks, *rest):
+    return "<%s>" % ",".join(str(int(x)) for x in (width, lanes, warps, blocks) + rest)
+
+
+def traj_kernel_name(W, N, sms, var=False, option=0):
+    """The trajectory kernel of a plan step of N samples at width W (the
+    library's rules in npp_rollout_w16/32/64.cu): var = speed limits or
+    features in the body frame, option = "traj_variant"."""
+    if option >= 3 and not var:
+        return "traj_kernel" + {16: kernel_shape(16, 8, 4, 4, 0, 0), 32: kernel_shape(32, 16, 4, 4, 0, 0),
+                                64: kernel_shape(64, 32, 1, 16, 0, 8)}[W]
+    if W == 64:
+        wide = N >= 16384
+    else:
+        wide = -(-N // {16: 16, 32: 8}[W]) > sms * 7 // 8
+    wide = option == 1 or (option != 2 and wide)
+    if W == 16 and wide and 16 * 8 * sms < N <= 20 * 8 * sms:
+        return "traj_tmem_kernel" + kernel_shape(16, 4, 20, 1, var, 4, 0, 1)
+    return "traj_tmem_kernel" + {(16, True): kernel_shape(16, 4, 4, 4, var, 4, 0, 0),
+                                 (16, False): kernel_shape(16, 8, 4, 6, var, 4, 0, 0),
+                                 (32, True): kernel_shape(32, 8, 4, 4, var, 8, 0, 0),
+                                 (32, False): kernel_shape(32, 16, 4, 5, var, 8, 0, 0),
+                                 (64, True): kernel_shape(64, 16, 4, 3, var, 8, 8, 0),
+                                 (64, False): kernel_shape(64, 32, 4, 4, var, 16, 0, 0)}[W, wide]
+
+
+def fused_kernel_name(W, N, sms, var=False, option=0):
+    """The trajectory kernel with the windowed check (same files)."""
+    if W == 64 and (option < 3 or var):
+        full = option == 1 or (option != 2 and N >= 160 * sms)
+        return "fused_tmem_kernel" + (kernel_shape(64, 32, 24, 1, var, 10, 6, 8, 4) if full
+                                      else kernel_shape(64, 32, 4, 4, var, 16, 0, 8, 4))
+    if W == 64:
+        return "fused_kernel" + kernel_shape(64, 32, 1, 16, 0, 12, 8, 4)
+    o = 0 if var else option
+    if W == 16:
+        return "fused_kernel" + kernel_shape(16, 8, 4, 4, var, 0, *{2: (8, 4), 3: (16, 2)}.get(o, (16, 4)))
+    return "fused_kernel" + {1: kernel_shape(32, 16, 4, 4, 0, 0, 16, 4), 2: kernel_shape(32, 16, 4, 4, 0, 0, 8, 4),
+                             3: kernel_shape(32, 16, 4, 3, 0, 0, 16, 4), 4: kernel_shape(32, 16, 4, 5, 0, 5, 16, 4)
+                             }.get(o, kernel_shape(32, 16, 4, 5, var, 5, 8, 4))
+
+
+def check_kernel_name(M, N, T, variant, poly=False, chunks=1):
+    """The collision kernel of a plan step that does not check as it rolls
+    out; variant: "collide_variant", 5 for the automatic binned choice."""
+    if poly:
+        return "collide_poly_kernel" if 0 <= variant < 5 else "collide_binned_kernel<1>"
+    if variant == 5:
+        grid = chunks == 1 and N >= 1024 and M <= GRID_POINTS and T < 65535
+        return "collide_grid_kernel" if grid else "collide_binned_kernel<0>"
+    return {0: "collide_block_kernel<16,128,1>", 1: "collide_block_kernel<8,64,2>", 2: "collide_warp_kernel<8,2>",
+            3: "collide_slice_kernel<4,2,0,2>", 4: "collide_slice_kernel<2,2,0,4>",
+            -1: "collide_states_kernel<%d>" % (16 if N >= 8192 and M < 64 and T < 128 else 32)}[variant]
+
+
+def grid_check_bytes(N, T, M, sms, states):
+    """Bytes that the check with a step's grid in shared memory reads and
+    writes per plan step: per block (a chunk of the samples at a step) the
+    step's 16-bit cell starts and its points, per state checked the state
+    (16 B) and the sample's first collision so far (4 B), per sample its free
+    cost, cost and first hit (12 B)."""
+    whole = lambda n: -(-n // 512) * 512
+    chunk = max(min(whole(-(-N // max(1, 3 * sms // (T + 1)))), 1024), whole(-(-N // 1024)))
+    return -(-N // chunk) * (T + 1) * (2.0 * BIN_DIM * BIN_DIM + 8.0 * M) + 20.0 * states + 12.0 * N
 
 
 def brute_auto(M, N):
@@ -515,35 +582,30 @@ def run_npp(args):
         nch = min(int(options.get("chunks", 0)) or (2 if W == 64 else 1), T)
     # per sampling time: plan step kernels, epilogue, vehicle and obstacle advance (one up to 4096 points)
     launches_per_step = (2 if fused else 1 + 2 * nch if binned and not poly else 3 if poly else 2) + 2 + (M > 4096)
-    # default launch shapes; the fifth template argument is the variant flag
-    # (off: no speed limits, features in the EV frame at t)
-    var = int(bool(p.get("v_limits", 0) or p.get("feature_frame", 0)))
+    # the kernels that ran
+    var = bool(p.get("v_limits", 0) or p.get("feature_frame", 0))
     sms = torch.cuda.get_device_properties(local).multi_processor_count
-    wide = N >= 16384 if W == 64 else -(-N // {16: 16, 32: 8}[W]) > sms * 7 // 8
-    shape = "_tmem_kernel" + ({16: "<16,4,4,4,%d,4,0>", 32: "<32,8,4,4,%d,8,0>", 64: "<64,16,4,3,%d,8,8>"} if wide else
-                              {16: "<16,8,4,6,%d,4,0>", 32: "<32,16,4,5,%d,8,0>", 64: "<64,32,4,4,%d,16,0>"})[W] % var
+    tname = traj_kernel_name(W, N, sms, var, int(options.get("traj_variant", 0)))
+    check = check_kernel_name(M, N, T, 5 if binned and not poly else cv, poly, nch)
     if fused:
         # [0] grid build, [1] the trajectory kernel with the windowed check
-        full = N >= 160 * sms
-        fshape = {16: "_kernel<16,8,4,4,%d,0,16,4>", 32: "_kernel<32,16,4,5,%d,5,8,4>",
-                  64: "_tmem_kernel<64,32,24,1,%d,10,6,8,4>" if full else "_tmem_kernel<64,32,4,4,%d,16,0,8,4>"}[W] % var
-        fname = "fused" + fshape
+        fname = fused_kernel_name(W, N, sms, var, int(options.get("traj_variant", 0)))
         fps = res["fma_t"] / (collide_ms / 1e3)
         rolled = res["rolled"] if res["rolled"] > 0 else float(N) * T * K
         fma_rolled = rolled * (W * W + 10 * W)
-        check = {}
+        window = {}
         if res["states"] > 0:
             # the window check's algorithmic reads (L2-resident grids): per
             # state checked the ten cell-run bounds of its query (40 B; the
             # state itself is in the warp's shared window), per candidate
             # test one point (8 B)
             wbytes = res["states"] * 40.0 + res["cand_tests"] * 8.0
-            check = {"candidate_tests_per_state": res["cand_tests"] / res["states"],
-                     "states_checked_per_plan_step": res["states"] / K,
-                     "candidate_tests_per_s": res["cand_tests"] / (collide_ms / 1e3),
-                     "bytes_per_step": wbytes / K, "achieved_gbs": wbytes / (collide_ms / 1e3) / 1e9,
-                     "bytes_note": "algorithmic grid reads: 40 B per state checked (ten cell-run "
-                                   "bounds), 8 B per candidate test, over the kernel's duration"}
+            window = {"candidate_tests_per_state": res["cand_tests"] / res["states"],
+                      "states_checked_per_plan_step": res["states"] / K,
+                      "candidate_tests_per_s": res["cand_tests"] / (collide_ms / 1e3),
+                      "bytes_per_step": wbytes / K, "achieved_gbs": wbytes / (collide_ms / 1e3) / 1e9,
+                      "bytes_note": "algorithmic grid reads: 40 B per state checked (ten cell-run "
+                                    "bounds), 8 B per candidate test, over the kernel's duration"}
         bin_bytes = grid_bytes(T, M)
         bin_s = traj_ms / K / 1e3
         bins = {"ms_per_step": traj_ms / K, "bytes_per_step": bin_bytes,
@@ -564,32 +626,34 @@ def run_npp(args):
                     "rolled_steps_achieved": fma_rolled / (collide_ms / 1e3) / 1e12,
                     "rolled_steps_frac": fma_rolled / (collide_ms / 1e3) / peak,
                     "kernel_ms_per_step": collide_ms / K,
-                    "windowed_check": check,
+                    "windowed_check": window,
                     "other": {"bin_build_kernel": bins},
                     "dominant": fname}
     elif binned:
         # the binned (or polygon) check does only the candidate work of the
         # cells a state overlaps, which has no fixed algorithmic count; the
         # MLP rollout is the work every plan step must do
-        tname = "traj" + shape
-        cname = "bin_build_kernel + " + ("collide_binned_kernel" if poly or nch > 1 or N < 1024 or M > 8702
-                                         else "collide_grid_kernel")
+        cname = "bin_build_kernel + " + check
         fps_t = res["fma_t"] / (traj_ms / 1e3)
         coll = {"ms_per_step": collide_ms / K}
         if not poly and res["states"] > 0:
-            # the check's algorithmic bytes: per state checked its stored
-            # state (16 B) and the ten cell-run bounds of its query (40 B),
-            # per candidate test one point (8 B), per sample its free cost
-            # read and cost / first-hit written (12 B)
-            nbytes = res["states"] * 56.0 + res["cand_tests"] * 8.0 + 12.0 * N * K
+            # the check's algorithmic bytes; the warp-per-sample kernel: per
+            # state checked its stored state (16 B) and the ten cell-run bounds
+            # of its query (40 B), per candidate test one point (8 B), per
+            # sample its free cost read and cost / first-hit written (12 B)
+            grid = check == "collide_grid_kernel"
+            nbytes = (K * grid_check_bytes(N, T, M, sms, res["states"] / K) if grid
+                      else res["states"] * 56.0 + res["cand_tests"] * 8.0 + 12.0 * N * K)
             coll.update(candidate_tests_per_s=res["cand_tests"] / (collide_ms / 1e3),
                         candidate_tests_per_state=res["cand_tests"] / res["states"],
                         states_per_s=res["states"] / (collide_ms / 1e3),
                         bytes_per_step=nbytes / K, achieved_gbs=nbytes / (collide_ms / 1e3) / 1e9,
-                        traffic=profiled_traffic(cname.split(" + ")[-1], args.workload),
-                        bytes_note="algorithmic: 56 B per state checked (state + ten cell-run bounds), "
-                                   "8 B per candidate test, 12 B per sample; traffic = DRAM bytes per "
-                                   "launch from profiles/traffic.json")
+                        traffic=profiled_traffic(check, args.workload),
+                        bytes_note=("algorithmic: per (chunk, step) block the 32 KB of cell starts and 8 B per "
+                                    "point, 20 B per state checked, 12 B per sample" if grid else
+                                    "algorithmic: 56 B per state checked (state + ten cell-run bounds), "
+                                    "8 B per candidate test, 12 B per sample") +
+                                   "; traffic = DRAM bytes per launch from profiles/traffic.json")
         # sample-steps the trajectory launches rolled out (N T per plan step
         # in one launch; fewer in step chunks, which drop collided samples)
         rolled = res["rolled"] if res["rolled"] > 0 else float(N) * T * K
@@ -607,11 +671,7 @@ def run_npp(args):
                     "other": {cname: coll},
                     "dominant": tname if traj_ms >= collide_ms else cname}
     else:
-        tname = "traj" + shape
-        cname = {0: "collide_block_kernel<16,128,1>", 1: "collide_block_kernel<8,64,2>",
-                 2: "collide_warp_kernel<8,2>", 3: "collide_slice_kernel<4,2,0,2>",
-                 4: "collide_slice_kernel<2,2,0,4>",
-                 -1: "collide_states_kernel<%d>" % (16 if N >= 8192 and M < 64 else 32)}[cv]
+        cname = check
         fps_c = res["fma_c"] / (collide_ms / 1e3)
         fps_t = res["fma_t"] / (traj_ms / 1e3)
         roofline = {"bound": "alu", "kernel": cname,
@@ -755,28 +815,43 @@ def run_batch(args):
     out.best, out.params, out.controls = best.data_ptr(), params.data_ptr(), ctrl.data_ptr()
     out.trajectory, out.costs, out.first_hit = traj.data_ptr(), costs.data_ptr(), fh.data_ptr()
     choice, tuned = autotune.tune_batch(B, obs, out, key="parking512", reps=1)
-    npp.npp_set_timing(pl.h, True)
+    # two graphs: the call as it is, for its duration, and the call with
+    # timing on, which runs the stages one after another, for theirs
     side = torch.cuda.Stream()
-    g = torch.cuda.CUDAGraph()
-    torch.cuda.synchronize()
-    with torch.cuda.graph(g, stream=side):
-        npp.npp_plan_batch(B, obs, out, stream=torch.cuda.current_stream())
+    graphs = []
+    for timing in (False, True):
+        npp.npp_set_timing(pl.h, timing)
+        graphs.append(torch.cuda.CUDAGraph())
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graphs[-1], stream=side):
+            npp.npp_plan_batch(B, obs, out, stream=torch.cuda.current_stream())
+    g, g_stages = graphs
     flush = torch.empty(64 * 1024 * 1024, dtype=torch.float32, device=dev)
     for _ in range(args.warmup):
         g.replay()
+        g_stages.replay()
     torch.cuda.synchronize()
     K = max(1, min(args.steps, 10))
     clocks = Clocks(local)
     clocks.start()
     tot, col, trj = [], [], []
+    start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     for _ in range(K):
         flush.zero_()
         torch.cuda.synchronize()
+        start.record()
         g.replay()
-        tm = npp.npp_last_timing(pl.h)
-        tot.append(tm["total"]); col.append(tm["collide"]); trj.append(tm["traj"])
-    torch.cuda.synchronize()
+        end.record()
+        torch.cuda.synchronize()
+        tot.append(start.elapsed_time(end))
     ck = clocks.stop()
+    for _ in range(K):
+        flush.zero_()
+        torch.cuda.synchronize()
+        g_stages.replay()
+        tm = npp.npp_last_timing(pl.h)
+        col.append(tm["collide"]); trj.append(tm["traj"])
+    torch.cuda.synchronize()
     fhs = fh.cpu().numpy()
     steps = float(sum(s["N"] * s["T"] for s in sc))
     checks = 0.0
