@@ -263,10 +263,6 @@ static npp_status run_chunked(npp_handle* h, RolloutArgs& a, cudaStream_t s, int
 
 npp_status run_rollout(npp_handle* h, RolloutArgs& a, cudaStream_t s, bool no_records)
 {
-    // no rows are stored: every collision kernel recomputes them from the
-    // stored states
-    a.coefA = nullptr;
-    a.coefB = nullptr;
     a.work = h->d_work;
     a.sm_count = h->sm_count;
     a.first = nullptr;
@@ -279,9 +275,7 @@ npp_status run_rollout(npp_handle* h, RolloutArgs& a, cudaStream_t s, bool no_re
     if (count) CUDA_TRY(h, cudaMemsetAsync(h->d_counts, 0, 4 * sizeof(unsigned long long), s));
     if (h->fp_faces > 0) {
         // general footprint: grids sized by its radius (side stream, as
-        // below), trajectories without the rectangle's rows, polygon check
-        a.coefA = nullptr;
-        a.coefB = nullptr;
+        // below), polygon check
         a.poly.faces = h->d_fp;
         a.poly.n_faces = h->fp_faces;
         a.poly.brute = (h->collide_variant >= 0 && h->collide_variant < COLLIDE_BINNED) ? 1 : 0;

@@ -366,15 +366,11 @@ __global__ void __launch_bounds__(NW * 32, MINB) batch_traj_kernel(const BatchAr
         job.bins = nullptr;
         job.stage = nullptr;
         job.w2s = nullptr;
-        job.N = s.N;
         job.T = s.T;
         job.traj = WIN ? nullptr : b.states + s.state_off;
         job.ctrl = nullptr;
         job.rec_stride = s.N;
         job.rec_shift = 0;
-        job.coefA = nullptr;
-        job.coefB = nullptr;
-        job.coef_base = 0;
         job.jfree = WIN ? nullptr : b.jfree + s.samp_off;
         job.vfirst = !WIN && b.vfirst ? b.vfirst + s.samp_off : nullptr;
         net.load(theta_src<Net::S::NT>(job, n, valid), gl);
@@ -600,15 +596,11 @@ __device__ void batch_reroll(const BatchArgs& b, const SceneDev& s, int idx, flo
     job.bins = nullptr;
     job.stage = nullptr;
     job.w2s = nullptr;
-    job.N = s.N;
     job.T = s.T;
     job.traj = b.trajectory ? reinterpret_cast<float4*>(b.trajectory) + s.traj_off : nullptr;
     job.ctrl = b.controls ? reinterpret_cast<float2*>(b.controls) + s.ctrl_off : nullptr;
     job.rec_stride = 1;
     job.rec_shift = idx;
-    job.coefA = nullptr;
-    job.coefB = nullptr;
-    job.coef_base = 0;
     job.jfree = nullptr;
     job.vfirst = nullptr;
     LaneNet<W, G> net;

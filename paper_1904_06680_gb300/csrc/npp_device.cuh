@@ -542,8 +542,6 @@ struct RolloutArgs {
     float* jfree;                      // [N] cost of each sample if collision-free
     int* vfirst;                       // [N] first speed-violating step (-1 none), written by the
                                        // trajectory kernel when c.vlim; null otherwise
-    float4* coefA;                     // [T+1][N] (A, B, -C, D) scaled inequality rows
-    float2* coefB;                     // [T+1][N] (E, -F)
     unsigned long long* best_key;      // packed (class, cost, index) minimum
     unsigned long long* reset_key;     // the minimum, for the trajectory kernel to start (null: started elsewhere)
     unsigned* work;                    // work-queue counter of the persistent collision kernel

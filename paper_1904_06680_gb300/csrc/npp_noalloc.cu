@@ -138,8 +138,6 @@ extern "C" npp_status npp_plan_step_noalloc(const npp_config* cfg, const npp_sta
                               : reinterpret_cast<float2*>(base + OFF_CTRL);
     a.jfree = reinterpret_cast<float*>(base + OFF_JFREE);
     a.vfirst = cfg->v_limits ? reinterpret_cast<int*>(base + OFF_VFIRST) : nullptr;
-    a.coefA = nullptr;                   // the collision kernels recompute the rows from the states
-    a.coefB = nullptr;
     a.best_key = reinterpret_cast<unsigned long long*>(base);
     a.work = reinterpret_cast<unsigned*>(base + 8);
     a.fault = reinterpret_cast<unsigned*>(base + 12);

@@ -528,9 +528,8 @@ __device__ __forceinline__ float wrap_pi(float a)
 // (an exact scaling).  |v| < 2 holds exactly when bit 30 of v's IEEE pattern
 // is clear, so "both inside" is bit 30 of (xi | eta) clear: one 3-input logic
 // op per point-sample pair accumulates "some point inside".
-// (Rounding fixed by explicit fmas and round-to-nearest products, so that the
-// rows stored by the trajectory kernel and the rows the fused check computes
-// are the same bits.)
+// (Rounding fixed by explicit fmas and round-to-nearest products, so that
+// every check computes the same bits.)
 __device__ __forceinline__ void coef_rows(const DevCfg& c, float x, float y, float sp, float cp, float4& A,
                                           float2& B)
 {
@@ -541,25 +540,13 @@ __device__ __forceinline__ void coef_rows(const DevCfg& c, float x, float y, flo
     B = make_float2(__fmul_rn(cp, sw), -__fmul_rn(across, sw));
 }
 
-// The rows of a stored state z = (x, y, phi, v): the trajectory kernel's own
-// arithmetic on the same FP32 values, so a collision kernel that recomputes
-// them from the stored state gets the same bits the rollout had (and no
-// rows need to be stored).
+// The rows of a stored state z = (x, y, phi, v): the windowed check's own
+// arithmetic on the same FP32 values, so every check gets the same bits.
 __device__ __forceinline__ void rows_of_state(const DevCfg& c, const float4& z, float4& A, float2& B)
 {
     float sp, cp;
     sincos_r(z.z, sp, cp);
     coef_rows(c, z.x, z.y, sp, cp, A, B);
-}
-
-__device__ __forceinline__ void write_coef(float4* coefA, float2* coefB, const DevCfg& c,
-                                           long long idx, float x, float y, float sp, float cp)
-{
-    float4 A;
-    float2 B;
-    coef_rows(c, x, y, sp, cp, A, B);
-    coefA[idx] = A;
-    coefB[idx] = B;
 }
 
 // The step at which a sample is discarded: the earlier of its first colliding
@@ -878,22 +865,18 @@ struct TrajKernel {
 };
 
 // One planning instance as the trajectory code sees it.  Records of sample n
-// at step h go to index h * rec_stride + n - rec_shift (states, controls);
-// coefficient rows to coef_base + h * N + n; the free cost to jfree[n].  Any
-// pointer may be null (nothing written).
+// at step h go to index h * rec_stride + n - rec_shift (states, controls),
+// the free cost to jfree[n].  Any pointer may be null (nothing written).
 struct TrajJob {
     StepIn si;
     SamplerKey key;               // t_index resolved
     const float* theta;           // explicit rows [N][n_theta] or null
     const float* warm;            // replaces sample 0 when non-null (and si.warm_ok)
     Proposal prop;                // sampling proposal (mu null: none)
-    int N, T;
+    int T;
     float4* traj;                 // [T+1] x stride
     float2* ctrl;                 // [T] x stride
     long long rec_stride, rec_shift;
-    float4* coefA;                // coefficient rows (scaled inequalities)
-    float2* coefB;
-    long long coef_base;
     float* jfree;
     int* vfirst;                  // first speed-violating step per sample (speed limits on), or null
     const BinView* bins;          // grids of the windowed check (traj_sample_windowed)
@@ -1073,8 +1056,8 @@ __device__ __forceinline__ float final_cost(const DevCfg& c, const GoalEV& g, fl
 
 // The trajectory of sample n (valid: n < N) computed by the G lanes of a
 // group (lane gl); hrow is the group's W-float shared exchange row.  Writes
-// the records the job asks for (states, controls, scaled inequality rows,
-// cost if collision-free, first speed-violating step).  VAR: the variants
+// the records the job asks for (states, controls, cost if collision-free,
+// first speed-violating step).  VAR: the variants
 // of c (body-frame goal offsets, speed limits) are honoured; without it the
 // kernel is the plain rollout, and the launchers pick VAR whenever c turns
 // a variant on.
@@ -1085,7 +1068,7 @@ __device__ __forceinline__ void traj_sample(const DevCfg& c, const TrajJob& job,
     const GoalEV g = goal_ev(job.si);
 
     float x = 0.f, y = 0.f, ph = 0.f, v = job.si.v0, ap0 = job.si.ap0, ap1 = job.si.ap1, E = 0.f;
-    const int T = job.T, N = job.N;
+    const int T = job.T;
     const float invT = 1.0f / (float)T;
     const bool writer = valid && gl == 0;
     const long long rec = (long long)n - job.rec_shift;
@@ -1110,16 +1093,6 @@ __device__ __forceinline__ void traj_sample(const DevCfg& c, const TrajJob& job,
         // pointer tests are uniform over the kernel; only the stores
         // depend on the writer lane
         if (job.traj && writer) job.traj[h * job.rec_stride + rec] = make_float4(x, y, ph, v);
-        if (job.coefA) {
-            float4 A;
-            float2 B;
-            coef_rows(c, x, y, sp, cp, A, B);
-            if (writer) {
-                const long long ci = job.coef_base + (long long)h * N + n;
-                job.coefA[ci] = A;
-                job.coefB[ci] = B;
-            }
-        }
         const float2 a = control_step<Net, VAR>(c, net, g, invT, gl, hrow, sp, cp, x, y, ph, v, ap0, ap1, E, rem);
         if (writer && job.ctrl) job.ctrl[h * job.rec_stride + rec] = a;
     }
@@ -1142,10 +1115,7 @@ __device__ __forceinline__ void traj_sample(const DevCfg& c, const TrajJob& job,
         if constexpr (VAR) {
             if (job.vfirst) job.vfirst[n] = vbad;
         }
-        float sp, cp;
-        sincos_r(ph, sp, cp);
         if (job.traj) job.traj[T * job.rec_stride + rec] = make_float4(x, y, ph, v);
-        if (job.coefA) write_coef(job.coefA, job.coefB, c, job.coef_base + (long long)T * N + n, x, y, sp, cp);
         if (job.jfree) job.jfree[n] = final_cost(c, g, x, y, ph, v, E, invT);
     }
 }
@@ -1272,15 +1242,11 @@ __global__ void __launch_bounds__(NW * 32, MINB) traj_kernel(const RolloutArgs a
     job.theta = a.theta;
     job.warm = a.warm;
     job.prop = a.prop;
-    job.N = a.N;
     job.T = a.T;
     job.traj = a.traj;
     job.ctrl = a.ctrl;
     job.rec_stride = a.N;
     job.rec_shift = 0;
-    job.coefA = a.coefA;
-    job.coefB = a.coefB;
-    job.coef_base = 0;
     job.jfree = a.jfree;
     job.vfirst = a.c.vlim ? a.vfirst : nullptr;
     job.bins = nullptr;
@@ -1338,15 +1304,11 @@ __global__ void __launch_bounds__(NW * 32, MINB) fused_kernel(const RolloutArgs 
     job.theta = a.theta;
     job.warm = a.warm;
     job.prop = a.prop;
-    job.N = a.N;
     job.T = a.T;
     job.traj = a.traj;
     job.ctrl = a.ctrl;
     job.rec_stride = a.N;
     job.rec_shift = 0;
-    job.coefA = nullptr;
-    job.coefB = nullptr;
-    job.coef_base = 0;
     job.jfree = nullptr;
     job.vfirst = nullptr;
     job.bins = &a.bins;
@@ -1410,15 +1372,11 @@ __device__ __forceinline__ TrajJob traj_job(const RolloutArgs& a)
     job.theta = a.theta;
     job.warm = a.warm;
     job.prop = a.prop;
-    job.N = a.N;
     job.T = a.T;
     job.traj = a.traj;
     job.ctrl = a.ctrl;
     job.rec_stride = a.N;
     job.rec_shift = 0;
-    job.coefA = nullptr;
-    job.coefB = nullptr;
-    job.coef_base = 0;
     job.jfree = a.jfree;
     job.vfirst = a.c.vlim ? a.vfirst : nullptr;
     job.bins = nullptr;
