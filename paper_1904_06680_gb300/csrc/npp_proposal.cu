@@ -600,6 +600,9 @@ npp_status npp_gemm_bf16(const uint16_t* A_dev, const uint16_t* B_dev, float* C_
     if (!A_dev || !B_dev || !C_dev) return perr(NPP_INVALID_ARG, "npp_gemm_bf16: NULL argument");
     if (M < 128 || M % 128 || N < 128 || N % 128 || K < 64 || K % 64)
         return perr(NPP_INVALID_ARG, "npp_gemm_bf16: M, N multiples of 128 and K a multiple of 64");
+    // (the tensor maps check A's and B's; the epilogue stores 16 bytes at a time)
+    if (reinterpret_cast<uintptr_t>(C_dev) & 15u)
+        return perr(NPP_INVALID_ARG, "npp_gemm_bf16: C must be 16-byte aligned");
     const int bn = (N % 256 == 0) ? 256 : 128, box_b = gemm_pairs(M, N) ? 128 : bn;
     CUtensorMap ta, tb;
     cudaError_t e = make_tmap_bf16(&ta, A_dev, M, K, 128);
