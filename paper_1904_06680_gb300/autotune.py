@@ -6,8 +6,10 @@ fixed per width), so tuning changes speed only.  It times each candidate on
 the caller's own workload with CUDA events on the launching stream and
 applies the fastest:
 
-* plan steps: the collision-kernel variant (block-balanced, warp items,
-  point-sliced items with 2 or 4 warps) for a given (width, N, T, M);
+* plan steps: the collision check (the library's own choice, block-balanced,
+  warp items, point-sliced items with 2 or 4 warps) for a given (width, N, T,
+  M), by the time of the whole plan step, since the check decides what runs
+  beside or inside the trajectories;
 * batches: the number of warps sharing one 8-sample collision item (the
   obstacle-point slice each warp checks) and the warps per trajectory block
   (samples per block).
@@ -23,7 +25,8 @@ import torch
 
 from . import npp
 
-PLAN_VARIANTS = (0, 1, 2, 3, 4)
+# -1: the library's own choice (the state-parallel or the binned check)
+PLAN_VARIANTS = (-1, 0, 1, 2, 3, 4)
 # (collision check, point slices, trajectory warps): check 1 = per-step bins
 # (slices unused), 0 = brute force over cell-sorted point tiles
 BATCH_CANDIDATES = tuple([(1, 4, w) for w in (4, 8)] + [(0, s, w) for s in (2, 4, 8) for w in (4, 8)])
@@ -69,7 +72,7 @@ def tune_plan_step(planner, state, goal, obs, N, T, seed, reps=3, path=None):
         ts = []
         for r in range(reps + 1):
             planner.plan(state, goal, obs, N, T, seed, r)
-            ts.append(npp.npp_last_timing(planner.h)["collide"])
+            ts.append(npp.npp_last_timing(planner.h)["total"])
         times[v] = float(np.median(ts[1:]))
     best = min(times, key=times.get)
     npp.npp_set_option(planner.h, "collide_variant", best)
