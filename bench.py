@@ -889,7 +889,7 @@ def run_batch(args):
                 "kernel_ms_per_step": trj_ms,
                 "other": {"batch_binned_kernel (widths 16/32)": {
                     "ms_per_step": col_ms,
-                    "note": "binned: checks only the points of the cells a state's disk overlaps"},
+                    "note": "binned: checks only the points of the cells the box around a state's vehicle overlaps"},
                     "obstacle_and_bin_streams": {
                         "bytes_per_step": bin_bytes,
                         "achieved_gbs_lower_bound": bin_bytes / (trj_ms / 1e3) / 1e9,

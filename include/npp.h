@@ -405,7 +405,7 @@ typedef struct {
 typedef struct npp_batch npp_batch;
 
 /* Validate the S scene descriptors, order the work, allocate the batch's
- * workspaces (24 bytes per sample-step plus the points) and upload the scene
+ * workspaces (16 bytes per sample-step plus the points and grids) and upload the scene
  * table (synchronous).  The batch uses h's constants and keeps a pointer to h. */
 npp_status npp_batch_create(npp_handle* h, const npp_scene* scenes, int32_t S, npp_batch** out);
 
@@ -424,7 +424,7 @@ npp_status npp_plan_batch(npp_batch* B, const float* obs_dev, const npp_batch_ou
 
 /* Launch shapes of the batch (no result changes): "collide" = collision
  * check: 1 (default) per-scene, per-step spatial bins (one warp per sample,
- * the points of the cells its rectangle's disk overlaps), 0 brute force over
+ * the points of the cells that the box around its rectangle overlaps), 0 brute force over
  * the scene's points, sorted by cell so that tiles out of reach of an
  * item's live samples are skipped; "slices" = warps that share one 8-sample
  * brute-force item, each on an interleaved share of the point tiles (2, 4 or
@@ -477,10 +477,13 @@ npp_status npp_plan_step_noalloc(const npp_config* cfg, const npp_state* state,
  * 3 / 4 items of 8 samples checked by 4 / 2 warps each taking a slice of the
  * points, 5 per-step spatial binning: the points extrapolated to each step
  * are counting-sorted into a uniform grid around the vehicle and each state
- * is tested only against the cells its bounding disk overlaps (the same
- * per-point test, so the same flags as checking every point); -1 (default)
- * takes 5 from 128 points and below that 2 for N >= 6144 or at most 64
- * points, else 3.
+ * is tested only against the cells that the box around the turned vehicle
+ * overlaps (the same per-point test, so the same flags as checking every
+ * point), one warp per sample, or from 1024 samples (up to 8702 points, one
+ * launch, the rectangle) a step's samples together on its grid in shared
+ * memory; -1 (default) takes one lane per state against every point below 160
+ * points (128 at width 64, 257 for at most 1024 samples at the smaller
+ * widths), else 5.
  * "fuse" -1 (default), 0 or 1: with the binned check (5) and no per-sample
  * records requested, 1 runs the check inside the trajectory kernel: each
  * warp rolls its samples through a window of steps, checks the window's
@@ -488,7 +491,7 @@ npp_status npp_plan_step_noalloc(const npp_config* cfg, const npp_state* state,
  * within one window of its first collision, storing states and controls up
  * to that window (every row the winner's outputs need).  Same results;
  * -1 takes it at width 64 (measured on GB300 at N = 65536, T = 100,
- * M = 8192: 2.72 ms per plan step against 3.83 in two kernels), 0 never.
+ * M = 8192: 1.98 ms per plan step against 2.73 in two kernels), 0 never.
  * "chunks" 0..8: with the binned check (5) and no per-sample records
  * requested (sample_traj and sample_ctrl NULL, and the closed loop), roll
  * the horizon out in that many chunks of steps, each followed by the check
@@ -515,8 +518,12 @@ npp_status npp_set_option(npp_handle* h, const char* name, int32_t value);
  * epilogue: [2] is 0); with the fused binned check, [0] is the grid build
  * and [1] the fused trajectory-and-check kernel; with the step chunks
  * ("chunks"), [0] and [1] are the sums over the chunks' trajectory and check
- * launches.  Disabled by default; enabling it adds four event records per
- * call (and two per chunk). */
+ * launches.  npp_plan_batch runs its widths side by side; with timing on they
+ * follow one another on the caller's stream, so that [0] (grids, trajectories
+ * and the checks inside them) and [1] (the other checks) are stages of their
+ * own; [3] then times that schedule, not the untimed call's.
+ * Disabled by default; enabling it adds four event records per call (and two
+ * per chunk). */
 npp_status npp_set_timing(npp_handle* h, int32_t enable);
 npp_status npp_last_timing(npp_handle* h, float* stage_ms, int32_t n);
 

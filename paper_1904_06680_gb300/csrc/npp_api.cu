@@ -209,11 +209,11 @@ static cudaError_t launch_fused(const npp_handle* h, const RolloutArgs& a, cudaS
 // Step chunks of a binned plan step: 1 (one trajectory launch and one check)
 // when the caller wants every sample's records or chooses so, else the
 // handle's setting or the automatic choice, at most one per step.  Each
-// chunk regenerates its samples' parameters (measured on GB300 at N = 65536,
-// T = 100, width 64: 0.59 ms per full generation, 0.12 ms of launch and tail
-// per chunk, 0.027 ms per step of all samples), so two chunks pay at width
-// 64 (3.83 -> 3.31 ms per plan step; 3, 4, 6 chunks: 3.50, 3.87, 4.69 ms)
-// and none at width 32 and T = 40 (0.258 ms in one launch, 0.293 in two).
+// chunk regenerates its samples' parameters, so chunks pay at width 64 over
+// long horizons only (GB300, us per plan step in 1, 2, 3, 4, 6 chunks:
+// N = 65536, T = 100 2733, 2509, 2531, 2857, 3275; N = 16384, T = 40 391 and
+// 505 in 2), where the windowed check is faster still: the automatic 2 is
+// for callers that turn it off.
 static int chunk_count(const npp_handle* h, const RolloutArgs& a, bool no_records)
 {
     if (!no_records || h->chunks == 1 || a.T < 2) return 1;
@@ -301,9 +301,11 @@ npp_status run_rollout(npp_handle* h, RolloutArgs& a, cudaStream_t s, bool no_re
     // few -> one lane per state against all of them (states_auto); at
     // width 64 the binned check runs window by window inside the
     // trajectory kernel unless the caller wants every sample's records
-    // (measured at N = 65536, T = 100, M = 8192: 2.72 ms per plan step
-    // against 3.83 in two kernels and 3.31 in two step chunks; at width 32,
-    // T = 40 the two kernels stay faster, 0.258 against 0.311 ms)
+    // (us per plan step, windowed / two kernels: N = 65536, T = 100, M = 8192
+    // 1984 / 2733, 2509 in two step chunks; the course's N = 16384, T = 40,
+    // M = 2000 380 / 391, N = 3000 113 / 101).  At the smaller widths the two
+    // kernels are faster: the course at width 32 219 / 142, with 40000 samples
+    // 455 / 298, T = 100 747 / 573; at width 16 182 / 84
     const int v = h->collide_variant >= 0 ? h->collide_variant
                 : (states_auto(a.M, a.N, h->cfg.width) ? COLLIDE_STATES : COLLIDE_BINNED);
     if (v == COLLIDE_BINNED) {

@@ -167,8 +167,8 @@ __device__ __forceinline__ float sfu_rsqrt(float x)
 // (reciprocal root), the product with it, and one correction by the exact
 // fma residual (Markstein, "Computation of elementary functions on the IBM
 // RISC System/6000 processor", IBM J. Res. Dev. 34, 1990).  The arguments
-// are the 2^23 values of u, for every one of which the results equal the
-// IEEE quotient and root (tests/test_gpu_sampler.py covers almost all of them).
+// are the 2^23 values of u; tests/test_gpu_sampler.py compares the results with
+// the IEEE quotient and root on 98 % of them.
 // Integer-to-float conversions are exact bit constructions (1.m minus a
 // constant) except the exponent's.
 //
@@ -344,7 +344,8 @@ __device__ __forceinline__ float4 sample_quad_mixed_tail(const SamplerKey& key, 
 // ------------------------------------------------------------------ spatial bins
 // Per-step grids of the binned collision check: for step h, cell_start[h]
 // [BIN_DIM^2 + 1 entries, stride BIN_CS_STRIDE] indexes the points of
-// step h sorted by cell, pts + h M.  A query disk of radius `reach` around a
+// step h sorted by cell, pts + h M (for the check with a step's grid in shared
+// memory, 16-bit entries in the same place).  A query box within `reach` of a
 // state spans at most five cells per axis.
 constexpr int BIN_DIM = 128;
 constexpr int BIN_NCELL = BIN_DIM * BIN_DIM;
@@ -633,7 +634,7 @@ int collide_resident_blocks_per_sm(int M, int variant);
 int collide_max_points(int smem_limit);
 // collisions through per-step spatial binning of the points (any M): builds
 // the grids in `workspace` (binned_workspace_bytes) and checks every sample
-// against the points of the cells its bounding disk overlaps
+// against the points of the cells that the box around it overlaps
 size_t binned_workspace_bytes(int max_T, int max_M);
 cudaError_t build_bins(RolloutArgs& a, float half_len, float half_wid, float c_off, void* workspace,
                        cudaStream_t s);          // fills a.bins

@@ -1,28 +1,33 @@
-// npp_rollout.cuh -- the two kernels of one plan step, instantiated per
-// network width by npp_rollout_w{16,32,64}.cu.
+// npp_rollout.cuh -- the kernels of one plan step: trajectories
+// (instantiated per network width by npp_rollout_w{16,32,64}.cu), the checks
+// by brute force (npp_collide.cu) and the parts that all checks share.
 //
 // The rollout of a sample (Sect. II-D "Sixth", Sect. IV) does not depend on
 // its collision checks: a collision only ends the sample (cost +inf).  The
 // step is therefore split into
 //
-//   traj_kernel    -- per sample: features (Eq. eq_def_stph), MLP
-//                     a = X(s, theta) (Eq. eq_def_at), rate-limited controls,
-//                     Euler step of the kinematic bicycle on the old state,
-//                     for h = 0..T; writes the states [T+1][N], the applied
-//                     controls [T][N] and the cost the sample has if it is
-//                     collision-free.  A group of G lanes of one warp holds
-//                     one sample's network in registers (each lane W/G hidden
-//                     units: its rows of W1, W2 and columns of W3), generated
-//                     straight from Philox and never stored.
-//   collide_kernel -- per block of SB samples: the M obstacle points staged in
-//                     shared memory in the EV-aligned frame at t, then for
-//                     h = 0..T the still-live samples are checked against the
-//                     points extrapolated at constant velocity (Sect. II-D
-//                     items (i)-(iv)) with the polytope inequalities of Eq.
-//                     eq_Apsietc_collAvoidIneqs; a sample leaves the live list
-//                     at its first collision.  Finally the (class, cost,
-//                     index) keys are reduced and folded into the global
-//                     minimum with one 64-bit atomicMin per block.
+//   trajectories -- per sample: features (Eq. eq_def_stph), MLP
+//                   a = X(s, theta) (Eq. eq_def_at), rate-limited controls,
+//                   Euler step of the kinematic bicycle on the old state,
+//                   for h = 0..T; writes the states [T+1][N], the applied
+//                   controls [T][N] and the cost the sample has if it is
+//                   collision-free.  A group of G lanes of one warp holds
+//                   one sample's network (each lane W/G hidden units: its rows
+//                   of W1, W2 and columns of W3), generated straight from
+//                   Philox and never stored: layer 2 in tensor memory, the
+//                   rest in registers (traj_tmem_kernel), or all of it in
+//                   registers and shared memory (traj_kernel).
+//   check        -- states h = 0..T against the M obstacle points
+//                   extrapolated at constant velocity (Sect. II-D items
+//                   (i)-(iv)) with the polytope inequalities of Eq.
+//                   eq_Apsietc_collAvoidIneqs, every point (collide_*_kernel
+//                   here and in npp_collide.cu) or those of the cells near a
+//                   state (npp_binned.cu); a sample ends at its first
+//                   collision, and the (class, cost, index) keys are folded
+//                   into the global minimum by 64-bit atomicMin.
+//
+// or done in turns, a window of steps and a window's check, by one kernel
+// (fused_tmem_kernel, fused_kernel).
 #pragma once
 
 #include <cfloat>

@@ -31,8 +31,8 @@ cudaError_t launch_traj_w32(const RolloutArgs& a, cudaStream_t s, int variant)
 // arguments after the trajectory kernel's: window of states, candidates
 // loaded ahead per lane).  Not the library's choice at this width: on the
 // course (N = 16384, T = 40, M = 2000) the default shape, 5 of 8 W2 quads in
-// shared memory and windows of 8, took 0.311 ms per plan step against 0.258
-// in two kernels (1: 0.348, 3: 0.330).
+// shared memory and windows of 8, takes 219 us per plan step against 142 in
+// two kernels (1 to 4: 262, 234, 258, 242).
 cudaError_t launch_fused_w32(const RolloutArgs& a, cudaStream_t s, int variant)
 {
     if (uses_variants(a.c)) return launch_fused<32, 16, 4, 5, true, 5, 8, 4>(a, s);
