@@ -302,27 +302,35 @@ __global__ void __launch_bounds__(GRID_THREADS, 2) collide_grid_kernel(const Rol
 // boxes overlap.  The check itself cannot count: which states of a collided
 // sample it still meets depends on the order in which the steps' blocks run.
 // Timed plan steps only, after the last event.
+// (One pair of global atomics a block: one a warp took 30 us on the course.)
 constexpr int COUNT_THREADS = 256;
+constexpr int COUNT_SAMPLES = 4 * COUNT_THREADS;
 __global__ void __launch_bounds__(COUNT_THREADS) count_grid_kernel(const RolloutArgs a)
 {
-    const int n = blockIdx.x * COUNT_THREADS + threadIdx.x, h = blockIdx.y;
+    __shared__ unsigned sum[2];
+    const int h = blockIdx.y, n0 = blockIdx.x * COUNT_SAMPLES, n1 = min(a.N, n0 + COUNT_SAMPLES);
     const BinView& g = a.bins;
+    const unsigned short* cs = reinterpret_cast<const unsigned short*>(g.cell_start + (size_t)h * BIN_CS_STRIDE);
+    if (threadIdx.x < 2) sum[threadIdx.x] = 0u;
+    __syncthreads();
     unsigned tests = 0, states = 0;
-    if (n < a.N && h <= a.first[n]) {
-        const unsigned short* cs = reinterpret_cast<const unsigned short*>(g.cell_start + (size_t)h * BIN_CS_STRIDE);
+    for (int n = n0 + threadIdx.x; n < n1; n += COUNT_THREADS) {
+        if (h > a.first[n]) continue;
         const float4 z = a.traj[(size_t)h * a.N + n];
         float sp, cp;
         sincos_r(z.z, sp, cp);
         const QueryCells q = query_cells(g, query_box(g, z.x, z.y, sp, cp));
         for (int iy = q.iy0; iy <= q.iy1; ++iy) tests += cs[iy * BIN_DIM + q.ix1 + 1] - cs[iy * BIN_DIM + q.ix0];
-        states = 1;
+        ++states;
     }
     tests = __reduce_add_sync(FULL, tests);
     states = __reduce_add_sync(FULL, states);
-    if ((threadIdx.x & 31) == 0 && states) {
-        atomicAdd(a.counts, (unsigned long long)tests);
-        atomicAdd(a.counts + 1, (unsigned long long)states);
+    if ((threadIdx.x & 31) == 0) {
+        atomicAdd(&sum[0], tests);
+        atomicAdd(&sum[1], states);
     }
+    __syncthreads();
+    if (threadIdx.x < 2 && sum[1]) atomicAdd(a.counts + threadIdx.x, (unsigned long long)sum[threadIdx.x]);
 }
 
 }  // namespace
@@ -390,7 +398,7 @@ cudaError_t launch_collide_grid(const RolloutArgs& a, cudaStream_t s)
 
 cudaError_t launch_count_grid(const RolloutArgs& a, cudaStream_t s)
 {
-    count_grid_kernel<<<dim3((a.N + COUNT_THREADS - 1) / COUNT_THREADS, a.T + 1), COUNT_THREADS, 0, s>>>(a);
+    count_grid_kernel<<<dim3((a.N + COUNT_SAMPLES - 1) / COUNT_SAMPLES, a.T + 1), COUNT_THREADS, 0, s>>>(a);
     return cudaGetLastError();
 }
 
