@@ -469,8 +469,10 @@ struct TmemNet {
 
     // the first 16 columns, read while layer 1 runs.  The read is the whole
     // warp's, and single lanes have just stored records: hence the __syncwarp
-    // (0 to 0.7 % of a plan step; with the stores moved ahead of one of the
-    // step's own instead, registers spill: up to 6 %)
+    // (most plan steps take as long as without it, width 16 in 20-warp blocks
+    // 1 % longer, with features in the body frame 2 %; the stores moved ahead
+    // of one of the step's own cost registers, up to 6 %, and predicated in PTX
+    // up to 4 %)
     struct Ahead { Tmem16 w; };
     __device__ __forceinline__ Ahead fetch_ahead() const {
         Ahead f;
